@@ -481,6 +481,20 @@ namespace {
 // Enqueues the W^2 reduction (Eq. (3)) and the copy of its sums into the
 // handle's pinned staging area.
 int enqueue_w2(oct_sim *s) {
+    if (s->L <= static_cast<int64_t>(oct::kW2SmallL)) {
+        // two launches that write the staging area themselves
+        oct::W2Job j{};
+        j.lat = s->lat;
+        j.L = j.nrows = j.plane_rows = static_cast<uint32_t>(s->L);
+        j.res = static_cast<oct::W2Result *>(s->h_small);
+        j.cnt = s->d_net;
+        j.cnt_n = j.cnt_off = oct::kNetSlots;
+        j.cnt_out = reinterpret_cast<long long *>(static_cast<char *>(s->h_small) + 128);
+        OCT_CUDA(oct::launch_w2_small_one(j, s->d_rows, s->stream));
+        s->w2_pending = true;
+        s->w2_t = s->t;
+        return OCT_OK;
+    }
     OCT_CUDA(oct::launch_net_sum(s->d_net, s->d_net + oct::kNetSlots, s->d_net + 2 * oct::kNetSlots,
                                  s->d_net_sum, s->stream));
     OCT_CUDA(oct::launch_w2(s->lat, static_cast<uint32_t>(s->L), s->d_rows, s->d_w2, s->stream));

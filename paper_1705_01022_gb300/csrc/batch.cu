@@ -22,6 +22,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/oct.h"
@@ -179,14 +180,17 @@ struct WorkBuf {
     cudaEvent_t copied = nullptr;  // recorded after that copy
 };
 
-// An asynchronous W^2 measurement: the exact sums, the replica's counters and
-// its time, copied to pinned host memory behind an event.
+// A W^2 measurement: the exact sums, the replica's counters and its time,
+// written to pinned host memory by the reduction itself.
 struct MeasureRecord {
     W2Result res;
-    unsigned long long cnt[2];
+    long long cnt[2];
     uint32_t t;
     uint32_t pad[3];
 };
+// Rows reduced by one launch of a measurement of all replicas (32 MiB of row
+// records); larger batches take several launches.
+constexpr uint64_t kMeasureRows = uint64_t{1} << 20;
 constexpr int kMeasureRing = 1024;
 constexpr int kMarkRing = 64;
 constexpr int kGraphMcs = 4;  // MCS in the batch's longer captured graph
@@ -223,8 +227,16 @@ struct oct_batch {
     uint32_t *d_queue = nullptr;  // 4 * kBranches counters: (device step, branch)
     oct::W2RowSums *d_rows = nullptr;
     int64_t rows_cap = 0;
-    oct::W2Result *d_w2 = nullptr;
     void *h_small = nullptr;
+    // measurement of all replicas: job list (device, and its pinned staging),
+    // records by slot, and the launches' ranges; rebuilt after a membership change
+    bool jobs_dirty = true;
+    oct::W2Job *d_jobs = nullptr;
+    oct::W2Job *h_jobs = nullptr;
+    oct::MeasureRecord *h_all = nullptr;
+    size_t all_cap = 0;
+    std::vector<std::pair<uint32_t, uint32_t>> job_ranges;  // (first job, warp tasks) of each launch
+    uint32_t n_jobs = 0;
     // two-time autocorrelations: per slot, the lattice at its waiting time
     std::vector<uint32_t *> snap;
     std::vector<int64_t> snap_t;
@@ -241,8 +253,7 @@ struct oct_batch {
     cudaStream_t side[kBranches] = {};
     cudaEvent_t fork_ev = nullptr;
     cudaEvent_t join_ev[kBranches] = {};
-    // asynchronous measurements: a ring of records (device and pinned host)
-    oct::MeasureRecord *d_req = nullptr;
+    // asynchronous measurements: a ring of pinned records
     oct::MeasureRecord *h_req = nullptr;
     std::vector<cudaEvent_t> req_ev;
     std::vector<int64_t> req_L;
@@ -289,7 +300,9 @@ void batch_free(oct_batch *b) {
         if (w.host) cudaFreeHost(w.host);
         if (w.copied) cudaEventDestroy(w.copied);
     }
-    cudaFree(b->d_req);
+    cudaFree(b->d_jobs);
+    if (b->h_jobs) cudaFreeHost(b->h_jobs);
+    if (b->h_all) cudaFreeHost(b->h_all);
     if (b->h_req) cudaFreeHost(b->h_req);
     for (cudaEvent_t e : b->req_ev)
         if (e) cudaEventDestroy(e);  // ring events are created on first use
@@ -302,7 +315,6 @@ void batch_free(oct_batch *b) {
     }
     if (b->fork_ev) cudaEventDestroy(b->fork_ev);
     cudaFree(b->d_rows);
-    cudaFree(b->d_w2);
     if (b->h_small) cudaFreeHost(b->h_small);
     for (cudaEvent_t e : b->ev)
         if (e) cudaEventDestroy(e);
@@ -392,6 +404,7 @@ cudaError_t grow_slots(oct_batch *b, size_t need) {
     b->counters = c;
     b->capacity = n;
     b->dirty = true;
+    b->jobs_dirty = true;
     return cudaSuccess;
 }
 
@@ -655,38 +668,8 @@ int add_replica(oct_batch *b, const oct_replica *in, int64_t *slot_out) {
     BATCH_CUDA(cudaMemsetAsync(b->d_t + slot, 0, sizeof(uint32_t), b->stream));
     BATCH_CUDA(cudaMemsetAsync(b->counters + 2 * slot, 0, 2 * sizeof(unsigned long long), b->stream));
     b->dirty = true;
+    b->jobs_dirty = true;
     if (slot_out) *slot_out = slot;
-    return OCT_OK;
-}
-
-int measure_slot(oct_batch *b, int64_t slot, oct_w2 *out) {
-    const int64_t L = b->reps[slot].L;
-    if (L > b->rows_cap) {
-        cudaFree(b->d_rows);
-        b->d_rows = nullptr;
-        b->rows_cap = 0;
-        BATCH_CUDA(cudaMalloc(&b->d_rows, sizeof(oct::W2RowSums) * L));
-        b->rows_cap = L;
-    }
-    auto *res = static_cast<oct::W2Result *>(b->h_small);
-    auto *cnt = reinterpret_cast<unsigned long long *>(static_cast<char *>(b->h_small) + 64);
-    auto *tt = reinterpret_cast<uint32_t *>(static_cast<char *>(b->h_small) + 96);
-    BATCH_CUDA(oct::launch_w2(b->lat[slot], static_cast<uint32_t>(L), b->d_rows, b->d_w2, b->stream));
-    BATCH_CUDA(cudaMemcpyAsync(res, b->d_w2, sizeof(oct::W2Result), cudaMemcpyDeviceToHost, b->stream));
-    BATCH_CUDA(cudaMemcpyAsync(cnt, b->counters + 2 * slot, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, b->stream));
-    BATCH_CUDA(cudaMemcpyAsync(tt, b->d_t + slot, sizeof(uint32_t), cudaMemcpyDeviceToHost, b->stream));
-    BATCH_CUDA(cudaStreamSynchronize(b->stream));
-    const __int128 N = static_cast<__int128>(L) * L;
-    const __int128 S2 = static_cast<__int128>((static_cast<unsigned __int128>(res->s2_hi) << 64) | res->s2_lo);
-    const __int128 num = N * S2 - static_cast<__int128>(res->s1) * res->s1;
-    out->t = static_cast<int64_t>(*tt);
-    out->n_sites = static_cast<int64_t>(N);
-    out->s1 = res->s1;
-    out->s2_lo = res->s2_lo;
-    out->s2_hi = res->s2_hi;
-    out->net_flips = static_cast<int64_t>(cnt[0]);
-    out->hmax = res->hmax;
-    out->w2 = static_cast<double>(num) / (static_cast<double>(N) * static_cast<double>(N));
     return OCT_OK;
 }
 
@@ -705,6 +688,88 @@ void record_to_w2(const oct::MeasureRecord &r, int64_t L, oct_w2 *out) {
     out->w2 = static_cast<double>(num) / (static_cast<double>(N) * static_cast<double>(N));
 }
 
+// The reduction of the replica in one slot into the pinned record m.
+oct::W2Job replica_job(const oct_batch *b, int64_t slot, oct::MeasureRecord *m) {
+    oct::W2Job j{};
+    j.lat = b->lat[slot];
+    j.L = j.nrows = j.plane_rows = static_cast<uint32_t>(b->reps[slot].L);
+    j.res = &m->res;
+    j.cnt = b->counters + 2 * slot;
+    j.cnt_n = 1;
+    j.cnt_off = 1;
+    j.cnt_out = m->cnt;
+    j.t = b->d_t + slot;
+    j.t_out = &m->t;
+    return j;
+}
+
+// Row records for `rows` rows; stream-ordered: an earlier measurement may
+// still use the old ones.
+int ensure_rows(oct_batch *b, int64_t rows) {
+    if (rows <= b->rows_cap) return OCT_OK;
+    if (b->d_rows) BATCH_CUDA(cudaFreeAsync(b->d_rows, b->stream));
+    b->d_rows = nullptr;
+    b->rows_cap = 0;
+    BATCH_CUDA(cudaMallocAsync(reinterpret_cast<void **>(&b->d_rows), sizeof(oct::W2RowSums) * rows, b->stream));
+    b->rows_cap = rows;
+    return OCT_OK;
+}
+
+int measure_slot(oct_batch *b, int64_t slot, oct_w2 *out) {
+    int rc = ensure_rows(b, b->reps[slot].L);
+    if (rc) return rc;
+    auto *m = static_cast<oct::MeasureRecord *>(b->h_small);
+    BATCH_CUDA(oct::launch_w2_small_one(replica_job(b, slot, m), b->d_rows, b->stream));
+    BATCH_CUDA(cudaStreamSynchronize(b->stream));
+    record_to_w2(*m, b->reps[slot].L, out);
+    return OCT_OK;
+}
+
+// The job list of all replicas, in launches of at most kMeasureRows rows.
+// Called with no measurement of all replicas in flight (each one waits for
+// its records), so the staging memory is free.
+int build_jobs(oct_batch *b) {
+    const size_t n = b->reps.size();
+    if (n > b->all_cap) {
+        const size_t cap = std::max<size_t>(b->capacity, n);
+        cudaFree(b->d_jobs);
+        if (b->h_jobs) cudaFreeHost(b->h_jobs);
+        if (b->h_all) cudaFreeHost(b->h_all);
+        b->d_jobs = nullptr;
+        b->h_jobs = nullptr;
+        b->h_all = nullptr;
+        b->all_cap = 0;
+        BATCH_CUDA(cudaMalloc(&b->d_jobs, sizeof(oct::W2Job) * cap));
+        BATCH_CUDA(cudaMallocHost(&b->h_jobs, sizeof(oct::W2Job) * cap));
+        BATCH_CUDA(cudaMallocHost(&b->h_all, sizeof(oct::MeasureRecord) * cap));
+        b->all_cap = cap;
+    }
+    b->job_ranges.clear();
+    uint32_t nj = 0;
+    int64_t most = 0;
+    size_t slot = 0;
+    while (slot < n) {
+        const uint32_t first = nj;
+        uint64_t rows = 0;
+        for (; slot < n; ++slot) {
+            if (!b->used[slot]) continue;
+            if (nj > first && rows + b->reps[slot].L > oct::kMeasureRows) break;
+            rows += b->reps[slot].L;
+            b->h_jobs[nj++] = replica_job(b, static_cast<int64_t>(slot), b->h_all + slot);
+        }
+        if (nj == first) break;
+        b->job_ranges.emplace_back(first, oct::w2_small_split(b->h_jobs + first, nj - first));
+        most = std::max<int64_t>(most, static_cast<int64_t>(rows));
+    }
+    b->n_jobs = nj;
+    if (nj)
+        BATCH_CUDA(cudaMemcpyAsync(b->d_jobs, b->h_jobs, sizeof(oct::W2Job) * nj, cudaMemcpyHostToDevice, b->stream));
+    int rc = ensure_rows(b, most);
+    if (rc) return rc;
+    b->jobs_dirty = false;
+    return OCT_OK;
+}
+
 int ticket_index(oct_batch *b, int64_t ticket, int *idx) {
     if (ticket < 0 || ticket >= b->req_next || ticket < b->req_next - oct::kMeasureRing)
         return bfail(OCT_EINVAL, "unknown or expired measurement ticket");
@@ -720,8 +785,7 @@ int oct_batch_measure_async(oct_batch *b, int64_t slot, int64_t *ticket) {
     if (!b || !ticket || !valid_slot(b, slot)) return bfail(OCT_EINVAL, "no replica in that slot");
     BATCH_CUDA(cudaSetDevice(b->device));
     const int64_t L = b->reps[slot].L;
-    if (!b->d_req) {
-        BATCH_CUDA(cudaMalloc(&b->d_req, sizeof(oct::MeasureRecord) * oct::kMeasureRing));
+    if (!b->h_req) {
         BATCH_CUDA(cudaMallocHost(&b->h_req, sizeof(oct::MeasureRecord) * oct::kMeasureRing));
         b->req_ev.assign(oct::kMeasureRing, nullptr);
         b->req_L.assign(oct::kMeasureRing, 0);
@@ -732,19 +796,9 @@ int oct_batch_measure_async(oct_batch *b, int64_t slot, int64_t *ticket) {
     } else {
         BATCH_CUDA(cudaEventCreateWithFlags(&b->req_ev[i], cudaEventDisableTiming));
     }
-    if (L > b->rows_cap) {  // stream-ordered: an earlier measurement may still use the old rows
-        if (b->d_rows) BATCH_CUDA(cudaFreeAsync(b->d_rows, b->stream));
-        b->d_rows = nullptr;
-        b->rows_cap = 0;
-        BATCH_CUDA(cudaMallocAsync(reinterpret_cast<void **>(&b->d_rows), sizeof(oct::W2RowSums) * L, b->stream));
-        b->rows_cap = L;
-    }
-    oct::MeasureRecord *d = b->d_req + i;
-    BATCH_CUDA(oct::launch_w2(b->lat[slot], static_cast<uint32_t>(L), b->d_rows, &d->res, b->stream));
-    BATCH_CUDA(cudaMemcpyAsync(d->cnt, b->counters + 2 * slot, 2 * sizeof(unsigned long long),
-                               cudaMemcpyDeviceToDevice, b->stream));
-    BATCH_CUDA(cudaMemcpyAsync(&d->t, b->d_t + slot, sizeof(uint32_t), cudaMemcpyDeviceToDevice, b->stream));
-    BATCH_CUDA(cudaMemcpyAsync(b->h_req + i, d, sizeof(oct::MeasureRecord), cudaMemcpyDeviceToHost, b->stream));
+    int rc = ensure_rows(b, L);
+    if (rc) return rc;
+    BATCH_CUDA(oct::launch_w2_small_one(replica_job(b, slot, b->h_req + i), b->d_rows, b->stream));
     BATCH_CUDA(cudaEventRecord(b->req_ev[i], b->stream));
     b->req_L[i] = L;
     *ticket = b->req_next++;
@@ -821,7 +875,6 @@ int oct_batch_create(int64_t n, const oct_replica *reps, void *stream, oct_batch
         }
     }
     if (e == cudaSuccess) e = cudaMalloc(&b->d_queue, sizeof(uint32_t) * 4 * kBranches);
-    if (e == cudaSuccess) e = cudaMalloc(&b->d_w2, sizeof(oct::W2Result));
     if (e == cudaSuccess) e = cudaMallocHost(&b->h_small, 256);
     if (e == cudaSuccess) {
         int sms = 0;
@@ -872,6 +925,7 @@ int oct_batch_remove(oct_batch *b, int64_t slot) {
     b->used[slot] = 0;
     b->free_slots.push_back(slot);
     b->dirty = true;
+    b->jobs_dirty = true;
     return OCT_OK;
 }
 
@@ -928,13 +982,21 @@ int oct_batch_measure_w2(oct_batch *b, oct_w2 *out, int64_t n) {
     if (!b || !out || n != static_cast<int64_t>(b->reps.size()))
         return bfail(OCT_EINVAL, "out must hold one entry per slot");
     BATCH_CUDA(cudaSetDevice(b->device));
-    for (int64_t slot = 0; slot < n; ++slot) {
-        if (!b->used[slot]) {
-            std::memset(&out[slot], 0, sizeof(oct_w2));
-            continue;
-        }
-        int rc = measure_slot(b, slot, &out[slot]);
+    if (b->jobs_dirty) {
+        int rc = build_jobs(b);
         if (rc) return rc;
+    }
+    for (size_t i = 0; i < b->job_ranges.size(); ++i) {
+        const uint32_t first = b->job_ranges[i].first;
+        const uint32_t end = i + 1 < b->job_ranges.size() ? b->job_ranges[i + 1].first : b->n_jobs;
+        BATCH_CUDA(oct::launch_w2_small(b->d_jobs + first, end - first, b->job_ranges[i].second, b->d_rows, b->stream));
+    }
+    BATCH_CUDA(cudaStreamSynchronize(b->stream));
+    for (int64_t slot = 0; slot < n; ++slot) {
+        if (b->used[slot])
+            record_to_w2(b->h_all[slot], b->reps[slot].L, &out[slot]);
+        else
+            std::memset(&out[slot], 0, sizeof(oct_w2));
     }
     return OCT_OK;
 }

@@ -14,6 +14,8 @@
 // 2 h0 R1 + R2) accumulate in 128-bit integers, per block of rows and then
 // over the blocks.  Per-row terms are bounded by
 // 4 L^3 < 2^63 for L <= 2^20, so only the cross-row sums need 128 bits.
+#include <algorithm>
+
 #include "oct_internal.h"
 
 namespace oct {
@@ -445,6 +447,190 @@ __global__ void __launch_bounds__(kW2CombineThreads)
     }
 }
 
+// Lattices of up to kW2SmallL sites a side: one or many of them in two
+// launches.  A row of 16384 sites is 512 words, one warp's chunk, so a row is
+// one step: 2^sl_log lanes take it, 2^lw_log words each, and a warp takes
+// 32 / 2^sl_log rows at once (w2_rows_kernel gives a row to a warp at 16 words
+// per lane: at L = 2048 four of its lanes have work).  Pass 2 is one block per
+// lattice and writes the result, the counters and the time to where the job
+// points (page-locked host memory: no copies).  Every sum of a lattice this
+// small fits 64 bits: S2 <= 2^28 sites x (2^14)^2 = 2^56.
+// Bound by launches and latency, not by work: one W^2 of L=256 went from four
+// kernels and two copies (33 us with the wait) to two kernels (17 us), and the
+// W^2 of 256 replicas (L = 64..2048, 375 M sites) from 256 such calls (8.3 ms)
+// to 0.5 ms.
+constexpr int kW2SmallThreads = 512;  // of the second launch
+
+// Words j .. j+3 of the lane's nw, as one 16-byte load where allowed.
+__device__ __forceinline__ void load_quad(const uint32_t *row, uint32_t j, uint32_t nw, bool vec_ok,
+                                          uint32_t (&v)[4]) {
+    if (vec_ok && j + 4u <= nw) {
+        const uint4 q = *reinterpret_cast<const uint4 *>(row + j);
+        v[0] = q.x;
+        v[1] = q.y;
+        v[2] = q.z;
+        v[3] = q.w;
+    } else {
+#pragma unroll
+        for (uint32_t i = 0; i < 4u; ++i) v[i] = (j + i < nw) ? row[j + i] : 0u;
+    }
+}
+
+__global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
+    w2_small_rows_kernel(const __grid_constant__ W2Job one, const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows) {
+    extern __shared__ __align__(16) unsigned char w2_table[];
+    for (int i = threadIdx.x; i < 256; i += blockDim.x) {
+        const uint2 e = byte_entry(static_cast<uint32_t>(i));
+#pragma unroll
+        for (int c = 0; c < 16; ++c) *reinterpret_cast<uint2 *>(w2_table + 256 * i + 8 * c) = e;
+    }
+    __syncthreads();
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t slot = 8u * (lane & 15u);
+    for (uint32_t task = blockIdx.x * kW2Warps + (threadIdx.x >> 5); task < n_tasks; task += gridDim.x * kW2Warps) {
+        const W2Job *J = &one;
+        if (jobs) {  // the last job whose first task is not past this one
+            uint32_t a = 0, b = n;
+            while (b - a > 1u) {
+                const uint32_t m = (a + b) >> 1;
+                if (jobs[m].task_first <= task) a = m; else b = m;
+            }
+            J = jobs + a;
+        }
+        const uint32_t wpr = J->L >> 5, nrows = J->nrows, lw = 1u << J->lw_log, sl = 1u << J->sl_log;
+        const uint32_t y = ((task - J->task_first) << (5u - J->sl_log)) + (lane >> J->sl_log);
+        const uint32_t li = lane & (sl - 1u), w = li * lw;
+        const uint32_t nw = (y < nrows && w < wpr) ? min(lw, wpr - w) : 0u;
+        const uint32_t *row = J->lat + static_cast<size_t>(min(y, nrows - 1u)) * wpr;
+        const bool vec_ok = lw >= 4u && (wpr & 3u) == 0u && (reinterpret_cast<uintptr_t>(J->lat) & 15u) == 0u;
+        W2Lane a{0, 0u, 0u, 0, 0xFFFFFFFFu};
+        uint32_t v[4], vn[4] = {0u, 0u, 0u, 0u};
+        load_quad(row + w, 0u, nw, vec_ok, v);
+        for (uint32_t j = 0; j < lw; j += 4u) {
+            if (j + 4u < lw) load_quad(row + w, j + 4u, nw, vec_ok, vn);
+#pragma unroll
+            for (uint32_t i = 0; i < 4u; ++i)
+                if (j + i < nw) w2_word(w2_table, slot, v[i], a);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = vn[i];
+        }
+        // as in w2_rows_kernel: the lane's sums, lifted by the steps before it
+        const int M2 = static_cast<int>(a.M2 - 512u * static_cast<uint32_t>(a.SPw) - 65536u * nw);
+        const int M1 = static_cast<int>(a.Mz + 32u * static_cast<uint32_t>(a.SPw) - 512u * nw) / 2;
+        int incl = a.P;
+        for (uint32_t o = 1; o < sl; o <<= 1) {
+            const int x = __shfl_up_sync(kFull, incl, o, sl);
+            if (li >= o) incl += x;
+        }
+        const long long B = incl - a.P, nbits = 32ll * nw;
+        long long q1 = nbits * B + M1, q2 = nbits * B * B + 2 * B * M1 + M2;
+        int qmin = 1 << 30, qmax = -(1 << 30);
+        if (nw > 0) {
+            qmin = static_cast<int>(B) + static_cast<int>(a.ext & 0xFFFFu) - static_cast<int>(kW2Bias);
+            qmax = static_cast<int>(B) + static_cast<int>(kW2Bias) - static_cast<int>(a.ext >> 16);
+        }
+        for (uint32_t o = sl >> 1; o > 0; o >>= 1) {
+            q1 += __shfl_xor_sync(kFull, q1, o);
+            q2 += __shfl_xor_sync(kFull, q2, o);
+            qmin = min(qmin, __shfl_xor_sync(kFull, qmin, o));
+            qmax = max(qmax, __shfl_xor_sync(kFull, qmax, o));
+        }
+        if (li == 0 && y < nrows) {
+            const long long s0 = (row[0] & 1u) ? 1 : -1;
+            const long long Ll = J->L;
+            W2RowSums o;
+            o.r1 = q1 - Ll * s0;
+            o.r2 = q2 - 2 * s0 * q1 + Ll;
+            o.rmin = qmin - static_cast<int>(s0);
+            o.rmax = qmax - static_cast<int>(s0);
+            o.c = static_cast<int>(row[static_cast<size_t>(J->plane_rows) * wpr] & 1u);
+            o.pad = 0;
+            rows[J->row_first + y] = o;
+        }
+    }
+}
+
+// Pass 2: one block per lattice, a run of consecutive rows per thread.
+__global__ void __launch_bounds__(kW2SmallThreads)
+    w2_small_finish_kernel(const __grid_constant__ W2Job one, const W2Job *jobs, const W2RowSums *all_rows) {
+    constexpr int kWarps = kW2SmallThreads / 32;
+    __shared__ int wsum[kWarps];
+    __shared__ long long red[6][kWarps];
+    __shared__ long long last_h;
+    const W2Job &J = jobs ? jobs[blockIdx.x] : one;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t nrows = J.nrows;
+    const W2RowSums *rows = all_rows + J.row_first;
+    const uint32_t per = (nrows + kW2SmallThreads - 1) / kW2SmallThreads;
+    const uint32_t y0 = min(nrows, tid * per), y1 = min(nrows, y0 + per);
+    int rise = 0;  // of the column heights over the thread's rows
+    for (uint32_t y = y0; y < y1; ++y) rise += y == 0 ? 0 : rows[y].c ? 1 : -1;
+    int incl = rise;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int x = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += x;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    long long h = incl - rise;
+    for (int w = 0; w < warp; ++w) h += wsum[w];
+    const long long Ll = J.L;
+    long long v[4] = {0, 0, 0, 0};  // S1, S2, counters
+    long long lo = 1ll << 40, hi = -(1ll << 40);
+    for (uint32_t y = y0; y < y1; ++y) {
+        const W2RowSums r = rows[y];
+        h += y == 0 ? 0 : r.c ? 1 : -1;
+        v[0] += Ll * h + r.r1;
+        v[1] += Ll * h * h + 2 * h * r.r1 + r.r2;
+        lo = min(lo, h + r.rmin);
+        hi = max(hi, h + r.rmax);
+    }
+    if (y0 < y1 && y1 == nrows) last_h = h;
+    if (J.cnt)
+        for (uint32_t i = tid; i < J.cnt_n; i += kW2SmallThreads) {
+            v[2] += static_cast<long long>(J.cnt[i]);
+            v[3] += static_cast<long long>(J.cnt[J.cnt_off + i]);
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] += __shfl_down_sync(kFull, v[i], o);
+        lo = min(lo, __shfl_down_sync(kFull, lo, o));
+        hi = max(hi, __shfl_down_sync(kFull, hi, o));
+    }
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) red[i][warp] = v[i];
+        red[4][warp] = lo;
+        red[5][warp] = hi;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < kWarps; ++w) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] += red[i][w];
+            lo = min(lo, red[4][w]);
+            hi = max(hi, red[5][w]);
+        }
+        W2Result o;
+        o.s1 = v[0];
+        o.s2_lo = static_cast<unsigned long long>(v[1]);
+        o.s2_hi = 0;
+        o.hmax = max(lo < 0 ? -lo : lo, hi < 0 ? -hi : hi);
+        o.lo = lo;
+        o.hi = hi;
+        o.e_last = last_h;
+        o.f0 = rows[0].c ? 1 : -1;
+        *J.res = o;
+        if (J.cnt) {
+            J.cnt_out[0] = v[2];
+            J.cnt_out[1] = v[3];
+        }
+        if (J.t) *J.t_out = *J.t;
+    }
+}
+
 // Interleave two 4-bit values: a0 b0 a1 b1 a2 b2 a3 b3 (LSB first).
 __device__ __forceinline__ uint32_t interleave4(uint32_t a, uint32_t b) {
     uint32_t r = 0;
@@ -523,6 +709,42 @@ __global__ void __launch_bounds__(kNetSlots)
     }
 }
 
+// SMs of the current device, with the shared-memory limit of a table kernel
+// raised once per device.
+cudaError_t table_kernel_setup(const void *kernel, int which, int *sm_count) {
+    constexpr int kMaxDevices = 64;
+    static int sms[kMaxDevices] = {};
+    static bool smem_set[2][kMaxDevices] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    if (sms[dev] <= 0) {
+        e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+    }
+    if (!smem_set[which][dev]) {
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kW2TableBytes);
+        if (e != cudaSuccess) return e;
+        smem_set[which][dev] = true;
+    }
+    *sm_count = sms[dev];
+    return cudaSuccess;
+}
+
+cudaError_t w2_small(const W2Job &one, const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows,
+                     cudaStream_t st) {
+    int sms = 0;
+    cudaError_t e = table_kernel_setup(reinterpret_cast<const void *>(w2_small_rows_kernel), 1, &sms);
+    if (e != cudaSuccess) return e;
+    const uint32_t want = (n_tasks + kW2Warps - 1) / kW2Warps, wave = static_cast<uint32_t>(sms) * kW2BlocksPerSM;
+    w2_small_rows_kernel<<<std::min(want, wave), kW2Warps * 32, kW2TableBytes, st>>>(one, jobs, n, n_tasks, rows);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    w2_small_finish_kernel<<<n, kW2SmallThreads, 0, st>>>(one, jobs, rows);
+    return cudaGetLastError();
+}
+
 int grid_for(uint64_t n, int threads) {
     const uint64_t b = (n + threads - 1) / threads;
     return static_cast<int>(b < 152ull * 32 ? (b ? b : 1) : 152ull * 32);
@@ -548,26 +770,21 @@ cudaError_t launch_w2(const uint32_t *lat, uint32_t L, W2RowSums *rows, W2Result
 
 cudaError_t launch_w2_rows(const uint32_t *lat, uint32_t L, uint32_t nrows, uint32_t plane_rows, W2RowSums *rows,
                            W2Result *out, cudaStream_t st) {
-    // one wave of resident blocks (64 KB of table each), rows taken grid-stride;
-    // the table needs the dynamic shared-memory limit raised once per device
-    constexpr int kMaxDevices = 64;
-    static int sms[kMaxDevices] = {};
-    static bool smem_set[kMaxDevices] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    if (L <= kW2SmallL) {
+        W2Job j{};
+        j.lat = lat;
+        j.L = L;
+        j.nrows = nrows;
+        j.plane_rows = plane_rows;
+        j.res = out;
+        return launch_w2_small_one(j, rows, st);
+    }
+    // one wave of resident blocks (64 KB of table each), rows taken grid-stride
+    int sms = 0;
+    cudaError_t e = table_kernel_setup(reinterpret_cast<const void *>(w2_rows_kernel), 0, &sms);
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (sms[dev] <= 0) {
-        e = cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-    }
-    if (!smem_set[dev]) {
-        e = cudaFuncSetAttribute(w2_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kW2TableBytes);
-        if (e != cudaSuccess) return e;
-        smem_set[dev] = true;
-    }
     const uint64_t want = (static_cast<uint64_t>(nrows) + kW2Warps - 1) / kW2Warps;
-    const uint64_t wave = static_cast<uint64_t>(sms[dev]) * kW2BlocksPerSM;
+    const uint64_t wave = static_cast<uint64_t>(sms) * kW2BlocksPerSM;
     const int blocks = static_cast<int>(want < wave ? want : wave);
     w2_rows_kernel<<<blocks, kW2Warps * 32, kW2TableBytes, st>>>(lat, L, nrows, plane_rows, rows);
     e = cudaGetLastError();
@@ -577,6 +794,41 @@ cudaError_t launch_w2_rows(const uint32_t *lat, uint32_t L, uint32_t nrows, uint
     if (e != cudaSuccess) return e;
     w2_combine_kernel<<<1, kW2CombineThreads, 0, st>>>(rows, L, nrows, out);
     return cudaGetLastError();
+}
+
+uint32_t w2_small_split(W2Job *jobs, uint32_t n) {
+    uint64_t words = 0;
+    for (uint32_t i = 0; i < n; ++i) words += static_cast<uint64_t>(jobs[i].nrows) * (jobs[i].L >> 5);
+    // As many words per lane (up to 16) as still leave a full device of
+    // warps: the scan and the sums over the lanes of a row cost about three
+    // words' work, but few warps leave the chip idle.
+    uint32_t lw = 0;
+    while (lw < 4u && (words >> (5u + lw + 1u)) >= 4096u) ++lw;
+    uint32_t tasks = 0, rows = 0;
+    for (uint32_t i = 0; i < n; ++i) {
+        W2Job &j = jobs[i];
+        const uint32_t wpr = j.L >> 5;
+        j.lw_log = lw;
+        while ((32u << j.lw_log) < wpr) ++j.lw_log;
+        while (j.lw_log > 0u && (1u << (j.lw_log - 1u)) >= wpr) --j.lw_log;  // a row of few words
+        j.sl_log = 0;
+        while (((1u << j.sl_log) << j.lw_log) < wpr) ++j.sl_log;
+        j.task_first = tasks;
+        j.row_first = rows;
+        const uint32_t per = 32u >> j.sl_log;
+        tasks += (j.nrows + per - 1u) / per;
+        rows += j.nrows;
+    }
+    return tasks;
+}
+
+cudaError_t launch_w2_small(const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows, cudaStream_t st) {
+    return w2_small(W2Job{}, jobs, n, n_tasks, rows, st);
+}
+
+cudaError_t launch_w2_small_one(W2Job job, W2RowSums *rows, cudaStream_t st) {
+    const uint32_t n_tasks = w2_small_split(&job, 1);
+    return w2_small(job, nullptr, 1, n_tasks, rows, st);
 }
 
 cudaError_t launch_pack_canonical(const uint32_t *lat, uint32_t L, uint32_t cy0, uint32_t ncy,

@@ -71,6 +71,34 @@ struct W2Result {
     long long e_last;  // h(0, .) of the last row
     long long f0;      // 2 Y(0, first row) - 1
 };
+// Largest side the one-pass roughness kernels (w2_small_*) take.
+constexpr uint32_t kW2SmallL = 16384;
+
+// One lattice of a w2_small launch.
+struct W2Job {
+    const uint32_t *lat;
+    uint32_t L, nrows, plane_rows;
+    uint32_t row_first;   // its first record in the launch's row scratch
+    uint32_t task_first;  // its first warp task
+    uint32_t lw_log, sl_log;  // log2 of the words per lane and of the lanes per row
+    W2Result *res;        // device or page-locked host memory, like cnt_out and t_out
+    // sums of cnt_n counters from cnt and from cnt + cnt_off on, and *t, go to
+    // cnt_out[0], cnt_out[1] and *t_out (each skipped where the source is null)
+    const unsigned long long *cnt;
+    uint32_t cnt_n, cnt_off;
+    long long *cnt_out;
+    const uint32_t *t;
+    uint32_t *t_out;
+};
+// Fills the split of every job (lw_log, sl_log, task_first, row_first) and
+// returns the number of warp tasks.
+uint32_t w2_small_split(W2Job *jobs, uint32_t n);
+// The exact sums of n lattices (sides up to kW2SmallL) in two launches.
+// jobs: the same list in device memory; rows: one record per row of them all.
+cudaError_t launch_w2_small(const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows, cudaStream_t st);
+// The same for one lattice, passed by value.
+cudaError_t launch_w2_small_one(W2Job job, W2RowSums *rows, cudaStream_t st);
+
 cudaError_t launch_w2(const uint32_t *lat, uint32_t L, W2RowSums *rows, W2Result *out,
                       cudaStream_t st);
 // The same over the first nrows rows of a buffer whose bit planes hold
