@@ -433,127 +433,239 @@ __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[1
     if (c.gy < c.GY - 1) D ^= vu;
 }
 
-// One collective step of single-hit DB (dead border) with 4 x 4-site thread
-// cells: every cell attempts a uniform site of the whole cell (site word m:
-// bits 4j, 4j+1 = x offset, 4j+2, 4j+3 = y offset of cell j in TC row m).
-// The cell's border is its last column (x = 3) and last row (y = 3), where
-// an update reaches the next cell.  DELAYED (both p and q non-zero): bulk
-// attempts, then border attempts, then corner attempts, each phase decided on
-// the state the earlier phases left; otherwise all attempts of the step are
-// decided on the state before the step, which with one rate zero never lets
-// two accepted flips meet.  Every candidate of a phase is found before any of
-// its flips is applied.
-// SPEC as for step_candidates: 1 deposition only, 2 both rates random.
-template <bool RANDOM, bool DELAYED, int SPEC = 0>
-__device__ __forceinline__ void db_step(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
-                                        const uint4 &site, uint32_t s, const LaneCtx &c, TailPool &tp,
-                                        int &net, int &draws) {
+// One-hot row masks of a DB step: sel[4m + r] holds, for every cell of TC row m
+// whose site lies in its row r, the site's column (site word m: bits 4j, 4j+1
+// = x offset, 4j+2, 4j+3 = y offset of cell j).
+__device__ __forceinline__ void db_select(const uint4 &site, uint32_t (&sel)[16]) {
     const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
-    uint32_t sel[16];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         const uint32_t u = sw[m];
-        const uint32_t A = u & kNib, B = (u >> 1) & kNib, C = (u >> 2) & kNib, Dd = (u >> 3) & kNib;
-        const uint32_t col = (~(A | B) & kNib) | ((A & ~B) << 1) | ((B & ~A) << 2) | ((A & B) << 3);
-        sel[4 * m + 0] = col & ((~(C | Dd) & kNib) * 0xFu);
-        sel[4 * m + 1] = col & ((C & ~Dd) * 0xFu);
-        sel[4 * m + 2] = col & ((Dd & ~C) * 0xFu);
-        sel[4 * m + 3] = col & ((C & Dd) * 0xFu);
+        const uint32_t base = (u & kNib) + kNib;              // 1 << (x & 1)
+        const uint32_t high = base & (((u >> 1) & kNib) * 3u);  // the cells with x >= 2
+        const uint32_t col = high * 3u + base;                  // 1 << x
+        const uint32_t C = ((u >> 2) & kNib) * 0xFu, Dd = ((u >> 3) & kNib) * 0xFu;
+        sel[4 * m + 0] = col & ~C & ~Dd;
+        sel[4 * m + 1] = col & C & ~Dd;
+        sel[4 * m + 2] = col & ~C & Dd;
+        sel[4 * m + 3] = col & C & Dd;
     }
-    uint4 W = make_uint4(0u, 0u, 0u, 0u);
-    if (RANDOM) W = level_words(s, c);
-    constexpr int kPhases = DELAYED ? 3 : 1;
+}
+
+// Flips f[R] of the lane's 16 rows and the exchange with the neighbouring
+// lanes (all lanes take part).  Flips of one row may be adjacent here (a last
+// column next to a first one), so the second X bit is a shift, not 3f.
+__device__ __forceinline__ void db_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
+                                         const uint32_t (&f)[16], const LaneCtx &c) {
+    uint32_t dE = 0u, dB0 = 0u;
 #pragma unroll
-    for (int ph = 0; ph < kPhases; ++ph) {
-        uint32_t cand[16];
+    for (int R = 0; R < 16; ++R) {
+        X[R] ^= f[R] ^ (f[R] << 1);
+        Y[R] ^= R ? f[R] ^ f[R - 1] : f[R];
+        dE |= (f[R] >> (31 - R)) & (1u << R);
+        dB0 |= (f[R] & 1u) << R;
+    }
+    D ^= f[15];
+    E ^= dE;
+    const uint32_t vr = __shfl_up_sync(kFull, dE, 1);
+    const uint32_t vl = __shfl_down_sync(kFull, dB0, 1);
+    if (c.gx > 0) {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) X[r] ^= (vr >> r) & 1u;
+    }
+    if (c.gx < c.GX - 1) E ^= vl;
+    const uint32_t vd = __shfl_up_sync(kFull, f[15], c.GX);
+    const uint32_t vu = __shfl_down_sync(kFull, f[0], c.GX);
+    if (c.gy > 0) Y[0] ^= vd;
+    if (c.gy < c.GY - 1) D ^= vu;
+}
+
+// One collective step of single-hit DB (dead border) with 4 x 4-site thread
+// cells, all attempts of the step decided on the state before it: with one
+// rate zero no two accepted flips meet.  Every cell attempts a uniform site of
+// the whole cell.  SPEC as for step_candidates: 1 deposition only.
+template <bool RANDOM, int SPEC = 0>
+__device__ __forceinline__ void db_step(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
+                                        const uint4 &site, uint32_t s, const LaneCtx &c, TailPool &tp,
+                                        int &net, int &draws) {
+    uint32_t f[16];  // the attempted sites, then the candidates, then the flips
+    db_select(site, f);
+#pragma unroll
+    for (int R = 0; R < 16; ++R) {
+        const uint32_t x = X[R];
+        const uint32_t xr = __funnelshift_r(x, E >> R, 1);
+        const uint32_t y = Y[R], yd = (R < 15) ? Y[(R + 1) & 15] : D;
+        if (SPEC == 1)
+            f[R] &= ~x & xr & ~y & yd;  // the minima
+        else
+            f[R] &= (x ^ xr) & (y ^ yd) & ~(x ^ y);
+    }
+    uint32_t acc = 0u;
+    if (RANDOM) {
         uint32_t pmin = 0u, pmax = 0u;
 #pragma unroll
-        for (int R = 0; R < 16; ++R) {
-            const bool last_row = (R & 3) == 3;
-            uint32_t mask = 0xFFFFFFFFu;  // columns of this phase in row R
-            if (DELAYED) {
-                if (ph == 0) mask = last_row ? 0u : 0x77777777u;
-                if (ph == 1) mask = last_row ? 0x77777777u : 0x88888888u;
-                if (ph == 2) mask = last_row ? 0x88888888u : 0u;
-            }
-            const uint32_t x = X[R];
-            const uint32_t xr = __funnelshift_r(x, E >> R, 1);
-            const uint32_t y = Y[R], yd = (R < 15) ? Y[(R + 1) & 15] : D;
-            if (SPEC == 1)
-                cand[R] = sel[R] & mask & ~x & xr & ~y & yd;  // the minima
-            else
-                cand[R] = sel[R] & mask & (x ^ xr) & (y ^ yd) & ~(x ^ y);
-        }
-        if (RANDOM) {
+        for (int m = 0; m < 4; ++m) {
+            uint32_t mn = 0u, mx = 0u;
 #pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                uint32_t mn = 0u, mx = 0u;
-#pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    mn |= cand[4 * m + r] & ~X[4 * m + r];
-                    mx |= cand[4 * m + r] & X[4 * m + r];
-                }
-                if (SPEC != 2) {
-                    mn &= c.p_random;
-                    mx &= c.q_random;
-                }
-                pmin |= ((mn | (mn >> 1) | (mn >> 2) | (mn >> 3)) & kNib) << m;
-                pmax |= ((mx | (mx >> 1) | (mx >> 2) | (mx >> 3)) & kNib) << m;
+            for (int r = 0; r < 4; ++r) {
+                mn |= f[4 * m + r] & ~X[4 * m + r];
+                mx |= f[4 * m + r] & X[4 * m + r];
             }
-            draws += __popc(pmin | pmax);
+            mn &= c.p_random;
+            mx &= c.q_random;
+            pmin |= ((mn | (mn >> 1) | (mn >> 2) | (mn >> 3)) & kNib) << m;
+            pmax |= ((mx | (mx >> 1) | (mx >> 2) | (mx >> 3)) & kNib) << m;
         }
-        uint32_t acc = 0u;
-        if (RANDOM) {
-            acc = accept_candidates<kPreDb>(pmin, pmax, W, c, tp);
-            net += random_net(acc, pmin, pmax);
-        }
-        uint32_t dE = 0u, dB0 = 0u, dD = 0u, dY0 = 0u;
-#pragma unroll
-        for (int R = 0; R < 16; ++R) {
-            const int m = R >> 2;
-            uint32_t amin = c.p_always, amax = c.q_always;
-            if (RANDOM) {
-                const uint32_t spread = ((acc >> m) & kNib) * 0xFu;
-                amin |= spread & c.p_random;
-                amax |= spread & c.q_random;
-            }
-            const uint32_t x = X[R];
-            uint32_t f;
-            if (SPEC == 1) {
-                f = cand[R];
-                net += __popc(f);
-            } else if (SPEC == 2) {
-                f = cand[R] & ((acc >> m) & kNib) * 0xFu;
-            } else {
-                f = cand[R] & ((~x & amin) | (x & amax));
-                net += always_net<RANDOM>(f, x, c);
-            }
-            X[R] = x ^ f ^ (f << 1);
-            Y[R] ^= f;
-            if (R < 15)
-                Y[(R + 1) & 15] ^= f;
-            else {
-                D ^= f;
-                dD = f;
-            }
-            dE |= (f >> 31) << R;
-            dB0 |= (f & 1u) << R;
-            if (R == 0) dY0 = f;
-        }
-        // exchange with the neighbouring lanes (all lanes take part)
-        E ^= dE;
-        const uint32_t vr = __shfl_up_sync(kFull, dE, 1);
-        const uint32_t vl = __shfl_down_sync(kFull, dB0, 1);
-        if (c.gx > 0) {
-#pragma unroll
-            for (int r = 0; r < 16; ++r) X[r] ^= (vr >> r) & 1u;
-        }
-        if (c.gx < c.GX - 1) E ^= vl;
-        const uint32_t vd = __shfl_up_sync(kFull, dD, c.GX);
-        const uint32_t vu = __shfl_down_sync(kFull, dY0, c.GX);
-        if (c.gy > 0) Y[0] ^= vd;
-        if (c.gy < c.GY - 1) D ^= vu;
+        draws += __popc(pmin | pmax);
+        acc = accept_candidates<kPreDb>(pmin, pmax, level_words(s, c), c, tp);
+        net += random_net(acc, pmin, pmax);
     }
+#pragma unroll
+    for (int R = 0; R < 16; ++R) {
+        if (SPEC == 1) {
+            net += __popc(f[R]);
+            continue;
+        }
+        const uint32_t x = X[R];
+        uint32_t amin = c.p_always, amax = c.q_always;
+        if (RANDOM) {
+            const uint32_t spread = ((acc >> (R >> 2)) & kNib) * 0xFu;
+            amin |= spread & c.p_random;
+            amax |= spread & c.q_random;
+        }
+        f[R] &= (~x & amin) | (x & amax);
+        net += always_net<RANDOM>(f[R], x, c);
+    }
+    db_apply(X, Y, E, D, f, c);
+}
+
+// Four words holding one value bit per cell of TC row m in nibble j (at most
+// one bit set, at any of its four places; a zero nibble is 0): packed to bit
+// 4j+m.  The words are folded in pairs, so that a fold serves two of them.
+__device__ __forceinline__ uint32_t pack_cells(uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+    constexpr uint32_t k3 = 0x33333333u, k5 = 0x55555555u;
+    v0 |= v0 >> 2;
+    v1 |= v1 >> 2;
+    v2 |= v2 >> 2;
+    v3 |= v3 >> 2;
+    uint32_t a = (v0 & k3) | ((v2 << 2) & ~k3);  // bits 0, 1: TC row 0; bits 2, 3: TC row 2
+    uint32_t b = (v1 & k3) | ((v3 << 2) & ~k3);
+    a |= a >> 1;
+    b |= b >> 1;
+    return (a & k5) | ((b << 1) & ~k5);
+}
+
+// The cells' bit b of their site word nibbles for all TC rows: q[b] bit 4j+m =
+// bit 4j+b of word m (a 4 x 4 transposition in every nibble).
+__device__ __forceinline__ void transpose_nibbles(const uint4 &site, uint32_t (&q)[4]) {
+    constexpr uint32_t k3 = 0x33333333u, k5 = 0x55555555u;
+    const uint32_t a0 = (site.x & k5) | ((site.y << 1) & ~k5), a1 = ((site.x >> 1) & k5) | (site.y & ~k5);
+    const uint32_t b0 = (site.z & k5) | ((site.w << 1) & ~k5), b1 = ((site.z >> 1) & k5) | (site.w & ~k5);
+    q[0] = (a0 & k3) | ((b0 << 2) & ~k3);
+    q[1] = (a1 & k3) | ((b1 << 2) & ~k3);
+    q[2] = ((a0 >> 2) & k3) | (b0 & ~k3);
+    q[3] = ((a1 >> 2) & k3) | (b1 & ~k3);
+}
+
+// The DB step with delayed borders (both rates non-zero): bulk attempts, then
+// border attempts (last column x = 3 or last row y = 3 of a cell, where an
+// update reaches the next cell), then corner attempts (both), each decided on
+// the state the earlier ones left.
+//
+// The rows are visited twice only, once to read the four slope bits of every
+// attempt and once to flip, instead of in each of the three phases: a cell
+// makes one attempt a step, so the only flips that a later attempt can see
+// are those of the cell to its right at the same height (it changes X(s+x) of
+// a border attempt in the last column by a bulk flip at x = 0, and of a corner
+// by a border flip at (0, 3)) and of the cell below it at the same column
+// (Y(s+y), by a bulk flip at y = 0, and for a corner by a border flip at
+// (3, 0)).  So the phases run on words of one bit per cell (bit 4j+m, where
+// the acceptance draws are anyway): a = X(s) != X(s+x) and b = Y(s) != Y(s+y)
+// before the step, toggled where such a flip was accepted.  A third fewer
+// shuffles too (8 instead of 12).  Bound by the integer pipe on large
+// lattices and by latency where a step has few warps per scheduler: 2 MCS of
+// L=12288 (256x64, p=0.95, q=0.05; 3.8 warps per scheduler) went from 628 to
+// 511 us.
+template <bool RANDOM, int SPEC = 0>
+__device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
+                                                const uint4 &site, uint32_t s, const LaneCtx &c, TailPool &tp,
+                                                int &net, int &draws) {
+    uint32_t sel[16];
+    db_select(site, sel);
+    uint32_t a[4], b[4], lo[4], hi[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        a[m] = b[m] = lo[m] = hi[m] = 0u;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int R = 4 * m + r;
+            const uint32_t x = X[R], xr = __funnelshift_r(x, E >> R, 1);
+            const uint32_t y = Y[R], yd = (R < 15) ? Y[(R + 1) & 15] : D;
+            a[m] |= sel[R] & (x ^ xr);
+            b[m] |= sel[R] & (y ^ yd);
+            lo[m] |= sel[R] & ~x & ~y;
+            hi[m] |= sel[R] & x & y;
+        }
+    }
+    uint32_t A = pack_cells(a[0], a[1], a[2], a[3]), B = pack_cells(b[0], b[1], b[2], b[3]);
+    const uint32_t LO = pack_cells(lo[0], lo[1], lo[2], lo[3]);  // X(s) = Y(s) = 0: a minimum where a and b
+    const uint32_t HI = pack_cells(hi[0], hi[1], hi[2], hi[3]);  // X(s) = Y(s) = 1: a maximum
+    uint32_t q[4];
+    transpose_nibbles(site, q);
+    const uint32_t x0 = q[0], x1 = q[1], y0 = q[2], y1 = q[3];  // site coordinates in the cell
+    const uint32_t xlast = x0 & x1, ylast = y0 & y1;
+    uint4 W = make_uint4(0u, 0u, 0u, 0u);
+    if (RANDOM) W = level_words(s, c);
+
+    // accepted flips of one phase (cls: its cells)
+    auto phase = [&](uint32_t cls) {
+        const uint32_t can = A & B & cls, mn = can & LO, mx = can & HI;
+        if (!RANDOM) {
+            const uint32_t fn = mn & c.p_always, fx = mx & c.q_always;
+            net += __popc(fn) - __popc(fx);
+            return fn | fx;
+        }
+        const uint32_t pmin = SPEC == 2 ? mn : mn & c.p_random, pmax = SPEC == 2 ? mx : mx & c.q_random;
+        draws += __popc(pmin | pmax);
+        uint32_t f = accept_candidates<kPreDb>(pmin, pmax, W, c, tp);
+        net += random_net(f, pmin, pmax);
+        if (SPEC != 2) {
+            const uint32_t fn = mn & c.p_always, fx = mx & c.q_always;
+            net += __popc(fn) - __popc(fx);
+            f |= fn | fx;
+        }
+        return f;
+    };
+    // v of the cell to the right (from the next lane's low nibble vr) and below (vb: the next lane row's TC row 0)
+    auto right = [](uint32_t v, uint32_t vr) { return __funnelshift_r(v, vr, 4); };
+    auto below = [](uint32_t v, uint32_t vb) { return ((v >> 1) & 0x77777777u) | ((vb & kNib) << 3); };
+    const bool has_r = c.gx < c.GX - 1, has_b = c.gy < c.GY - 1;
+
+    uint32_t F = phase(~(xlast | ylast));  // bulk
+    {
+        const uint32_t gl = F & ~(x0 | x1), gt = F & ~(y0 | y1);  // flips in a cell's first column, first row
+        uint32_t pr = (gl & 15u) | ((y0 & 15u) << 4) | ((y1 & 15u) << 8);
+        uint32_t pb = (gt & kNib) | ((x0 & kNib) << 1) | ((x1 & kNib) << 2);
+        pr = __shfl_down_sync(kFull, pr, 1);
+        pb = __shfl_down_sync(kFull, pb, c.GX);
+        if (!has_r) pr = 0u;
+        if (!has_b) pb = 0u;
+        A ^= xlast & right(gl, pr) & ~(y0 ^ right(y0, pr >> 4)) & ~(y1 ^ right(y1, pr >> 8));
+        B ^= ylast & below(gt, pb) & ~(x0 ^ below(x0, pb >> 1)) & ~(x1 ^ below(x1, pb >> 2));
+    }
+    const uint32_t F2 = phase(xlast ^ ylast);  // borders
+    {
+        const uint32_t gl = F2 & ~(x0 | x1) & ylast, gt = F2 & ~(y0 | y1) & xlast;
+        uint32_t pr = __shfl_down_sync(kFull, gl, 1), pb = __shfl_down_sync(kFull, gt, c.GX);
+        if (!has_r) pr = 0u;
+        if (!has_b) pb = 0u;
+        A ^= right(gl, pr);
+        B ^= below(gt, pb);
+    }
+    F |= F2 | phase(xlast & ylast);  // corners
+#pragma unroll
+    for (int R = 0; R < 16; ++R) sel[R] &= ((F >> (R >> 2)) & kNib) * 0xFu;
+    db_apply(X, Y, E, D, sel, c);
 }
 
 // A collective step of DTrDTr (Sec. 4.1.2): DT whose
@@ -1022,13 +1134,13 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             // DB: one site word per TC row and step, 4 bits per cell
             site = philox4x32_10(c.t, c.k | (s << 2), c.T, (kTagSiteDb << 28) | c.g, c.k0, c.k1);
             if (SCHEME == 2)
-                db_step<RANDOM, true>(X, Y, E, D, site, s, c, tp, net, draws);
+                db_step_delayed<RANDOM>(X, Y, E, D, site, s, c, tp, net, draws);
             else if (SCHEME == 7)
-                db_step<RANDOM, true, 2>(X, Y, E, D, site, s, c, tp, net, draws);
+                db_step_delayed<RANDOM, 2>(X, Y, E, D, site, s, c, tp, net, draws);
             else if (SCHEME == 6)
-                db_step<RANDOM, false, 1>(X, Y, E, D, site, s, c, tp, net, draws);
+                db_step<RANDOM, 1>(X, Y, E, D, site, s, c, tp, net, draws);
             else
-                db_step<RANDOM, false>(X, Y, E, D, site, s, c, tp, net, draws);
+                db_step<RANDOM>(X, Y, E, D, site, s, c, tp, net, draws);
             continue;
         }
         if ((s & 1u) == 0u)
