@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
         c.gx = sub % c.GX;
         c.gy = sub / c.GX;
         c.active = active;
-        c.last = lane | (G - 1);
+        c.base = lane & ~(G - 1);
         c.t = t;
         c.k = k;
         c.T = it.T;

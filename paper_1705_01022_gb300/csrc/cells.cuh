@@ -337,7 +337,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacke
     const uint32_t G = a.GX * a.GY;
     const bool active = static_cast<uint32_t>(lane) < G;
     c.active = active;
-    c.last = static_cast<int>(G - 1u);
+    c.base = 0;
     c.t = t;
     c.k = a.k;
     c.T = T;

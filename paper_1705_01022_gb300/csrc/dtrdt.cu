@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     c.gy = static_cast<int>(sub) / c.GX;
     const bool active = sub < G && w < n_tiles;
     c.active = active;
-    c.last = static_cast<int>(seg * S + G - 1u);
+    c.base = static_cast<int>(seg * S);
     c.t = t;
     c.k = a.k;
     c.T = T;
@@ -109,6 +109,9 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     run_subtile<RANDOM, PACKED, SCHEME>(a.lat, L, a.plane_rows, wpr, a.Bx, a.By, x0, y0, active, c,
                                         ring + ((threadIdx.x >> 5) * 32 + seg * S) * kRingWordsPerLane,
                                         net, draws, tails);
+    // lanes that hold no group (a packed sub-tile of, say, six groups has eight
+    // lanes) see phantom slopes of the next sub-tile: they count nothing
+    if (PACKED && !active) net = draws = 0;
 
     // Net flips (and acceptance draws): one atomic per warp into a spread of counters.
     const uint32_t T0 = warp_id * per_warp;  // (work index: only spreads the atomics)
@@ -131,10 +134,8 @@ __global__ void advance_t_kernel(uint32_t *t_ptr) { *t_ptr += 1u; }
 cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t st) {
     if (a.cx != 4u || a.cy != 4u) return launch_cells_step(a, any_random, st);
     const uint32_t n_tiles = work_tiles(a);
-    // DTrDTr routes cells between the lanes of one sub-tile with warp-wide
-    // shuffles whose pattern depends on its own draws: one sub-tile per warp.
     const uint32_t S = segment_lanes(a.GX * a.GY);
-    const bool packed = S < 32u && a.scheme != 3u;
+    const bool packed = S < 32u;
     const uint32_t per_block = kStepWarpsPerBlock * (packed ? 32u / S : 1u);
     const uint32_t blocks = (n_tiles + per_block - 1) / per_block;
     const dim3 grid(blocks), block(kStepWarpsPerBlock * 32);
@@ -163,7 +164,13 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t s
                 OCT_LAUNCH(2, false);
             break;
         case 3:
-            OCT_LAUNCH(3, false);
+            // Packed like the others: 2 MCS of 64x64 sub-tiles (four to a warp) at L=8192,
+            // p=0.95, q=0.05 take 304 us, 804 with one sub-tile per warp; 4 MCS at L=512
+            // (16 sub-tiles a step, no shortage of warps to hide) 402 and 457 us.
+            if (packed)
+                OCT_LAUNCH(3, true);
+            else
+                OCT_LAUNCH(3, false);
             break;
         default:
             if (!any_random && a.p_always == 0xFFFFFFFFu && a.q_always == 0u) {

@@ -44,7 +44,7 @@ struct LaneCtx {
     uint32_t thr_p, thr_q;
     uint32_t p_always, q_always, p_random, q_random;
     int gx, gy, GX, GY;
-    int last;      // lane holding the sub-tile's last group
+    int base;      // lane of the sub-tile's first group
     bool active;   // this lane holds a group of a sub-tile
 };
 
@@ -682,26 +682,29 @@ __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)
 // uniforms, and the order of ties, stay those of the owning thread cell), and
 // the decision returns to the holder, which flips.  The neighbour copies E, D
 // are kept as in DT: the lattice itself does not wrap inside the sub-tile.
-// As for DT the step runs in three phases (candidates and flips specialised
-// on R0, one copy of the acceptance code between them).
+// As for DT the step runs in three phases, with one copy of the acceptance code
+// between the candidates and the flips.
+// PACKED: the warp holds several sub-tiles, each with its own phase (c0, R0),
+// so every shuffle runs on all lanes and its value is taken where the lane's
+// phase asks for it (a lane only reads lanes of its own sub-tile).
 struct DtrLanes {
-    int lL, lR, lA, lB, lAL, lBR;  // lanes left, right, above, below, above-left, below-right (wrapping)
+    int lL, lR, lA, lB, lAL, lBR;  // lanes of the sub-tile left, right, above, below, above-left, below-right (wrapping)
 };
 
 __device__ __forceinline__ DtrLanes dtr_lanes(const LaneCtx &c) {
     const int gxl = c.gx == 0 ? c.GX - 1 : c.gx - 1, gxr = c.gx == c.GX - 1 ? 0 : c.gx + 1;
     const int gya = c.gy == 0 ? c.GY - 1 : c.gy - 1, gyb = c.gy == c.GY - 1 ? 0 : c.gy + 1;
     DtrLanes n;
-    n.lL = gxl + c.gy * c.GX;
-    n.lR = gxr + c.gy * c.GX;
-    n.lA = c.gx + gya * c.GX;
-    n.lB = c.gx + gyb * c.GX;
-    n.lAL = gxl + gya * c.GX;
-    n.lBR = gxr + gyb * c.GX;
+    n.lL = c.base + gxl + c.gy * c.GX;
+    n.lR = c.base + gxr + c.gy * c.GX;
+    n.lA = c.base + c.gx + gya * c.GX;
+    n.lB = c.base + c.gx + gyb * c.GX;
+    n.lAL = c.base + gxl + gya * c.GX;
+    n.lBR = c.base + gxr + gyb * c.GX;
     return n;
 }
 
-// v[k] for a run-time k in 0..3 (k uniform over the warp: selects, no branch).
+// v[k] for a run-time k in 0..3 (selects, no branch).
 __device__ __forceinline__ uint32_t pick4(uint32_t k, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
     const uint32_t lo = (k & 1u) ? v1 : v0, hi = (k & 1u) ? v3 : v2;
     return (k & 2u) ? hi : lo;
@@ -713,13 +716,13 @@ __device__ __forceinline__ uint32_t pick4(uint32_t k, uint32_t v0, uint32_t v1, 
 // row 16 (m = 3, R0 = 3) is the lane below's row 0, and cb[3] then holds this
 // lane's row 0 (the wrapped row of the lane above) instead.
 // pmin / pmax: packed candidates of this lane's own thread cells.
-template <bool RANDOM>
+template <bool RANDOM, bool PACKED>
 __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const uint32_t (&Y)[16], uint32_t E,
                                                uint32_t D, const uint4 &site, uint32_t s, uint32_t c0,
                                                uint32_t R0, const LaneCtx &c, const DtrLanes &n,
                                                uint32_t (&ca)[4], uint32_t (&cb)[4], uint32_t &pmin,
                                                uint32_t &pmax) {
-    const bool SX = c0 == 3u;  // pairs reach column 32 (uniform over the warp)
+    const bool SX = c0 == 3u;  // pairs reach column 32
     const bool SY = R0 == 3u;  // pairs reach row 16
     const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
     const uint32_t par = 2u * (s & 1u);
@@ -746,8 +749,9 @@ __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const ui
         }
     }
     // sites of neighbouring lanes' thread cells held by this lane
-    if (SX) {
-        const uint32_t v = __shfl_sync(kFull, xw, n.lL);
+    if (PACKED || SX) {
+        uint32_t v = __shfl_sync(kFull, xw, n.lL);
+        if (PACKED) v = SX ? v : 0u;
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             const uint32_t ya = 4u * m + R0;
@@ -755,10 +759,11 @@ __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const ui
             if (!(m == 3 && SY)) cb[m] |= (v >> (ya + 1u)) & 1u;
         }
     }
-    if (SY) {
+    if (PACKED || SY) {
         const uint32_t v = __shfl_sync(kFull, yw, n.lA);
-        const uint32_t corner = SX ? (__shfl_sync(kFull, xw, n.lAL) >> 16) & 1u : 0u;
-        cb[3] = v | corner;  // row 0
+        uint32_t corner = 0u;
+        if (PACKED || SX) corner = (__shfl_sync(kFull, xw, n.lAL) >> 16) & (SX ? 1u : 0u);
+        if (SY) cb[3] = v | corner;  // row 0
     }
     // eligibility; rows a and b of TC row m picked by the row phase (for
     // m = 3 the row after 15 is D for Y, and row b = "16" is row 0)
@@ -790,10 +795,12 @@ __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const ui
     pmin = 0u;
     pmax = 0u;
     if (RANDOM) {
-        const uint32_t cwR = SX ? __shfl_sync(kFull, cw, n.lR) : 0u;
-        const uint32_t cwBR = (SX && SY) ? __shfl_sync(kFull, cw, n.lBR) : 0u;
-        uint32_t bmin = 0u, bmax = 0u;  // row 0 of the lane below
-        if (SY) {
+        uint32_t cwR = 0u, cwBR = 0u;
+        if (PACKED || SX) cwR = __shfl_sync(kFull, cw, n.lR);
+        if (PACKED || (SX && SY)) cwBR = __shfl_sync(kFull, cw, n.lBR);
+        if (PACKED && !SX) cwR = cwBR = 0u;
+        uint32_t bmin = 0u, bmax = 0u;  // row 0 of the lane below (used with R0 = 3)
+        if (PACKED || SY) {
             bmin = __shfl_sync(kFull, cb[3] & ~X[0], n.lB);
             bmax = __shfl_sync(kFull, cb[3] & X[0], n.lB);
         }
@@ -833,7 +840,7 @@ __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const ui
 // row r come from TC row m = r / 4 when r % 4 is R0 (row a) or R0 + 1 (row b),
 // and from TC row m - 1 (mod 4: row 0 takes the wrapped row of TC row 3) when
 // r % 4 = 0 and R0 = 3.
-template <bool RANDOM>
+template <bool RANDOM, bool PACKED>
 __device__ __forceinline__ void dtr_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                           uint32_t c0, uint32_t R0, uint32_t acc, const uint32_t (&ca)[4],
                                           const uint32_t (&cb)[4], const LaneCtx &c, const DtrLanes &n,
@@ -842,9 +849,10 @@ __device__ __forceinline__ void dtr_apply(uint32_t (&X)[16], uint32_t (&Y)[16], 
     const bool SY = R0 == 3u;
     uint32_t accL = 0u, accA = 0u, accAL = 0u;
     if (RANDOM) {
-        if (SX) accL = __shfl_sync(kFull, acc, n.lL);
-        if (SY) accA = __shfl_sync(kFull, acc, n.lA);
-        if (SX && SY) accAL = __shfl_sync(kFull, acc, n.lAL);
+        // (read only by the columns and rows that wrap)
+        if (PACKED || SX) accL = __shfl_sync(kFull, acc, n.lL);
+        if (PACKED || SY) accA = __shfl_sync(kFull, acc, n.lA);
+        if (PACKED || (SX && SY)) accAL = __shfl_sync(kFull, acc, n.lAL);
     }
     // accepted candidates of rows a and b of every TC row (fb[3] with R0 = 3: row 0)
     uint32_t fa[4], fb[4];
@@ -1120,14 +1128,14 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             const uint32_t r0 = (((byte >> 4) & 3u) + 2u * (d >> 1)) & 3u;
             const DtrLanes n = dtr_lanes(c);
             uint32_t ca[4], cb[4], pmin, pmax;
-            dtr_candidates<RANDOM>(X, Y, E, D, site, s, c0, r0, c, n, ca, cb, pmin, pmax);
+            dtr_candidates<RANDOM, LANE_SETS>(X, Y, E, D, site, s, c0, r0, c, n, ca, cb, pmin, pmax);
             uint32_t acc = 0u;
             if (RANDOM) {
                 draws += __popc(pmin | pmax);
                 acc = accept_candidates<SCHEME == 3 ? kPreDtr : (LANE_SETS ? kPrePacked : kPreDt)>(pmin, pmax, level_words(s, c), c, tp);
                 net += random_net(acc, pmin, pmax);
             }
-            dtr_apply<RANDOM>(X, Y, E, D, c0, r0, acc, ca, cb, c, n, net);
+            dtr_apply<RANDOM, LANE_SETS>(X, Y, E, D, c0, r0, acc, ca, cb, c, n, net);
             continue;
         }
         if (SCHEME == 1 || SCHEME == 2 || SCHEME == 6 || SCHEME == 7) {
