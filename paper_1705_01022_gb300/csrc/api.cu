@@ -254,6 +254,10 @@ int sim_create(const oct_params *prm, oct_sim **out) {
     a.tiles_y = static_cast<uint32_t>(s->L / (2 * By));
     a.k0 = static_cast<uint32_t>(s->seed & 0xFFFFFFFFu);
     a.k1 = static_cast<uint32_t>(s->seed >> 32);
+    for (uint32_t r = 0; r < 10u; ++r) {  // Philox round keys
+        a.rk0[r] = a.k0 + r * 0x9E3779B9u;
+        a.rk1[r] = a.k1 + r * 0xBB67AE85u;
+    }
     const bool p_rand = s->p > 0.0 && s->p < 1.0, q_rand = s->q > 0.0 && s->q < 1.0;
     a.thr_p = p_rand ? threshold32(s->p) : 0u;
     a.thr_q = q_rand ? threshold32(s->q) : 0u;

@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
             (static_cast<uint64_t>(ox) + 2ull * R.Bx * tx + static_cast<uint64_t>(R.Bx) * (sigma & 1)) % L);
         const uint32_t y0 = static_cast<uint32_t>(
             (static_cast<uint64_t>(oy) + 2ull * R.By * ty + static_cast<uint64_t>(R.By) * (sigma >> 1)) % L);
-        LaneCtx c;
+        LaneCtx<KeysWeyl> c;
         c.GX = static_cast<int>(wd.GX);
         c.GY = G / c.GX;
         c.gx = sub % c.GX;
@@ -100,8 +100,8 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
         c.k = k;
         c.T = it.T;
         c.g = static_cast<uint32_t>(sub);
-        c.k0 = R.k0;
-        c.k1 = R.k1;
+        c.key = KeysWeyl{R.k0, R.k1};
+        c.first_round();
         c.thr_p = R.thr_p;
         c.thr_q = R.thr_q;
         c.p_always = R.p_always;

@@ -58,7 +58,7 @@ struct CellShape {
 // (for the tail-stream refill); gr, gh its group row and lane row inside the
 // group; m0 the TC row m of its first TC row.
 struct CellCtx {
-    LaneCtx c;
+    LaneCtx<KeysConst> c;
     int lane;
     int gr, gh;
     uint32_t m0;
@@ -139,7 +139,7 @@ __device__ __forceinline__ void cells_candidates(const uint32_t (&X)[16], const 
 template <int GS>
 __device__ __forceinline__ uint32_t cells_accept(uint32_t pmin, uint32_t pmax, const uint4 &W, const CellCtx &cc,
                                                  TailPool &tp) {
-    const LaneCtx &c = cc.c;
+    const LaneCtx<KeysConst> &c = cc.c;
     const uint32_t lw[4] = {W.x, W.y, W.z, W.w};
     uint32_t acc = 0, und = pmin | pmax;
 #pragma unroll
@@ -190,7 +190,7 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
                                             uint32_t dx, uint32_t acc, const uint32_t (&cand)[8], const CellCtx &cc,
                                             int &net) {
     using S = CellShape<CX, CY>;
-    const LaneCtx &c = cc.c;
+    const LaneCtx<KeysConst> &c = cc.c;
     uint32_t dE = 0u, dB0 = 0u, dD = 0u, dY0 = 0u;
 #pragma unroll
     for (int i = 0; i < S::NTR; ++i) {
@@ -265,24 +265,25 @@ __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uin
                                                   uint32_t x0, uint32_t y0, bool active, const CellCtx &cc,
                                                   uint32_t *ring, int &net, int &draws, int &tails) {
     using S = CellShape<CX, CY>;
-    const LaneCtx &c = cc.c;
+    const LaneCtx<KeysConst> &c = cc.c;
     TailPool tp;
     tp.ring = ring + static_cast<uint32_t>(kRingWordsPerLane) * static_cast<uint32_t>(cc.lane);  // own slot
     tp.head = 0u;
     tp.end = 0u;
     tp.rounds = 0u;
-    const LaneGeom q = lane_geom(lat, L, plane_rows, wpr, By, x0, y0, c);
+    const LaneGeom q = lane_geom(lat, L, plane_rows, wpr, x0, y0, c);
     uint32_t X[16], Y[16], E, D;
-    stage_lane(q, L, wpr, Bx, x0, active, c, X, Y, E, D);
+    const bool straight = lane_straight(q, L, active);
+    stage_lane(q, L, wpr, straight, active, X, Y, E, D);
 
     uint4 setw = make_uint4(0u, 0u, 0u, 0u), site = make_uint4(0u, 0u, 0u, 0u), lvl = make_uint4(0u, 0u, 0u, 0u);
     for (uint32_t s = 0; s < static_cast<uint32_t>(S::STEPS); ++s) {
-        if ((s & 63u) == 0u) setw = philox4x32_10(c.t, c.k | ((s >> 6) << 2), c.T, kTagSet << 28, c.k0, c.k1);
+        if ((s & 63u) == 0u) setw = c.draw(c.k | ((s >> 6) << 2), kTagSet << 28);
         // the set, broadcast from lane 0 (all lanes drew the same one) so that the
         // branches on it are warp-uniform for the compiler
         const uint32_t d = __shfl_sync(kFull, (word_of(setw, (s >> 4) & 3u) >> (2u * (s & 15u))) & 3u, 0);
         if (s % S::SPW == 0u)
-            site = philox4x32_10(c.t, c.k | ((s / S::SPW) << 2), c.T, (kTagSite << 28) | c.g, c.k0, c.k1);
+            site = c.draw(c.k | ((s / S::SPW) << 2), (kTagSite << 28) | c.g);
         uint32_t cand[8], pmin, pmax;
         if (d & 2u)
             cells_candidates<CX, CY, 1, RANDOM, SPEC>(X, Y, E, D, site, s, d & 1u, cc, cand, pmin, pmax);
@@ -292,7 +293,7 @@ __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uin
         if (RANDOM) {
             draws += __popc(pmin | pmax);
             if (s % S::SPL == 0u)
-                lvl = philox4x32_10(c.t, c.k | (((s / S::SPL) * 8u) << 2), c.T, (kTagAcc << 28) | c.g, c.k0, c.k1);
+                lvl = c.draw(c.k | (((s / S::SPL) * 8u) << 2), (kTagAcc << 28) | c.g);
             const uint32_t sh = (s % S::SPL) * 4u * S::TPB;  // this step's positions
             const uint4 W = make_uint4(lvl.x >> sh, lvl.y >> sh, lvl.z >> sh, lvl.w >> sh);
             acc = cells_accept<S::GS>(pmin, pmax, W, cc, tp);
@@ -303,7 +304,7 @@ __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uin
         else
             cells_apply<CX, CY, 0, RANDOM, SPEC>(X, Y, E, D, d & 1u, acc, cand, cc, net);
     }
-    write_back<false>(q, L, wpr, active, c, X, Y, E, D);
+    write_back<false>(q, L, wpr, straight, active, c, X, Y, E, D);
     tails = static_cast<int>(tp.rounds);
 }
 
@@ -316,7 +317,7 @@ __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uin
 // By (sigma>>1)) mod L.
 template <int CX, int CY, bool RANDOM, int SPEC>
 __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacked)
-    cells_step_kernel(const StepArgs a) {
+    cells_step_kernel(const __grid_constant__ StepArgs a) {
     using S = CellShape<CX, CY>;
     __shared__ __align__(16) uint32_t ring[kStepWarpsPerBlock * 32 * kRingWordsPerLane];
     const int lane = threadIdx.x & 31;
@@ -329,7 +330,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacke
     const uint32_t T = pl.T, x0 = pl.x0, y0 = pl.y0;
 
     CellCtx cc;
-    LaneCtx &c = cc.c;
+    LaneCtx<KeysConst> &c = cc.c;
     c.GX = static_cast<int>(a.GX);
     c.GY = static_cast<int>(a.GY);
     c.gx = lane % c.GX;
@@ -341,8 +342,8 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacke
     c.t = t;
     c.k = a.k;
     c.T = T;
-    c.k0 = a.k0;
-    c.k1 = a.k1;
+    c.key.a = &a;
+    c.first_round();
     c.thr_p = a.thr_p;
     c.thr_q = a.thr_q;
     c.p_always = a.p_always;

@@ -36,6 +36,8 @@
 //             four words of (t, k|(s*8)<<2, T, ACC<<28|g); bits 27..0, needed
 //             only when those tie with P32's, are the top of the next word of
 //             the sub-tile's tail stream (t, k|(i/4)<<2, T, TAIL<<28)
+#include <type_traits>
+
 #include "oct_internal.h"
 
 #include "subtile.cuh"
@@ -65,7 +67,7 @@ constexpr int step_min_blocks(int scheme, bool packed) {
 
 template <bool RANDOM, int SCHEME, bool PACKED>
 __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEME, PACKED))
-    dtrdt_step_kernel(const StepArgs a) {
+    dtrdt_step_kernel(const __grid_constant__ StepArgs a) {
     __shared__ __align__(16) uint32_t ring[kStepWarpsPerBlock * 32 * kRingWordsPerLane];
     const int lane = threadIdx.x & 31;
     const uint32_t G = a.GX * a.GY;
@@ -83,7 +85,11 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     const TilePlace pl = place_tile(a, w < n_tiles ? w : 0u, t);
     const uint32_t T = pl.T, x0 = pl.x0, y0 = pl.y0;
 
-    LaneCtx c;
+    // Deposition only draws one block per two steps: there the key additions are
+    // cheaper than the constant operands (127.6 and 135.0 us for one MCS at L=16384,
+    // 256x64); with draws the constants win (L=2^17, 1024x16, p=0.95: see subtile.cuh).
+    constexpr bool kWeyl = SCHEME == 4;
+    LaneCtx<std::conditional_t<kWeyl, KeysWeyl, KeysConst>> c;
     c.GX = static_cast<int>(a.GX);
     c.GY = static_cast<int>(a.GY);
     c.gx = static_cast<int>(sub) % c.GX;
@@ -95,8 +101,11 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     c.k = a.k;
     c.T = T;
     c.g = sub;
-    c.k0 = a.k0;
-    c.k1 = a.k1;
+    if constexpr (kWeyl)
+        c.key = KeysWeyl{a.k0, a.k1};
+    else
+        c.key.a = &a;
+    c.first_round();
     c.thr_p = a.thr_p;
     c.thr_q = a.thr_q;
     c.p_always = a.p_always;

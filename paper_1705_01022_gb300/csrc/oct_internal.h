@@ -18,6 +18,7 @@ struct StepArgs {
     uint32_t GX, GY;           // groups per sub-tile: Bx / 32 columns, By / 16 rows
     uint32_t tiles_x, tiles_y; // device tiles per direction: L / (2Bx), L / (2By)
     uint32_t k0, k1;           // Philox key
+    uint32_t rk0[10], rk1[10]; // its round keys
     uint32_t thr_p, thr_q;     // P32(p), P32(q) when the probability is strictly inside (0,1)
     uint32_t p_always, q_always;   // all-ones if p == 1 (resp. q == 1), else 0
     uint32_t p_random, q_random;   // all-ones if 0 < p < 1 (resp. q), else 0

@@ -7,6 +7,7 @@
 #pragma once
 #include <cstdint>
 
+#include "oct_internal.h"
 #include "philox.cuh"
 
 namespace oct {
@@ -38,9 +39,47 @@ __device__ __forceinline__ void reduce_bits(uint32_t *w, uint32_t v, uint32_t ma
     atomicOr(w, v & mask);
 }
 
+// Round keys of Philox: from the launch's arguments (constant memory, so that
+// they cost neither registers nor additions) or from the key itself.  With the
+// first round's products kept per sub-tile, one MCS at L=2^17 (1024x16, p=0.95,
+// q=0.05) takes 1.4 % less.
+struct KeysConst {
+    const StepArgs *a;
+    __device__ __forceinline__ uint32_t lo(int r) const { return a->rk0[r]; }
+    __device__ __forceinline__ uint32_t hi(int r) const { return a->rk1[r]; }
+};
+struct KeysWeyl {
+    uint32_t k0, k1;
+    __device__ __forceinline__ uint32_t lo(int r) const { return k0 + static_cast<uint32_t>(r) * 0x9E3779B9u; }
+    __device__ __forceinline__ uint32_t hi(int r) const { return k1 + static_cast<uint32_t>(r) * 0xBB67AE85u; }
+};
+
+template <class Keys>
 struct LaneCtx {
     uint32_t t, k, T, g;
-    uint32_t k0, k1;
+    Keys key;
+    // the first round's products of (t, ., T, .), the high halves with its keys
+    uint32_t h0, l0, h1, l1;
+    __device__ __forceinline__ void first_round() {
+        h0 = __umulhi(0xD2511F53u, t) ^ key.hi(0);
+        l0 = 0xD2511F53u * t;
+        h1 = __umulhi(0xCD9E8D57u, T) ^ key.lo(0);
+        l1 = 0xCD9E8D57u * T;
+    }
+    // Philox-4x32-10 at counter (t, c1, T, c3)
+    __device__ __forceinline__ uint4 draw(uint32_t c1, uint32_t c3) const {
+        uint32_t x0 = h1 ^ c1, x1 = l1, x2 = h0 ^ c3, x3 = l0;
+#pragma unroll
+        for (int r = 1; r < 10; ++r) {
+            const uint32_t a0 = __umulhi(0xD2511F53u, x0), b0 = 0xD2511F53u * x0;
+            const uint32_t a1 = __umulhi(0xCD9E8D57u, x2), b1 = 0xCD9E8D57u * x2;
+            x0 = a1 ^ x1 ^ key.lo(r);
+            x2 = a0 ^ x3 ^ key.hi(r);
+            x1 = b1;
+            x3 = b0;
+        }
+        return make_uint4(x0, x1, x2, x3);
+    }
     uint32_t thr_p, thr_q;
     uint32_t p_always, q_always, p_random, q_random;
     int gx, gy, GX, GY;
@@ -52,8 +91,8 @@ struct LaneCtx {
 // row's X bits before the flips) that were accepted without a draw (p = 1 or
 // q = 1).  Flips decided by a draw are counted once per step from the packed
 // acceptance bits instead (random_net).
-template <bool RANDOM>
-__device__ __forceinline__ int always_net(uint32_t f, uint32_t x, const LaneCtx &c) {
+template <bool RANDOM, class Ctx>
+__device__ __forceinline__ int always_net(uint32_t f, uint32_t x, const Ctx &c) {
     if (RANDOM) {
         if ((c.p_always | c.q_always) == 0u) return 0;
         return __popc(f & ~x & c.p_always) - __popc(f & x & c.q_always);
@@ -89,9 +128,10 @@ struct TailPool {
 // Tops up the lane's slot until it holds the `need` words after head; every
 // lane of the warp takes part in each round (one Philox block per lane, block
 // end/4 of its group's stream, kept only if the slot has room).
-__device__ __forceinline__ void tail_refill(uint32_t need, uint32_t g, const LaneCtx &c, TailPool &tp) {
+template <class Ctx>
+__device__ __forceinline__ void tail_refill(uint32_t need, uint32_t g, const Ctx &c, TailPool &tp) {
     while (__any_sync(kFull, tp.end < tp.head + need)) {
-        const uint4 B = philox4x32_10(c.t, c.k | ((tp.end >> 2) << 2), c.T, (kTagTail << 28) | g, c.k0, c.k1);
+        const uint4 B = c.draw(c.k | ((tp.end >> 2) << 2), (kTagTail << 28) | g);
         if (tp.end - tp.head <= static_cast<uint32_t>(kRingWordsPerLane - 4)) {
             *reinterpret_cast<uint4 *>(tp.ring + (tp.end & static_cast<uint32_t>(kRingWordsPerLane - 1))) = B;
             tp.end += 4u;
@@ -110,15 +150,16 @@ __device__ __forceinline__ void tail_refill(uint32_t need, uint32_t g, const Lan
 //    of its group's tail stream (word i = word i%4 of Philox(t, k|(i/4)<<2, T,
 //    TAIL<<28|g), counted from 0 each device step), the group's ties of a step
 //    in order of position.  A lane holds one group, so it takes its own words.
-__device__ __forceinline__ uint4 level_words(uint32_t s, const LaneCtx &c) {
-    return philox4x32_10(c.t, c.k | ((s * 8u) << 2), c.T, (kTagAcc << 28) | c.g, c.k0, c.k1);
+template <class Ctx>
+__device__ __forceinline__ uint4 level_words(uint32_t s, const Ctx &c) {
+    return c.draw(c.k | ((s * 8u) << 2), (kTagAcc << 28) | c.g);
 }
 
 // PRE: tail words the lane reads at once for its first ties (0: one word per
 // tie in the loop); the fastest choice differs between the block layers.
-template <int PRE>
+template <int PRE, class Ctx>
 __device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pmax, const uint4 &W,
-                                                      const LaneCtx &c, TailPool &tp) {
+                                                      const Ctx &c, TailPool &tp) {
     const uint32_t lw[4] = {W.x, W.y, W.z, W.w};
     uint32_t acc = 0, und = pmin | pmax;
 #pragma unroll
@@ -177,10 +218,10 @@ __device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pm
 // minimum flips and no maximum does, so the candidates are the minima
 // themselves.  SPEC 2 (both 0 < p < 1 and 0 < q < 1): every candidate needs a
 // draw, so no always/never masks are applied.
-template <int DY, bool RANDOM, int SPEC = 0>
+template <int DY, bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_candidates(const uint32_t (&X)[16], const uint32_t (&Y)[16],
                                                 uint32_t E, uint32_t D, const uint4 &site, uint32_t s,
-                                                uint32_t dx, const LaneCtx &c, uint32_t (&cnd0)[4],
+                                                uint32_t dx, const Ctx &c, uint32_t (&cnd0)[4],
                                                 uint32_t (&cnd1)[4], uint32_t &pmin, uint32_t &pmax) {
     const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
     const uint32_t sh2 = 2u * dx;
@@ -228,10 +269,10 @@ __device__ __forceinline__ void step_candidates(const uint32_t (&X)[16], const u
 
 // Phase 3 with sub-cell set (dx, DY): flips of the accepted candidates (acc:
 // packed acceptance bits) and the exchange with the neighbouring lanes.
-template <int DY, bool RANDOM, int SPEC = 0>
+template <int DY, bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                            uint32_t dx, uint32_t acc, const uint32_t (&cnd0)[4],
-                                           const uint32_t (&cnd1)[4], const LaneCtx &c, int &net) {
+                                           const uint32_t (&cnd1)[4], const Ctx &c, int &net) {
     uint32_t f0s[4], f1s[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -316,10 +357,10 @@ __device__ __forceinline__ void step_apply(uint32_t (&X)[16], uint32_t (&Y)[16],
 // sub-tiles, each with its own set draw: the row offset dy is a run-time value
 // per lane (rows picked with selects instead of branches), and every shuffle
 // runs unconditionally so that all 32 lanes take part.
-template <bool RANDOM, int SPEC = 0>
+template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_candidates_rt(const uint32_t (&X)[16], const uint32_t (&Y)[16],
                                                    uint32_t E, uint32_t D, const uint4 &site, uint32_t s,
-                                                   uint32_t dx, uint32_t dy, const LaneCtx &c,
+                                                   uint32_t dx, uint32_t dy, const Ctx &c,
                                                    uint32_t (&cnd0)[4], uint32_t (&cnd1)[4],
                                                    uint32_t &pmin, uint32_t &pmax) {
     const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
@@ -357,10 +398,10 @@ __device__ __forceinline__ void step_candidates_rt(const uint32_t (&X)[16], cons
     }
 }
 
-template <bool RANDOM, int SPEC = 0>
+template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                               uint32_t dy, uint32_t acc, const uint32_t (&cnd0)[4],
-                                              const uint32_t (&cnd1)[4], const LaneCtx &c, int &net) {
+                                              const uint32_t (&cnd1)[4], const Ctx &c, int &net) {
     const uint32_t ro = 2u * dy;
     const uint32_t dym = dy ? 0xFFFFFFFFu : 0u;
     uint32_t dE = 0, dB0 = 0, dD = 0, dY0 = 0;
@@ -455,8 +496,9 @@ __device__ __forceinline__ void db_select(const uint4 &site, uint32_t (&sel)[16]
 // Flips f[R] of the lane's 16 rows and the exchange with the neighbouring
 // lanes (all lanes take part).  Flips of one row may be adjacent here (a last
 // column next to a first one), so the second X bit is a shift, not 3f.
+template <class Ctx>
 __device__ __forceinline__ void db_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
-                                         const uint32_t (&f)[16], const LaneCtx &c) {
+                                         const uint32_t (&f)[16], const Ctx &c) {
     uint32_t dE = 0u, dB0 = 0u;
 #pragma unroll
     for (int R = 0; R < 16; ++R) {
@@ -484,9 +526,9 @@ __device__ __forceinline__ void db_apply(uint32_t (&X)[16], uint32_t (&Y)[16], u
 // cells, all attempts of the step decided on the state before it: with one
 // rate zero no two accepted flips meet.  Every cell attempts a uniform site of
 // the whole cell.  SPEC as for step_candidates: 1 deposition only.
-template <bool RANDOM, int SPEC = 0>
+template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void db_step(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
-                                        const uint4 &site, uint32_t s, const LaneCtx &c, TailPool &tp,
+                                        const uint4 &site, uint32_t s, const Ctx &c, TailPool &tp,
                                         int &net, int &draws) {
     uint32_t f[16];  // the attempted sites, then the candidates, then the flips
     db_select(site, f);
@@ -586,9 +628,9 @@ __device__ __forceinline__ void transpose_nibbles(const uint4 &site, uint32_t (&
 // lattices and by latency where a step has few warps per scheduler: 2 MCS of
 // L=12288 (256x64, p=0.95, q=0.05; 3.8 warps per scheduler) went from 628 to
 // 511 us.
-template <bool RANDOM, int SPEC = 0>
+template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
-                                                const uint4 &site, uint32_t s, const LaneCtx &c, TailPool &tp,
+                                                const uint4 &site, uint32_t s, const Ctx &c, TailPool &tp,
                                                 int &net, int &draws) {
     uint32_t sel[16];
     db_select(site, sel);
@@ -691,7 +733,8 @@ struct DtrLanes {
     int lL, lR, lA, lB, lAL, lBR;  // lanes of the sub-tile left, right, above, below, above-left, below-right (wrapping)
 };
 
-__device__ __forceinline__ DtrLanes dtr_lanes(const LaneCtx &c) {
+template <class Ctx>
+__device__ __forceinline__ DtrLanes dtr_lanes(const Ctx &c) {
     const int gxl = c.gx == 0 ? c.GX - 1 : c.gx - 1, gxr = c.gx == c.GX - 1 ? 0 : c.gx + 1;
     const int gya = c.gy == 0 ? c.GY - 1 : c.gy - 1, gyb = c.gy == c.GY - 1 ? 0 : c.gy + 1;
     DtrLanes n;
@@ -716,10 +759,10 @@ __device__ __forceinline__ uint32_t pick4(uint32_t k, uint32_t v0, uint32_t v1, 
 // row 16 (m = 3, R0 = 3) is the lane below's row 0, and cb[3] then holds this
 // lane's row 0 (the wrapped row of the lane above) instead.
 // pmin / pmax: packed candidates of this lane's own thread cells.
-template <bool RANDOM, bool PACKED>
+template <bool RANDOM, bool PACKED, class Ctx>
 __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const uint32_t (&Y)[16], uint32_t E,
                                                uint32_t D, const uint4 &site, uint32_t s, uint32_t c0,
-                                               uint32_t R0, const LaneCtx &c, const DtrLanes &n,
+                                               uint32_t R0, const Ctx &c, const DtrLanes &n,
                                                uint32_t (&ca)[4], uint32_t (&cb)[4], uint32_t &pmin,
                                                uint32_t &pmax) {
     const bool SX = c0 == 3u;  // pairs reach column 32
@@ -840,10 +883,10 @@ __device__ __forceinline__ void dtr_candidates(const uint32_t (&X)[16], const ui
 // row r come from TC row m = r / 4 when r % 4 is R0 (row a) or R0 + 1 (row b),
 // and from TC row m - 1 (mod 4: row 0 takes the wrapped row of TC row 3) when
 // r % 4 = 0 and R0 = 3.
-template <bool RANDOM, bool PACKED>
+template <bool RANDOM, bool PACKED, class Ctx>
 __device__ __forceinline__ void dtr_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                           uint32_t c0, uint32_t R0, uint32_t acc, const uint32_t (&ca)[4],
-                                          const uint32_t (&cb)[4], const LaneCtx &c, const DtrLanes &n,
+                                          const uint32_t (&cb)[4], const Ctx &c, const DtrLanes &n,
                                           int &net) {
     const bool SX = c0 == 3u;
     const bool SY = R0 == 3u;
@@ -909,16 +952,16 @@ __device__ __forceinline__ void dtr_apply(uint32_t (&X)[16], uint32_t (&Y)[16], 
 }
 
 // Where a lane's group lies in the planar lattice: the two words wA, wB of
-// every row that hold its 32 sites (from bit sh of wA), its first row ybase
-// and the sub-tile's halo row yh.
+// every row that hold its 32 sites (from bit sh of wA), and its first row ybase.
 struct LaneGeom {
     uint32_t *Xp, *Yp;
-    uint32_t sh, wA, wB, ybase, yh;
+    uint32_t sh, wA, wB, ybase;
 };
 
 // (y0 in buffer rows; the Y plane follows plane_rows rows of X.)
+template <class Ctx>
 __device__ __forceinline__ LaneGeom lane_geom(uint32_t *lat, uint32_t L, uint32_t plane_rows, uint32_t wpr,
-                                              uint32_t By, uint32_t x0, uint32_t y0, const LaneCtx &c) {
+                                              uint32_t x0, uint32_t y0, const Ctx &c) {
     LaneGeom q;
     q.Xp = lat;
     q.Yp = lat + static_cast<size_t>(plane_rows) * wpr;
@@ -927,103 +970,121 @@ __device__ __forceinline__ LaneGeom lane_geom(uint32_t *lat, uint32_t L, uint32_
     q.wB = (q.wA + 1u == wpr) ? 0u : q.wA + 1u;
     q.ybase = y0 + 16u * static_cast<uint32_t>(c.gy);
     if (q.ybase >= L) q.ybase -= L;
-    q.yh = y0 + By;
-    if (q.yh >= L) q.yh -= L;
     return q;
 }
 
+// The staging and the write-back of a lane, 33 rows' words each, were a ninth
+// of the instructions of a device step when every row's address was formed
+// anew: one MCS at L=2^17 (1024x16, p=0.95, q=0.05) went from 11.15 to 10.1 ms
+// with running addresses, and with E and D taken from the words read instead
+// of by shuffles and loads of the edge lanes.
+//
+// Row r of the lane's group in words from the planes' start.  STRAIGHT: neither
+// the rows nor the two words of any lane of the warp wrap around the lattice,
+// so a row is one addition from the last and word wB follows wA; a warp that
+// wraps (one in about L/32 by words, L/16 by rows) takes the general form.
+template <bool STRAIGHT>
+struct LaneRows {
+    const LaneGeom &q;
+    uint32_t L, wpr;
+    size_t at;     // word wA of the current row
+    uint32_t row;  // the current row
+    __device__ __forceinline__ LaneRows(const LaneGeom &g, uint32_t L_, uint32_t wpr_)
+        : q(g), L(L_), wpr(wpr_), at(static_cast<size_t>(g.ybase) * wpr_ + g.wA), row(g.ybase) {}
+    __device__ __forceinline__ void next() {
+        at += wpr;
+        if (!STRAIGHT && ++row == L) {
+            row = 0u;
+            at = q.wA;
+        }
+    }
+    __device__ __forceinline__ size_t a() const { return at; }
+    __device__ __forceinline__ size_t b() const { return STRAIGHT ? at + 1u : at - q.wA + q.wB; }
+};
+
 // Stage the lane's group: 16 rows of X and Y, funnel-shifted to local bit 0;
-// E: column 0 of the right neighbour (the halo column x0 + Bx for the last
-// lane column); D: row 0 of the lane below (the halo row y0 + By for the last
-// lane row).
-__device__ __forceinline__ void stage_lane(const LaneGeom &q, uint32_t L, uint32_t wpr, uint32_t Bx, uint32_t x0,
-                                           bool active, const LaneCtx &c, uint32_t (&X)[16], uint32_t (&Y)[16],
-                                           uint32_t &E, uint32_t &D) {
-    const uint32_t *const Xp = q.Xp;
-    const uint32_t *const Yp = q.Yp;
+// E: column 32 of its rows (column 0 of the right neighbour, or the sub-tile's
+// halo column); D: its row 16 of Y (row 0 of the lane below, or the halo row).
+template <bool STRAIGHT>
+__device__ __forceinline__ void load_lane_rows(const LaneGeom &q, uint32_t L, uint32_t wpr, uint32_t (&X)[16],
+                                               uint32_t (&Y)[16], uint32_t &E, uint32_t &D) {
+    LaneRows<STRAIGHT> w(q, L, wpr);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+        const uint32_t xb = q.Xp[w.b()];
+        X[r] = __funnelshift_r(q.Xp[w.a()], xb, q.sh);
+        Y[r] = __funnelshift_r(q.Yp[w.a()], q.Yp[w.b()], q.sh);
+        E |= ((xb >> q.sh) & 1u) << r;
+        w.next();
+    }
+    D = __funnelshift_r(q.Yp[w.a()], q.Yp[w.b()], q.sh);
+}
+
+__device__ __forceinline__ bool lane_straight(const LaneGeom &q, uint32_t L, bool active) {
+    return __all_sync(kFull, !active || (q.ybase + 17u <= L && q.wB == q.wA + 1u));
+}
+
+__device__ __forceinline__ void stage_lane(const LaneGeom &q, uint32_t L, uint32_t wpr, bool straight, bool active,
+                                           uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D) {
 #pragma unroll
     for (int r = 0; r < 16; ++r) {
         X[r] = 0u;
         Y[r] = 0u;
     }
+    E = 0u;
+    D = 0u;
     if (active) {
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            uint32_t yr = q.ybase + r;
-            if (yr >= L) yr -= L;
-            const size_t ro = static_cast<size_t>(yr) * wpr;
-            X[r] = __funnelshift_r(Xp[ro + q.wA], Xp[ro + q.wB], q.sh);
-            Y[r] = __funnelshift_r(Yp[ro + q.wA], Yp[ro + q.wB], q.sh);
-        }
-    }
-    uint32_t b0 = 0;
-#pragma unroll
-    for (int r = 0; r < 16; ++r) b0 |= (X[r] & 1u) << r;
-    E = __shfl_down_sync(kFull, b0, 1);
-    D = __shfl_down_sync(kFull, Y[0], c.GX);
-    if (active && c.gx == c.GX - 1) {  // halo column x0 + Bx
-        uint32_t xc = x0 + Bx;
-        if (xc >= L) xc -= L;
-        const uint32_t wc = xc >> 5, bc = xc & 31u;
-        E = 0u;
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            uint32_t yr = q.ybase + r;
-            if (yr >= L) yr -= L;
-            E |= ((Xp[static_cast<size_t>(yr) * wpr + wc] >> bc) & 1u) << r;
-        }
-    }
-    if (active && c.gy == c.GY - 1) {  // halo row y0 + By
-        const size_t ro = static_cast<size_t>(q.yh) * wpr;
-        D = __funnelshift_r(Yp[ro + q.wA], Yp[ro + q.wB], q.sh);
+        if (straight)
+            load_lane_rows<true>(q, L, wpr, X, Y, E, D);
+        else
+            load_lane_rows<false>(q, L, wpr, X, Y, E, D);
     }
 }
 
-template <bool LANE_SETS>
-__device__ __forceinline__ void write_back(const LaneGeom &q, uint32_t L, uint32_t wpr, bool active,
-                                           const LaneCtx &c, const uint32_t (&X)[16], const uint32_t (&Y)[16],
-                                           uint32_t E, uint32_t D) {
+// Write back.  Global word wA of a row receives the high bits of the left lane
+// and the low bits of this lane; the leftmost lane shares word wA with the
+// bits left of x0, the rightmost lane also owns the low bits of word wB (its
+// own high bits, and for X the halo-column bit).  The bits of those shared
+// words outside the sub-tile belong to neighbouring sub-tiles, which this
+// device step does not update, and no other warp writes these words (active
+// sub-tiles are at least 32 sites apart).  Full words are stored.  Shared words
+// are merged in one of two ways:
+//  * a warp holding one sub-tile (few shared words per lane): an AND/OR
+//    reduction pair, which returns nothing, so the warp does not wait;
+//  * a warp holding several small sub-tiles (many shared words per lane): a
+//    fresh read of the outside bits, all reads of eight rows before their
+//    stores (one wait for memory per eight rows), and one plain store per
+//    word; there the reductions' throughput would bind the step.
+template <bool LANE_SETS, bool STRAIGHT, class Ctx>
+__device__ __forceinline__ void store_lane_rows(const LaneGeom &q, uint32_t L, uint32_t wpr, bool active,
+                                                const Ctx &c, const uint32_t (&X)[16], const uint32_t (&Y)[16],
+                                                uint32_t E, uint32_t D) {
     uint32_t *const Xp = q.Xp;
     uint32_t *const Yp = q.Yp;
-    const uint32_t sh = q.sh, wA = q.wA, wB = q.wB, ybase = q.ybase, yh = q.yh;
-    // Write back.  Global word wA of a row receives the high bits of the left
-    // lane and the low bits of this lane; the leftmost lane shares word wA
-    // with the bits left of x0, the rightmost lane also owns the low bits of
-    // word wB (its own high bits, and for X the halo-column bit).  The bits of
-    // those shared words outside the sub-tile belong to neighbouring sub-tiles,
-    // which this device step does not update, and no other warp writes these
-    // words (active sub-tiles are at least 32 sites apart).  Full words are
-    // stored.  Shared words are merged in one of two ways:
-    //  * a warp holding one sub-tile (few shared words per lane): an AND/OR
-    //    reduction pair, which returns nothing, so the warp does not wait;
-    //  * a warp holding several small sub-tiles (many shared words per lane):
-    //    a fresh read of the outside bits, all reads of eight rows before
-    //    their stores (one wait for memory per eight rows), and one plain
-    //    store per word; there the reductions' throughput would bind the step.
+    const uint32_t sh = q.sh;
     const bool left_edge = active && c.gx == 0 && sh != 0u;
     const bool right_edge = active && c.gx == c.GX - 1;
     const uint32_t lo_mask = (1u << sh) - 1u;  // bits [0, sh): left of x0 in word wA
     const uint32_t xb_mask = (2u << sh) - 1u;  // bits [0, sh]: ours in word wB of X (halo bit at sh)
-    const bool by_read = LANE_SETS;
+    LaneRows<STRAIGHT> w(q, L, wpr);
 #pragma unroll
     for (int h = 0; h < 16; h += 8) {
         uint32_t oX[8], oY[8];  // outside bits of the lane's edge words (wA's in lo_mask, wB's above)
-        if (by_read) {
+        if (LANE_SETS) {
+            LaneRows<STRAIGHT> v = w;
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-                uint32_t yr = ybase + h + i;
-                if (yr >= L) yr -= L;
-                const size_t ro = static_cast<size_t>(yr) * wpr;
                 oX[i] = 0u;
                 oY[i] = 0u;
                 if (left_edge) {
-                    oX[i] = Xp[ro + wA] & lo_mask;
-                    oY[i] = Yp[ro + wA] & lo_mask;
+                    oX[i] = Xp[v.a()] & lo_mask;
+                    oY[i] = Yp[v.a()] & lo_mask;
                 }
                 if (right_edge) {
-                    oX[i] |= Xp[ro + wB] & ~xb_mask;
-                    oY[i] |= Yp[ro + wB] & ~lo_mask;
+                    oX[i] |= Xp[v.b()] & ~xb_mask;
+                    oY[i] |= Yp[v.b()] & ~lo_mask;
                 }
+                v.next();
             }
         }
 #pragma unroll
@@ -1032,61 +1093,70 @@ __device__ __forceinline__ void write_back(const LaneGeom &q, uint32_t L, uint32
             const uint32_t leftX = __shfl_up_sync(kFull, X[r], 1);
             const uint32_t leftY = __shfl_up_sync(kFull, Y[r], 1);
             if (active) {
-                uint32_t yr = ybase + r;
-                if (yr >= L) yr -= L;
-                const size_t ro = static_cast<size_t>(yr) * wpr;
+                const size_t A = w.a(), B = w.b();
                 if (left_edge) {
-                    if (by_read) {
-                        Xp[ro + wA] = (oX[i] & lo_mask) | (X[r] << sh);
-                        Yp[ro + wA] = (oY[i] & lo_mask) | (Y[r] << sh);
+                    if (LANE_SETS) {
+                        Xp[A] = (oX[i] & lo_mask) | (X[r] << sh);
+                        Yp[A] = (oY[i] & lo_mask) | (Y[r] << sh);
                     } else {
-                        reduce_bits(&Xp[ro + wA], X[r] << sh, ~lo_mask);
-                        reduce_bits(&Yp[ro + wA], Y[r] << sh, ~lo_mask);
+                        reduce_bits(&Xp[A], X[r] << sh, ~lo_mask);
+                        reduce_bits(&Yp[A], Y[r] << sh, ~lo_mask);
                     }
                 } else {
-                    Xp[ro + wA] = __funnelshift_l(leftX, X[r], sh);
-                    Yp[ro + wA] = __funnelshift_l(leftY, Y[r], sh);
+                    Xp[A] = __funnelshift_l(leftX, X[r], sh);
+                    Yp[A] = __funnelshift_l(leftY, Y[r], sh);
                 }
                 if (right_edge) {
                     const uint32_t hiX = (sh ? (X[r] >> (32u - sh)) : 0u) | (((E >> r) & 1u) << sh);
                     const uint32_t hiY = sh ? (Y[r] >> (32u - sh)) : 0u;
-                    if (by_read) {
-                        Xp[ro + wB] = (oX[i] & ~xb_mask) | hiX;
-                        if (sh) Yp[ro + wB] = (oY[i] & ~lo_mask) | hiY;
+                    if (LANE_SETS) {
+                        Xp[B] = (oX[i] & ~xb_mask) | hiX;
+                        if (sh) Yp[B] = (oY[i] & ~lo_mask) | hiY;
                     } else {
-                        reduce_bits(&Xp[ro + wB], hiX, xb_mask);
-                        if (sh) reduce_bits(&Yp[ro + wB], hiY, lo_mask);
+                        reduce_bits(&Xp[B], hiX, xb_mask);
+                        if (sh) reduce_bits(&Yp[B], hiY, lo_mask);
                     }
                 }
             }
+            w.next();
         }
     }
     {
-        const bool d_row = active && c.gy == c.GY - 1;
-        const size_t ro = static_cast<size_t>(yh) * wpr;
+        const bool d_row = active && c.gy == c.GY - 1;  // the halo row, below the sub-tile's last lanes
+        const size_t A = w.a(), B = w.b();
         uint32_t oD = 0u;
-        if (by_read && d_row) {
-            if (left_edge) oD = Yp[ro + wA] & lo_mask;
-            if (right_edge && sh) oD |= Yp[ro + wB] & ~lo_mask;
+        if (LANE_SETS && d_row) {
+            if (left_edge) oD = Yp[A] & lo_mask;
+            if (right_edge && sh) oD |= Yp[B] & ~lo_mask;
         }
         const uint32_t leftD = __shfl_up_sync(kFull, D, 1);
         if (d_row) {
             if (left_edge) {
-                if (by_read)
-                    Yp[ro + wA] = (oD & lo_mask) | (D << sh);
+                if (LANE_SETS)
+                    Yp[A] = (oD & lo_mask) | (D << sh);
                 else
-                    reduce_bits(&Yp[ro + wA], D << sh, ~lo_mask);
+                    reduce_bits(&Yp[A], D << sh, ~lo_mask);
             } else {
-                Yp[ro + wA] = __funnelshift_l(leftD, D, sh);
+                Yp[A] = __funnelshift_l(leftD, D, sh);
             }
             if (right_edge && sh) {
-                if (by_read)
-                    Yp[ro + wB] = (oD & ~lo_mask) | (D >> (32u - sh));
+                if (LANE_SETS)
+                    Yp[B] = (oD & ~lo_mask) | (D >> (32u - sh));
                 else
-                    reduce_bits(&Yp[ro + wB], D >> (32u - sh), lo_mask);
+                    reduce_bits(&Yp[B], D >> (32u - sh), lo_mask);
             }
         }
     }
+}
+
+template <bool LANE_SETS, class Ctx>
+__device__ __forceinline__ void write_back(const LaneGeom &q, uint32_t L, uint32_t wpr, bool straight, bool active,
+                                           const Ctx &c, const uint32_t (&X)[16], const uint32_t (&Y)[16],
+                                           uint32_t E, uint32_t D) {
+    if (straight)
+        store_lane_rows<LANE_SETS, true>(q, L, wpr, active, c, X, Y, E, D);
+    else
+        store_lane_rows<LANE_SETS, false>(q, L, wpr, active, c, X, Y, E, D);
 }
 
 // Device step on one sub-tile (Bx x By sites at (x0, y0)) held by the lanes of
@@ -1097,30 +1167,31 @@ __device__ __forceinline__ void write_back(const LaneGeom &q, uint32_t L, uint32
 // delayed borders, 3 DTrDTr, 4 DTrDT with deposition only (p = 1, q = 0),
 // 5 DTrDT with both rates strictly inside (0, 1), 6 DTrDB with deposition only,
 // 7 DTrDB with delayed borders and both rates random.
-template <bool RANDOM, bool LANE_SETS, int SCHEME = 0>
+template <bool RANDOM, bool LANE_SETS, int SCHEME = 0, class Ctx>
 __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t plane_rows, uint32_t wpr,
                                             uint32_t Bx, uint32_t By, uint32_t x0, uint32_t y0, bool active,
-                                            const LaneCtx &c, uint32_t *ring, int &net, int &draws,
+                                            const Ctx &c, uint32_t *ring, int &net, int &draws,
                                             int &tails) {
     TailPool tp;
     tp.ring = ring + static_cast<uint32_t>(kRingWordsPerLane) * c.g;  // the lane's own slot
     tp.head = 0u;
     tp.end = 0u;
     tp.rounds = 0u;
-    const LaneGeom q = lane_geom(lat, L, plane_rows, wpr, By, x0, y0, c);
+    const LaneGeom q = lane_geom(lat, L, plane_rows, wpr, x0, y0, c);
     uint32_t X[16], Y[16], E, D;
-    stage_lane(q, L, wpr, Bx, x0, active, c, X, Y, E, D);
+    const bool straight = lane_straight(q, L, active);
+    stage_lane(q, L, wpr, straight, active, X, Y, E, D);
 
     // Block layer: 16 single-hit collective steps.
-    const uint4 setw = philox4x32_10(c.t, c.k, c.T, kTagSet << 28, c.k0, c.k1);
+    const uint4 setw = c.draw(c.k, kTagSet << 28);
     uint4 site = make_uint4(0u, 0u, 0u, 0u);
     uint4 borg = make_uint4(0u, 0u, 0u, 0u);
-    if (SCHEME == 3) borg = philox4x32_10(c.t, c.k, c.T, kTagBorg << 28, c.k0, c.k1);
+    if (SCHEME == 3) borg = c.draw(c.k, kTagBorg << 28);
     for (uint32_t s = 0; s < 16u; ++s) {
         if (SCHEME == 3) {
             // DTrDTr: the set, plus a block-layer origin (ax, ay) per step
             if ((s & 1u) == 0u)
-                site = philox4x32_10(c.t, c.k | ((s >> 1) << 2), c.T, (kTagSite << 28) | c.g, c.k0, c.k1);
+                site = c.draw(c.k | ((s >> 1) << 2), (kTagSite << 28) | c.g);
             const uint32_t d = (setw.x >> (2u * s)) & 3u;
             const uint32_t bw = (s < 4u) ? borg.x : (s < 8u) ? borg.y : (s < 12u) ? borg.z : borg.w;
             const uint32_t byte = (bw >> (8u * (s & 3u))) & 0xFFu;
@@ -1140,7 +1211,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
         }
         if (SCHEME == 1 || SCHEME == 2 || SCHEME == 6 || SCHEME == 7) {
             // DB: one site word per TC row and step, 4 bits per cell
-            site = philox4x32_10(c.t, c.k | (s << 2), c.T, (kTagSiteDb << 28) | c.g, c.k0, c.k1);
+            site = c.draw(c.k | (s << 2), (kTagSiteDb << 28) | c.g);
             if (SCHEME == 2)
                 db_step_delayed<RANDOM>(X, Y, E, D, site, s, c, tp, net, draws);
             else if (SCHEME == 7)
@@ -1152,7 +1223,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             continue;
         }
         if ((s & 1u) == 0u)
-            site = philox4x32_10(c.t, c.k | ((s >> 1) << 2), c.T, (kTagSite << 28) | c.g, c.k0, c.k1);
+            site = c.draw(c.k | ((s >> 1) << 2), (kTagSite << 28) | c.g);
         else
             site = make_uint4(site.x >> 2, site.y >> 2, site.z >> 2, site.w >> 2);
         // the set (every lane of a one-sub-tile warp drew the same one; the broadcast
@@ -1188,7 +1259,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             step_apply<0, RANDOM, kSpec>(X, Y, E, D, d & 1u, acc, cnd0, cnd1, c, net);
     }
 
-    write_back<LANE_SETS>(q, L, wpr, active, c, X, Y, E, D);
+    write_back<LANE_SETS>(q, L, wpr, straight, active, c, X, Y, E, D);
     tails = static_cast<int>(tp.rounds);
 }
 
