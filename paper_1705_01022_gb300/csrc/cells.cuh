@@ -373,16 +373,4 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacke
     }
 }
 
-template <int CX, int CY>
-void launch_cells_shape(const StepArgs &a, bool any_random, const dim3 &grid, const dim3 &block, cudaStream_t st) {
-    if (!any_random && a.p_always == 0xFFFFFFFFu && a.q_always == 0u)
-        cells_step_kernel<CX, CY, false, 1><<<grid, block, 0, st>>>(a);  // deposition only (p = 1, q = 0)
-    else if (any_random && a.p_random && a.q_random)
-        cells_step_kernel<CX, CY, true, 2><<<grid, block, 0, st>>>(a);   // both rates inside (0, 1)
-    else if (any_random)
-        cells_step_kernel<CX, CY, true, 0><<<grid, block, 0, st>>>(a);
-    else
-        cells_step_kernel<CX, CY, false, 0><<<grid, block, 0, st>>>(a);
-}
-
 }  // namespace oct
