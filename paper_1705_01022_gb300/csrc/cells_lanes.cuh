@@ -397,7 +397,7 @@ cudaError_t launch_lane_cells(const StepArgs &a, const LaneSplit &q, cudaStream_
 // and the sub-tile; the bit-parallel one costs a step of a lane for 512 / (cx cy)
 // attempts, with GX * GY of 32 lanes at work.  One MCS at L=8192, p=0.95, q=0.05
 // (us, bit-parallel and lane per cell):
-//   256x64 sub-tiles (32 groups): 8x8 326, 585; 16x8 500, 629; 32x8 773, 634;
+//   256x64 sub-tiles (32 groups): 8x8 276, 585; 16x8 487, 629; 32x8 773, 634;
 //                                 16x16 906, 637; 32x16 1503, 744
 //   64x64 (8 groups):             8x4 504, 525; 16x4 716, 443; 8x8 847, 461;
 //                                 16x16 2332, 561; 32x16 3850, 780
