@@ -39,6 +39,7 @@ int cuda_fail(cudaError_t e, const char *what) {
 uint32_t threshold32(double p) { return static_cast<uint32_t>(std::floor(std::ldexp(p, 32))); }
 
 constexpr int kEventPairs = 256;
+constexpr int64_t kRunMcs = 1024;  // MCS of a small lattice in one launch (about 10 ms at most)
 
 }  // namespace
 
@@ -338,7 +339,17 @@ int oct_run_mcs(oct_sim *s, int64_t n) {
     if (n < 0) return fail(OCT_EINVAL, "n must be >= 0");
     if (s->t + static_cast<uint64_t>(n) > 0xFFFFFFFFull) return fail(OCT_EINVAL, "MCS counter would pass 2^32-1");
     OCT_CUDA(cudaSetDevice(s->device));
+    if (!s->timing && oct::rows_take(s->args) && oct::rows_fit_cluster(s->args)) {
+        // whole MCS in one launch (which advances the counter), at most kRunMcs each
+        s->args.dt = 0;
+        for (int64_t left = n; left > 0; left -= kRunMcs)
+            OCT_CUDA(oct::launch_row_run(s->args, s->any_random, s->d_t,
+                                         static_cast<uint32_t>(std::min<int64_t>(left, kRunMcs)), s->stream));
+        s->t += static_cast<uint64_t>(n);
+        return OCT_OK;
+    }
     for (int64_t i = 0; i < n; ++i) {
+        s->args.dt = static_cast<uint32_t>(i);
         for (uint32_t k = 0; k < 4; ++k) {
             s->args.k = k;
             if (s->timing) {
@@ -348,15 +359,16 @@ int oct_run_mcs(oct_sim *s, int64_t n) {
                 }
                 OCT_CUDA(cudaEventRecord(s->ev[2 * s->ev_used], s->stream));
             }
-            OCT_CUDA(oct::launch_dtrdt_step(s->args, s->any_random, s->stream));
+            // a step's head may overlap the tail of the step before it in this call
+            OCT_CUDA(oct::launch_dtrdt_step(s->args, s->any_random, !s->timing && (i > 0 || k > 0), s->stream));
             if (s->timing) {
                 OCT_CUDA(cudaEventRecord(s->ev[2 * s->ev_used + 1], s->stream));
                 ++s->ev_used;
                 ++s->step_launches;
             }
         }
-        OCT_CUDA(oct::launch_advance_t(s->d_t, s->stream));
     }
+    if (n > 0) OCT_CUDA(oct::launch_advance_t(s->d_t, static_cast<uint32_t>(n), s->stream));
     s->t += static_cast<uint64_t>(n);
     return OCT_OK;
 }
@@ -368,6 +380,7 @@ int oct_device_step(oct_sim *s, int k) {
     if (s->t >= 0xFFFFFFFFull) return fail(OCT_EINVAL, "MCS counter would pass 2^32-1");
     OCT_CUDA(cudaSetDevice(s->device));
     s->args.k = static_cast<uint32_t>(k);
+    s->args.dt = 0;
     if (s->timing) {
         if (s->ev_used == kEventPairs) {
             int rc = flush_timing(s);
@@ -375,7 +388,7 @@ int oct_device_step(oct_sim *s, int k) {
         }
         OCT_CUDA(cudaEventRecord(s->ev[2 * s->ev_used], s->stream));
     }
-    OCT_CUDA(oct::launch_dtrdt_step(s->args, s->any_random, s->stream));
+    OCT_CUDA(oct::launch_dtrdt_step(s->args, s->any_random, false, s->stream));
     if (s->timing) {
         OCT_CUDA(cudaEventRecord(s->ev[2 * s->ev_used + 1], s->stream));
         ++s->ev_used;
@@ -389,7 +402,7 @@ int oct_end_mcs(oct_sim *s) {
     if (!s) return fail(OCT_EINVAL, "NULL handle");
     if (s->next_k != 4) return fail(OCT_EINVAL, "oct_end_mcs needs device steps 0..3 first");
     OCT_CUDA(cudaSetDevice(s->device));
-    OCT_CUDA(oct::launch_advance_t(s->d_t, s->stream));
+    OCT_CUDA(oct::launch_advance_t(s->d_t, 1u, s->stream));
     s->t += 1;
     s->next_k = 0;
     return OCT_OK;

@@ -80,15 +80,13 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
         const uint32_t t = t_of[it.rep];  // this replica's MCS index
         const uint32_t L = R.L;
         const uint4 M = philox4x32_10(t, 0u, 0u, kTagMcs << 28, R.k0, R.k1);
-        const uint32_t ox = static_cast<uint32_t>((static_cast<uint64_t>(M.x) * L) >> 32);
-        const uint32_t oy = static_cast<uint32_t>((static_cast<uint64_t>(M.y) * L) >> 32);
-        const uint32_t pidx = static_cast<uint32_t>((static_cast<uint64_t>(M.z) * 24u) >> 32);
-        const int sigma = perm_element(pidx, k);
-        const uint32_t tx = it.T % R.tiles_x, ty = it.T / R.tiles_x;
-        const uint32_t x0 = static_cast<uint32_t>(
-            (static_cast<uint64_t>(ox) + 2ull * R.Bx * tx + static_cast<uint64_t>(R.Bx) * (sigma & 1)) % L);
-        const uint32_t y0 = static_cast<uint32_t>(
-            (static_cast<uint64_t>(oy) + 2ull * R.By * ty + static_cast<uint64_t>(R.By) * (sigma >> 1)) % L);
+        const uint32_t sigma = static_cast<uint32_t>(perm_element(__umulhi(M.z, 24u), k));
+        const uint32_t ty = it.T / R.tiles_x, tx = it.T - ty * R.tiles_x;
+        // (an offset plus a place lies below 2L)
+        uint32_t x0 = __umulhi(M.x, L) + R.Bx * (2u * tx + (sigma & 1u));
+        if (x0 >= L) x0 -= L;
+        uint32_t y0 = __umulhi(M.y, L) + R.By * (2u * ty + (sigma >> 1));
+        if (y0 >= L) y0 -= L;
         LaneCtx<KeysWeyl> c;
         c.GX = static_cast<int>(wd.GX);
         c.GY = G / c.GX;

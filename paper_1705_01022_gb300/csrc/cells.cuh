@@ -377,9 +377,9 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacke
     const uint32_t w = blockIdx.x * kStepWarpsPerBlock + (threadIdx.x >> 5);
     if (w >= work_tiles(a)) return;  // the whole warp leaves together
 
-    const uint32_t t = *a.t_ptr;
+    const uint32_t t = *a.t_ptr + a.dt;
     const uint32_t L = a.L;
-    const TilePlace pl = place_tile(a, w, t);
+    const TilePlace pl = place_tile(a, w, t, a.k);
     const uint32_t T = pl.T, x0 = pl.x0, y0 = pl.y0;
 
     CellCtx cc;

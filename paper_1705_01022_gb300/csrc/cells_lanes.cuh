@@ -201,8 +201,8 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
     const uint32_t gl = lane / C::GSZ, i = lane % C::GSZ, j = i >> 2, m = i & 3u;
     const uint32_t seg = q.pk > 1u ? gl / q.ngp : 0u;
     const uint32_t w = warp * q.pk + seg;
-    const uint32_t t = *a.t_ptr;
-    const TilePlace pl = place_tile(a, w < n_tiles ? w : 0u, t);
+    const uint32_t t = *a.t_ptr + a.dt;
+    const TilePlace pl = place_tile(a, w < n_tiles ? w : 0u, t, a.k);
     const uint32_t T = pl.T;
     uint32_t rb[C::NCMAX], db[C::NCMAX];  // half 0 of the next cell's row 0; row 0 of the cell below
     uint32_t on = 0u;                     // turns in which the lane holds a cell
@@ -397,7 +397,7 @@ cudaError_t launch_lane_cells(const StepArgs &a, const LaneSplit &q, cudaStream_
 // and the sub-tile; the bit-parallel one costs a step of a lane for 512 / (cx cy)
 // attempts, with GX * GY of 32 lanes at work.  One MCS at L=8192, p=0.95, q=0.05
 // (us, bit-parallel and lane per cell):
-//   256x64 sub-tiles (32 groups): 8x8 276, 585; 16x8 487, 629; 32x8 773, 634;
+//   256x64 sub-tiles (32 groups): 8x8 281, 585; 16x8 487, 629; 32x8 773, 634;
 //                                 16x16 906, 637; 32x16 1503, 744
 //   64x64 (8 groups):             8x4 504, 525; 16x4 716, 443; 8x8 847, 461;
 //                                 16x16 2332, 561; 32x16 3850, 780

@@ -40,6 +40,7 @@
 
 #include "oct_internal.h"
 
+#include "overlap.cuh"
 #include "subtile.cuh"
 #include "tiles.cuh"
 
@@ -79,10 +80,10 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     const uint32_t seg = static_cast<uint32_t>(lane) / S, sub = static_cast<uint32_t>(lane) % S;
     const uint32_t w = warp_id * per_warp + seg;  // work index of the lane's sub-tile
 
-    const uint32_t t = *a.t_ptr;
+    const uint32_t t = *a.t_ptr + a.dt;
     const uint32_t L = a.L;
     // Device layer: origin and set order of this MCS (same for every warp).
-    const TilePlace pl = place_tile(a, w < n_tiles ? w : 0u, t);
+    const TilePlace pl = place_tile(a, w < n_tiles ? w : 0u, t, a.k);
     const uint32_t T = pl.T, x0 = pl.x0, y0 = pl.y0;
 
     // Deposition only draws one block per two steps: there the key additions are
@@ -136,31 +137,33 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     }
 }
 
-__global__ void advance_t_kernel(uint32_t *t_ptr) { *t_ptr += 1u; }
+__global__ void advance_t_kernel(uint32_t *t_ptr, uint32_t n) { *t_ptr += n; }
 
 }  // namespace
 
-cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t st) {
+cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, cudaStream_t st) {
     if (a.cx != 4u || a.cy != 4u) return launch_cells_step(a, any_random, st);
+    if (rows_take(a)) return launch_row_step(a, any_random, overlap, st);
     const uint32_t n_tiles = work_tiles(a);
     const uint32_t S = segment_lanes(a.GX * a.GY);
     const bool packed = S < 32u;
     const uint32_t per_block = kStepWarpsPerBlock * (packed ? 32u / S : 1u);
     const uint32_t blocks = (n_tiles + per_block - 1) / per_block;
     const dim3 grid(blocks), block(kStepWarpsPerBlock * 32);
+    cudaError_t e = cudaSuccess;
 #define OCT_LAUNCH(SCHEME, PACKED)                                                   \
     do {                                                                             \
         if (any_random)                                                              \
-            dtrdt_step_kernel<true, SCHEME, PACKED><<<grid, block, 0, st>>>(a);      \
+            e = launch_overlapped(dtrdt_step_kernel<true, SCHEME, PACKED>, grid, block, overlap, st, a);      \
         else                                                                         \
-            dtrdt_step_kernel<false, SCHEME, PACKED><<<grid, block, 0, st>>>(a);     \
+            e = launch_overlapped(dtrdt_step_kernel<false, SCHEME, PACKED>, grid, block, overlap, st, a);     \
     } while (0)
     switch (a.scheme) {
         case 1:
             if (packed)
                 OCT_LAUNCH(1, true);
             else if (!any_random && a.p_always == 0xFFFFFFFFu && a.q_always == 0u)
-                dtrdt_step_kernel<false, 6, false><<<grid, block, 0, st>>>(a);  // deposition only
+                e = launch_overlapped(dtrdt_step_kernel<false, 6, false>, grid, block, overlap, st, a);  // deposition only
             else
                 OCT_LAUNCH(1, false);
             break;
@@ -168,7 +171,7 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t s
             if (packed)
                 OCT_LAUNCH(2, true);
             else if (a.p_random && a.q_random)
-                dtrdt_step_kernel<true, 7, false><<<grid, block, 0, st>>>(a);  // both rates random
+                e = launch_overlapped(dtrdt_step_kernel<true, 7, false>, grid, block, overlap, st, a);  // both rates random
             else
                 OCT_LAUNCH(2, false);
             break;
@@ -185,15 +188,15 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t s
             if (!any_random && a.p_always == 0xFFFFFFFFu && a.q_always == 0u) {
                 // deposition only (the KPZ case p = 1, q = 0): no acceptance masks
                 if (packed)
-                    dtrdt_step_kernel<false, 4, true><<<grid, block, 0, st>>>(a);
+                    e = launch_overlapped(dtrdt_step_kernel<false, 4, true>, grid, block, overlap, st, a);
                 else
-                    dtrdt_step_kernel<false, 4, false><<<grid, block, 0, st>>>(a);
+                    e = launch_overlapped(dtrdt_step_kernel<false, 4, false>, grid, block, overlap, st, a);
             } else if (any_random && a.p_random && a.q_random) {
                 // both rates strictly inside (0, 1): every candidate is decided by its draw
                 if (packed)
-                    dtrdt_step_kernel<true, 5, true><<<grid, block, 0, st>>>(a);
+                    e = launch_overlapped(dtrdt_step_kernel<true, 5, true>, grid, block, overlap, st, a);
                 else
-                    dtrdt_step_kernel<true, 5, false><<<grid, block, 0, st>>>(a);
+                    e = launch_overlapped(dtrdt_step_kernel<true, 5, false>, grid, block, overlap, st, a);
             } else if (packed) {
                 OCT_LAUNCH(0, true);
             } else {
@@ -201,11 +204,11 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t s
             }
     }
 #undef OCT_LAUNCH
-    return cudaGetLastError();
+    return e;
 }
 
-cudaError_t launch_advance_t(uint32_t *t_ptr, cudaStream_t st) {
-    advance_t_kernel<<<1, 1, 0, st>>>(t_ptr);
+cudaError_t launch_advance_t(uint32_t *t_ptr, uint32_t n, cudaStream_t st) {
+    advance_t_kernel<<<1, 1, 0, st>>>(t_ptr, n);
     return cudaGetLastError();
 }
 

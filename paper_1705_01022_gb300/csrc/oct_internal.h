@@ -23,6 +23,7 @@ struct StepArgs {
     uint32_t p_always, q_always;   // all-ones if p == 1 (resp. q == 1), else 0
     uint32_t p_random, q_random;   // all-ones if 0 < p < 1 (resp. q), else 0
     const uint32_t *t_ptr;     // device-resident MCS counter
+    uint32_t dt;               // MCS since *t_ptr: a run advances the counter once, at its end
     uint32_t k;                // device step 0..3
     unsigned long long *net;   // kNetSlots signed flip counters (two's complement)
     unsigned long long *draws; // kNetSlots counters of attempts that needed an acceptance draw
@@ -40,16 +41,26 @@ constexpr int kStepWarpsPerBlock = 4;
 constexpr int kStepBlocksPerSM = 5;  // occupancy target: 20 warps per SM
 constexpr int kStepBlocksPerSMPacked = 4;  // several sub-tiles per warp: per-lane row offsets need more registers
 
-// Launches one device step; returns the CUDA launch status.
-cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, cudaStream_t st);
+// Launches one device step; returns the CUDA launch status.  overlap: its head
+// may run during the tail of the kernel before it in the stream, which must be
+// the device step before it of the same run.
+cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, cudaStream_t st);
+
+// The device step with one TC row per lane (rowlanes.cu), for lattices too small
+// to fill the chip: whether it takes a step, one step, and n MCS in one launch
+// for lattices that fit a cluster.
+bool rows_take(const StepArgs &a);
+bool rows_fit_cluster(const StepArgs &a);
+cudaError_t launch_row_step(const StepArgs &a, bool any_random, bool overlap, cudaStream_t st);
+cudaError_t launch_row_run(const StepArgs &a, bool any_random, uint32_t *t_out, uint32_t n, cudaStream_t st);
 
 // DTrDT thread cells other than 4 x 4 sites (cells.cu): whether a cell shape
 // has a kernel, and the launch of one device step with it.
 bool cells_shape_supported(int cx, int cy);
 cudaError_t launch_cells_step(const StepArgs &a, bool any_random, cudaStream_t st);
 
-// Adds one to the device MCS counter.
-cudaError_t launch_advance_t(uint32_t *t_ptr, cudaStream_t st);
+// Adds n to the device MCS counter.
+cudaError_t launch_advance_t(uint32_t *t_ptr, uint32_t n, cudaStream_t st);
 
 // Flat start h = (x+y) mod 2 on the planar lattice (or on `rows` rows from an
 // even lattice row on, bit planes of `rows` rows each).

@@ -8,6 +8,7 @@
 #include <cstdint>
 
 #include "oct_internal.h"
+#include "overlap.cuh"
 #include "philox.cuh"
 
 namespace oct {
@@ -15,21 +16,17 @@ namespace oct {
 constexpr uint32_t kFull = 0xFFFFFFFFu;
 constexpr uint32_t kNib = 0x11111111u;  // bit 0 of every 4-bit TC column
 
-// Element k of the idx-th permutation of (0,1,2,3) in lexicographic order.
+// Element k of the idx-th permutation of (0,1,2,3) in lexicographic order: the
+// first one is idx / 6, the others are the (idx % 6)-th permutation of the
+// three that are left, in order.
 __device__ __forceinline__ int perm_element(uint32_t idx, uint32_t k) {
-    uint32_t remaining = 0x3210u;  // nibbles: the symbols not used yet, in order
-    uint32_t radix = 6u;            // (3 - i)!
-    int e = 0;
-    for (uint32_t i = 0; i <= k; ++i) {
-        const uint32_t pick = idx / radix;
-        idx -= pick * radix;
-        e = static_cast<int>((remaining >> (4u * pick)) & 0xFu);
-        const uint32_t low = remaining & ((1u << (4u * pick)) - 1u);
-        const uint32_t high = remaining >> (4u * (pick + 1u));
-        remaining = low | (high << (4u * pick));
-        radix = (i == 0) ? 2u : 1u;
-    }
-    return e;
+    // two bits per element: 012 021 102 120 201 210
+    constexpr uint64_t kPerm3 = (0x24ull << 0) | (0x18ull << 6) | (0x21ull << 12) | (0x09ull << 18) | (0x12ull << 24) |
+                                (0x06ull << 30);
+    const uint32_t first = idx / 6u, r = idx - 6u * first;
+    if (k == 0u) return static_cast<int>(first);
+    const uint32_t e = static_cast<uint32_t>(kPerm3 >> (6u * r + 2u * (k - 1u))) & 3u;
+    return static_cast<int>(e + (e >= first ? 1u : 0u));
 }
 
 // Sets the bits of *w selected by mask to those of v, leaving the others, as
@@ -1179,6 +1176,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
     tp.rounds = 0u;
     const LaneGeom q = lane_geom(lat, L, plane_rows, wpr, x0, y0, c);
     uint32_t X[16], Y[16], E, D;
+    wait_for_previous_grid();  // nothing above reads the lattice
     const bool straight = lane_straight(q, L, active);
     stage_lane(q, L, wpr, straight, active, X, Y, E, D);
 
@@ -1259,6 +1257,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             step_apply<0, RANDOM, kSpec>(X, Y, E, D, d & 1u, acc, cnd0, cnd1, c, net);
     }
 
+    launch_dependents();  // the next step's head overlaps this one's write-back
     write_back<LANE_SETS>(q, L, wpr, straight, active, c, X, Y, E, D);
     tails = static_cast<int>(tp.rounds);
 }

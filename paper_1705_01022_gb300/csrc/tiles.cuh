@@ -27,14 +27,14 @@ __host__ __device__ __forceinline__ uint32_t work_tiles(const StepArgs &a) {
     return a.tiles_x * (a.strip_tiles_y ? a.strip_tiles_y : a.tiles_y);
 }
 
-__device__ __forceinline__ TilePlace place_tile(const StepArgs &a, uint32_t w, uint32_t t) {
+// Work index w in device step k of MCS t.  Sums of an offset and a place stay
+// below 2L, so they are folded into [0, L) by one subtraction.
+__device__ __forceinline__ TilePlace place_tile(const StepArgs &a, uint32_t w, uint32_t t, uint32_t k) {
     const uint32_t L = a.L;
     const uint4 M = philox4x32_10(t, 0u, 0u, kTagMcs << 28, a.k0, a.k1);
-    const uint32_t ox = static_cast<uint32_t>((static_cast<uint64_t>(M.x) * L) >> 32);
-    const uint32_t oy = static_cast<uint32_t>((static_cast<uint64_t>(M.y) * L) >> 32);
-    const uint32_t pidx = static_cast<uint32_t>((static_cast<uint64_t>(M.z) * 24u) >> 32);
-    const int sigma = perm_element(pidx, a.k);
-    const uint32_t tx = w % a.tiles_x, j = w / a.tiles_x;
+    const uint32_t ox = __umulhi(M.x, L), oy = __umulhi(M.y, L);
+    const uint32_t sigma = static_cast<uint32_t>(perm_element(__umulhi(M.z, 24u), k));
+    const uint32_t j = w / a.tiles_x, tx = w - j * a.tiles_x;
     uint32_t ty = j;
     if (a.strip_tiles_y) {
         // tile rows whose first row lies in the strip: ty = (j - q) mod tiles_y,
@@ -45,11 +45,11 @@ __device__ __forceinline__ TilePlace place_tile(const StepArgs &a, uint32_t w, u
     }
     TilePlace p;
     p.T = ty * a.tiles_x + tx;
-    p.x0 = static_cast<uint32_t>(
-        (static_cast<uint64_t>(ox) + 2ull * a.Bx * tx + static_cast<uint64_t>(a.Bx) * (sigma & 1)) % L);
-    const uint32_t yg = static_cast<uint32_t>(
-        (static_cast<uint64_t>(oy) + 2ull * a.By * ty + static_cast<uint64_t>(a.By) * (sigma >> 1)) % L);
-    p.y0 = (yg + L - a.row0) % L;
+    p.x0 = ox + a.Bx * (2u * tx + (sigma & 1u));
+    if (p.x0 >= L) p.x0 -= L;
+    p.y0 = oy + a.By * (2u * ty + (sigma >> 1));
+    if (p.y0 >= L) p.y0 -= L;
+    p.y0 += p.y0 >= a.row0 ? 0u - a.row0 : L - a.row0;  // buffer row
     return p;
 }
 
