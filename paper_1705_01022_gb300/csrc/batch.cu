@@ -14,7 +14,8 @@
 // sub-tiles of 32 groups fill a warp alone and take the uniform path.  All
 // replicas advance in lock step: one MCS is four device steps, each one launch
 // per acceptance mode and warp kind, captured once in a CUDA graph and
-// replayed.
+// replayed.  A batch too small to fill the chip takes one launch per device step
+// for all modes, with a TC row per lane (batch_row_kernel).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -27,6 +28,8 @@
 
 #include "../../include/oct.h"
 #include "oct_internal.h"
+#include "overlap.cuh"
+#include "rowlanes.cuh"
 #include "subtile.cuh"
 
 namespace oct {
@@ -50,6 +53,7 @@ struct WarpDesc {
     uint32_t n;      // items in this warp (32 / G at most)
     uint32_t G;      // lanes per item
     uint32_t GX;     // lane columns per item
+    uint32_t kpz;    // row lanes: every item's replica is deposition only (p = 1, q = 0)
 };
 
 constexpr int kBatchWarps = 4;
@@ -123,10 +127,90 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
     }
 }
 
-// Advances the MCS counter of every active replica.
-__global__ void batch_advance_kernel(uint32_t *t_of, const uint32_t *active, uint32_t n_active) {
+// A batch too small to fill the chip: one device step of every replica in one
+// launch, a TC row per lane (rowlanes.cuh), a descriptor per warp.  All modes
+// share the launch (two forms of the step: deposition only, and the general
+// one), so that no replica waits for another's kernel, and there is no graph to
+// capture after every membership change.  Latency bound like rowlanes.cuh: 16
+// MCS and the W^2 of 64 replicas of L = 64..512 go from 2.0 ms with the graph to
+// 0.74 ms; at kRowWarpsMax both are level (24 replicas of L=2048, 6144 warps: 2.44
+// ms with the graph).
+template <bool RANDOM, int SPEC, bool ONE>
+__device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDesc &wd, uint32_t T, bool held, uint32_t t,
+                                               uint32_t k, uint32_t *sm) {
+    const uint32_t lane = threadIdx.x & 31u, S = ONE ? 32u : wd.G, seg = lane / S, sub = lane % S;
+    const uint32_t L = R.L;
+    const uint4 M = philox4x32_10(t, 0u, 0u, kTagMcs << 28, R.k0, R.k1);
+    const uint32_t sigma = static_cast<uint32_t>(perm_element(__umulhi(M.z, 24u), k));
+    const uint32_t ty = T / R.tiles_x, tx = T - ty * R.tiles_x;
+    uint32_t x0 = __umulhi(M.x, L) + R.Bx * (2u * tx + (sigma & 1u));
+    if (x0 >= L) x0 -= L;
+    uint32_t y0 = __umulhi(M.y, L) + R.By * (2u * ty + (sigma >> 1));
+    if (y0 >= L) y0 -= L;
+    RowLane rl;
+    rl.GX = static_cast<int>(wd.GX);
+    rl.TR = static_cast<int>(R.By / 4u);
+    rl.gx = static_cast<int>(sub % wd.GX);
+    rl.tr = static_cast<int>(sub / wd.GX);
+    rl.m = static_cast<uint32_t>(rl.tr) & 3u;
+    rl.active = held;
+    LaneCtx<KeysWeyl> c;
+    c.t = t;
+    c.k = k;
+    c.T = T;
+    c.g = (static_cast<uint32_t>(rl.tr) >> 2) * wd.GX + static_cast<uint32_t>(rl.gx);
+    rl.gw = seg * (S / 4u) + c.g;
+    c.key = KeysWeyl{R.k0, R.k1};
+    c.first_round();
+    c.thr_p = R.thr_p;
+    c.thr_q = R.thr_q;
+    c.p_always = R.p_always;
+    c.q_always = R.q_always;
+    c.p_random = R.p_random;
+    c.q_random = R.q_random;
+    int net = 0, draws = 0, tails = 0;
+    run_rows<RANDOM, SPEC, ONE, false>(R.lat, L, L, R.wpr, x0, y0, c, rl, sm, net, draws, tails,
+                                       [] { wait_for_previous_grid(); }, [] { launch_dependents(); });
+    for (uint32_t o = S >> 1; o > 0; o >>= 1) {
+        net += __shfl_xor_sync(kFull, net, o);
+        if (RANDOM) draws += __shfl_xor_sync(kFull, draws, o);
+    }
+    if (held && sub == 0) {
+        if (net != 0) atomicAdd(&R.counters[0], static_cast<unsigned long long>(static_cast<long long>(net)));
+        if (RANDOM && draws != 0) atomicAdd(&R.counters[1], static_cast<unsigned long long>(draws));
+    }
+}
+
+__global__ void __launch_bounds__(kBatchWarps * 32)
+    batch_row_kernel(const ReplicaDev *reps, const BatchItem *items, const WarpDesc *descs, uint32_t n_descs,
+                     const uint32_t *t_of, uint32_t dt, uint32_t k) {
+    __shared__ __align__(16) uint32_t smem[kBatchWarps * row_smem_words<true>()];
+    const uint32_t di = blockIdx.x * kBatchWarps + (threadIdx.x >> 5);
+    if (di >= n_descs) return;  // the whole warp leaves together
+    const WarpDesc wd = descs[di];
+    const uint32_t slot = (threadIdx.x & 31u) / wd.G;
+    const bool held = slot < wd.n;
+    const BatchItem it = items[wd.first + (held ? slot : 0u)];
+    const ReplicaDev R = reps[it.rep];
+    const uint32_t t = t_of[it.rep] + dt;
+    uint32_t *const sm = smem + (threadIdx.x >> 5) * row_smem_words<true>();
+    if (wd.G == 32u) {
+        if (wd.kpz)
+            batch_row_item<false, 1, true>(R, wd, it.T, held, t, k, sm);
+        else
+            batch_row_item<true, 0, true>(R, wd, it.T, held, t, k, sm);
+    } else {
+        if (wd.kpz)
+            batch_row_item<false, 1, false>(R, wd, it.T, held, t, k, sm);
+        else
+            batch_row_item<true, 0, false>(R, wd, it.T, held, t, k, sm);
+    }
+}
+
+// Adds n to the MCS counter of every active replica.
+__global__ void batch_advance_kernel(uint32_t *t_of, const uint32_t *active, uint32_t n_active, uint32_t n) {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_active; i += gridDim.x * blockDim.x)
-        t_of[active[i]] += 1u;
+        t_of[active[i]] += n;
 }
 
 }  // namespace
@@ -222,6 +306,7 @@ struct oct_batch {
     // the active replicas ordered by branch: act_n[br] of them from act_first[br]
     uint32_t act_first[kBranches] = {};
     uint32_t act_n[kBranches] = {};
+    uint32_t row_descs = 0;       // warps of a device step in row lanes; 0: the branches below carry the batch
     uint32_t *d_queue = nullptr;  // 4 * kBranches counters: (device step, branch)
     oct::W2RowSums *d_rows = nullptr;
     int64_t rows_cap = 0;
@@ -406,6 +491,41 @@ cudaError_t grow_slots(oct_batch *b, size_t need) {
     return cudaSuccess;
 }
 
+// The batch in row lanes, if every sub-tile fits a warp that way and a device
+// step has at most kRowWarpsMax warps: items of one form and lane layout
+// packed into descriptors.  Leaves the lists empty otherwise.
+void row_lists(const std::vector<oct::ReplicaDev> &rd, const std::vector<uint32_t> &active,
+               std::vector<oct::BatchItem> &items, std::vector<oct::WarpDesc> &descs) {
+    uint64_t lanes = 0;
+    for (uint32_t slot : active) {
+        const oct::ReplicaDev &D = rd[slot];
+        if (D.GX * (D.By / 4u) > 32u) return;
+        lanes += static_cast<uint64_t>(D.tiles_x) * D.tiles_y * oct::row_segment(D.GX, D.By);
+    }
+    if (lanes > 32ull * oct::kRowWarpsMax) return;
+    std::vector<oct::BatchItem> bucket[2][6][6];  // form, log2 of GX, of the lanes per sub-tile
+    for (uint32_t slot : active) {
+        const oct::ReplicaDev &D = rd[slot];
+        int gi = 0, si = 0;
+        while ((1u << gi) < D.GX) ++gi;
+        while ((1u << si) < oct::row_segment(D.GX, D.By)) ++si;
+        const bool kpz = D.p_always && !D.q_always && !D.q_random;
+        auto &bk = bucket[kpz ? 1 : 0][gi][si];
+        for (uint32_t T = 0; T < D.tiles_x * D.tiles_y; ++T) bk.push_back({slot, T});
+    }
+    for (uint32_t kpz = 0; kpz < 2u; ++kpz)
+        for (uint32_t gi = 0; gi < 6u; ++gi)
+            for (uint32_t si = 0; si < 6u; ++si) {
+                const auto &bk = bucket[kpz][gi][si];
+                const size_t per = 32u >> si;
+                for (size_t i = 0; i < bk.size(); i += per) {
+                    const uint32_t n = static_cast<uint32_t>(std::min<size_t>(per, bk.size() - i));
+                    descs.push_back({static_cast<uint32_t>(items.size()), n, 1u << si, 1u << gi, kpz});
+                    items.insert(items.end(), bk.begin() + i, bk.begin() + i + n);
+                }
+            }
+}
+
 // Rebuilds the replica table and the warp work list of the active replicas
 // into the work-list copy the enqueued work does not read, by asynchronous
 // copies on the batch's stream (the host waits only for the staging memory of
@@ -445,10 +565,16 @@ cudaError_t rebuild(oct_batch *b) {
     std::vector<uint32_t> active;
     std::vector<oct::BatchItem> items;
     std::vector<oct::WarpDesc> descs;
+    for (int br = 0; br < kBranches; ++br) active.insert(active.end(), by_branch[br].begin(), by_branch[br].end());
+    row_lists(rd, active, items, descs);
+    b->row_descs = static_cast<uint32_t>(descs.size());
+    active.clear();
     for (int br = 0; br < kBranches; ++br) {
         b->act_first[br] = static_cast<uint32_t>(active.size());
         b->act_n[br] = static_cast<uint32_t>(by_branch[br].size());
         active.insert(active.end(), by_branch[br].begin(), by_branch[br].end());
+        b->n_desc[br] = 0;
+        if (b->row_descs) continue;
         // the branch's items bucketed by lane layout, then packed into warps
         std::vector<oct::BatchItem> bucket[6][6];
         for (uint32_t slot : by_branch[br]) {
@@ -471,6 +597,7 @@ cudaError_t rebuild(oct_batch *b) {
                     d.n = static_cast<uint32_t>(std::min<size_t>(per, bk.size() - i));
                     d.G = G;
                     d.GX = GX;
+                    d.kpz = 0;
                     for (uint32_t j = 0; j < d.n; ++j) items.push_back(bk[i + j]);
                     descs.push_back(d);
                 }
@@ -550,8 +677,18 @@ cudaError_t enqueue_branch_step(oct_batch *b, uint32_t k, int br, cudaStream_t s
     return cudaGetLastError();
 }
 
+// Enqueues device step k, dt MCS past the counters, of a batch in row lanes.
+// overlap: its head may run during the tail of the step enqueued before it.
+cudaError_t enqueue_row_step(oct_batch *b, uint32_t dt, uint32_t k, bool overlap, cudaStream_t st) {
+    const oct::WorkBuf &w = b->wb[b->cur];
+    const dim3 grid((b->row_descs + oct::kBatchWarps - 1) / oct::kBatchWarps), block(oct::kBatchWarps * 32);
+    return oct::launch_overlapped(oct::batch_row_kernel, grid, block, overlap, st, w.reps, w.items, w.descs,
+                                  b->row_descs, b->d_t, dt, k);
+}
+
 // Enqueues device step k of the current MCS of every active replica, branch by branch.
 cudaError_t enqueue_step(oct_batch *b, uint32_t k, cudaStream_t st) {
+    if (b->row_descs) return enqueue_row_step(b, 0, k, false, st);
     for (int br = 0; br < kBranches; ++br) {
         if (b->n_desc[br] == 0) continue;
         cudaError_t e = enqueue_branch_step(b, k, br, st);
@@ -560,10 +697,10 @@ cudaError_t enqueue_step(oct_batch *b, uint32_t k, cudaStream_t st) {
     return cudaSuccess;
 }
 
-cudaError_t enqueue_advance(oct_batch *b, cudaStream_t st) {
+cudaError_t enqueue_advance(oct_batch *b, uint32_t n, cudaStream_t st) {
     if (b->n_active == 0) return cudaSuccess;
     const int blocks = static_cast<int>(std::min<uint32_t>(1024u, (b->n_active + 255u) / 256u));
-    oct::batch_advance_kernel<<<blocks, 256, 0, st>>>(b->d_t, b->wb[b->cur].active, b->n_active);
+    oct::batch_advance_kernel<<<blocks, 256, 0, st>>>(b->d_t, b->wb[b->cur].active, b->n_active, n);
     return cudaGetLastError();
 }
 
@@ -572,7 +709,7 @@ cudaError_t enqueue_advance_branch(oct_batch *b, int br, cudaStream_t st) {
     const uint32_t n = b->act_n[br];
     if (n == 0) return cudaSuccess;
     const int blocks = static_cast<int>(std::min<uint32_t>(1024u, (n + 255u) / 256u));
-    oct::batch_advance_kernel<<<blocks, 256, 0, st>>>(b->d_t, b->wb[b->cur].active + b->act_first[br], n);
+    oct::batch_advance_kernel<<<blocks, 256, 0, st>>>(b->d_t, b->wb[b->cur].active + b->act_first[br], n, 1u);
     return cudaGetLastError();
 }
 
@@ -950,7 +1087,18 @@ int oct_batch_run(oct_batch *b, int64_t n) {
                 ++b->ev_used;
                 ++b->step_launches;
             }
-            BATCH_CUDA(enqueue_advance(b, b->stream));
+            BATCH_CUDA(enqueue_advance(b, 1u, b->stream));
+        }
+    } else if (b->row_descs) {
+        // launch by launch, each overlapping the one before; the counters advance
+        // at the end (2^16 MCS at a time, far inside their range)
+        for (int64_t done = 0; done < n;) {
+            const uint32_t part = static_cast<uint32_t>(std::min<int64_t>(n - done, 1 << 16));
+            for (uint32_t i = 0; i < part; ++i)
+                for (uint32_t k = 0; k < 4; ++k)
+                    BATCH_CUDA(enqueue_row_step(b, i, k, i > 0 || k > 0, b->stream));
+            BATCH_CUDA(enqueue_advance(b, part, b->stream));
+            done += part;
         }
     } else {
         // kGraphMcs MCS per graph launch while that many are left, then one

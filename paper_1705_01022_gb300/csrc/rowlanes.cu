@@ -22,21 +22,9 @@ constexpr uint32_t kClusterWarpsPerCta = 8;
 constexpr uint32_t kClusterWarps = kClusterCtas * kClusterWarpsPerCta;
 constexpr uint32_t kBlockWarps = 8;               // of a lattice in one block
 constexpr uint32_t kBlockLattice = 64u * 1024u;  // bytes of its lattice at most (L = 512)
-// Device steps of more warps than this keep the chip busy either way, and then
-// the lane of four TC rows needs fewer instructions per attempt (64 x 64
-// sub-tiles, us per MCS here and there: p=q=0.5, L=4096 47, 81; p=0.95, q=0.05,
-// L=8192 86, 107; L=16384 292, 262).
-constexpr uint32_t kRowWarpsMax = 152u * 32u;
 
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
-
-// Lanes of a sub-tile, rounded up to a power of two.
-__host__ __device__ inline uint32_t row_segment(uint32_t GX, uint32_t By) {
-    uint32_t s = 1u;
-    while (s < GX * (By / 4u)) s <<= 1;
-    return s;
-}
 
 template <bool RANDOM, int SPEC, bool ONE, bool SHARED = false, class Ready, class Done>
 __device__ __forceinline__ void row_step(const StepArgs &a, uint32_t *lat, uint32_t warp, uint32_t t, uint32_t k, uint32_t *sm,

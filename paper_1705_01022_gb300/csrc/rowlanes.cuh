@@ -41,6 +41,19 @@ struct RowLane {
     bool active;
 };
 
+// Lanes of a sub-tile, rounded up to a power of two.
+__host__ __device__ inline uint32_t row_segment(uint32_t GX, uint32_t By) {
+    uint32_t s = 1u;
+    while (s < GX * (By / 4u)) s <<= 1;
+    return s;
+}
+
+// Device steps of more warps than this keep the chip busy either way, and then
+// the lane of four TC rows needs fewer instructions per attempt (64 x 64
+// sub-tiles, us per MCS here and there: p=q=0.5, L=4096 47, 81; p=0.95, q=0.05,
+// L=8192 86, 107; L=16384 292, 262).
+constexpr uint32_t kRowWarpsMax = 152u * 32u;
+
 // ONE: one sub-tile per warp (the set is warp-uniform); otherwise the rows of
 // the set are picked per lane with selects.  `ready` waits for the device step
 // before this one; everything ahead of it does not read the lattice.  `done` is
