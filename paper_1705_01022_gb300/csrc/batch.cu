@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
 // share the launch (two forms of the step: deposition only, and the general
 // one), so that no replica waits for another's kernel, and there is no graph to
 // capture after every membership change.  Latency bound like rowlanes.cuh: 16
-// MCS and the W^2 of 64 replicas of L = 64..512 go from 2.0 ms with the graph to
+// MCS and the W^2 of 64 replicas of L = 64..512 take
 // 0.74 ms; at kRowWarpsMax both are level (24 replicas of L=2048, 6144 warps: 2.44
 // ms with the graph).
 template <bool RANDOM, int SPEC, bool ONE>

@@ -5,11 +5,11 @@
 // sites bit-parallel (cells.cuh) tests all eight rows that an attempt can fall
 // on for the sake of its 512 / (cx cy) attempts: two for 16 x 16 cells.  Here
 // the sub-tile lies in shared memory and a lane makes one attempt at a time,
-// three loads and up to three stores of it, whatever the cell: 171 instructions
-// per 32 attempts with acceptance draws (16 x 16 cells, 64 x 64 sub-tiles; bound
-// by instruction issue and their fixed latency, 2.3 per clock), against about
-// 600 per two attempts of each lane.  One MCS at L=8192 with them: 2.31 ms to
-// 0.56 ms.  A warp takes the cells of a sub-tile in turns of 32 (NC of them), or
+// three loads and up to three stores of it, whatever the cell.  Bound by
+// instruction issue and fixed latency (16 x 16 cells in 64 x 64 sub-tiles, p=0.95,
+// q=0.05: one MCS at L=8192 from 2.31 to 0.56 ms at 171 instructions per 32
+// attempts, then to 0.48 ms with the draws' places constant in loops over the
+// steps of a level block).  A warp takes the cells of a sub-tile in turns of 32 (NC of them), or
 // several sub-tiles of fewer than 32 cells at once.
 //
 // Cells and random streams are those of cells.cuh (same sites, uniforms and tie
@@ -206,10 +206,10 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
     const uint32_t T = pl.T;
     uint32_t rb[C::NCMAX], db[C::NCMAX];  // half 0 of the next cell's row 0; row 0 of the cell below
     uint32_t on = 0u;                     // turns in which the lane holds a cell
-    uint32_t hd[C::NCMAX];                // tail words of the lane's group: used | generated << 16
+    uint32_t hd[C::NCMAX], gen[C::NCMAX];  // tail words of the lane's group: used, generated
 #pragma unroll
     for (int c = 0; c < C::NCMAX; ++c) {
-        rb[c] = db[c] = hd[c] = 0u;
+        rb[c] = db[c] = hd[c] = gen[c] = 0u;
         if (c >= static_cast<int>(q.nc)) continue;
         const uint32_t base = q.pk > 1u ? seg * q.ngp : 0u;  // the sub-tile's first lane group
         const uint32_t gw = static_cast<uint32_t>(c) * C::GPI + gl, G = gw - base;
@@ -243,36 +243,8 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
     const uint32_t tp4 = a.thr_p >> 28, tq4 = a.thr_q >> 28, low_p = a.thr_p << 4, low_q = a.thr_q << 4;
     constexpr uint32_t kM = 1u | (1u << C::UX);  // X(s) and Y(s) of a half row, at the site's place
     constexpr int U = C::NCMAX < 4 ? C::NCMAX : 4;  // turns in flight
-    uint4 setw = make_uint4(0u, 0u, 0u, 0u);
-    for (uint32_t s = 0; s < static_cast<uint32_t>(S::STEPS); ++s) {
-        if ((s & 63u) == 0u) setw = philox4x32_10(t, a.k | ((s >> 6) << 2), T, kTagSet << 28, a.k0, a.k1);
-        if (s % C::P == 0u) {
-            // the draws of the next P steps, one Philox block per lane at a time
-            const uint32_t n_site = (C::P / S::SPW) * q.ngw, n_all = n_site + (RANDOM ? (C::P / S::SPL) * q.ngw : 0u);
-            for (uint32_t v = lane; v < n_all; v += 32u) {
-                const bool lv = v >= n_site;
-                const uint32_t vv = lv ? v - n_site : v, blk = vv / q.ngw, gw = vv % q.ngw;
-                const uint2 tg = tab[gw];
-                const uint32_t index = lv ? (s / S::SPL + blk) * 8u : s / S::SPW + blk;
-                const uint4 B = philox4x32_10(t, a.k | (index << 2), tg.x, ((lv ? kTagAcc : kTagSite) << 28) | tg.y,
-                                              a.k0, a.k1);
-                if (lv) {
-                    uint32_t pre[4];
-                    transpose_nibbles(make_uint4(B.w, B.z, B.y, B.x), pre);
-                    lvl_w[vv] = make_uint4(pre[0], pre[1], pre[2], pre[3]);
-                } else {
-                    site_w[vv] = B;
-                }
-            }
-            __syncwarp();
-        }
-        uint32_t d = (word_of(setw, (s >> 4) & 3u) >> (2u * (s & 15u))) & 3u;
-        if (q.pk == 1u) d = __shfl_sync(kFull, d, 0);
-        const uint32_t dx = d & 1u, dy = d >> 1;
-        const uint32_t site_sh = (s % S::SPW) * (CX / S::SPW) + CX * j;
-        const uint32_t lvl_sh = 4u * ((s % S::SPL) * S::TPB + j);
-        const uint32_t *const sw = reinterpret_cast<const uint32_t *>(site_w + ((s % C::P) / S::SPW) * q.ngw + gl) + m;
-        const uint32_t *const lw = reinterpret_cast<const uint32_t *>(lvl_w + ((s % C::P) / S::SPL) * q.ngw + gl) + m;
+    // One step: the site word's field at sub, the level word's nibbles at lev.
+    auto step = [&](const uint32_t *sw, uint32_t sub, const uint32_t *lw, uint32_t lev, uint32_t dx, uint32_t dy) {
 #pragma unroll
         for (int c0 = 0; c0 < C::NCMAX; c0 += U) {
             if (c0 >= static_cast<int>(q.nc)) break;
@@ -281,7 +253,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
             for (int u = 0; u < U; ++u) {
                 const int c = c0 + u;
                 if (c >= static_cast<int>(q.nc)) break;
-                const uint32_t f = (sw[c * C::GPI * 4] >> site_sh) & ((1u << S::BPT) - 1u);
+                const uint32_t f = (sw[c * C::GPI * 4] >> (CX * j) >> sub) & ((1u << S::BPT) - 1u);
                 rx[u] = f & static_cast<uint32_t>(C::UX - 1);
                 const uint32_t ly = dy * C::UY + (f >> S::BXB);
                 const uint32_t own = static_cast<uint32_t>(c) * C::TURN + lane * 4u;
@@ -311,7 +283,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
                     acc = (mn && a.p_always) || (mx && a.q_always);
                 } else {
                     const bool drw = SPEC == 2 ? mn || mx : (mn && a.p_random) || (mx && a.q_random);
-                    const uint32_t u4 = (lw[c * C::GPI * 4] >> lvl_sh) & 15u, t4 = mn ? tp4 : tq4;
+                    const uint32_t u4 = (lw[c * C::GPI * 4] >> (4u * j) >> lev) & 15u, t4 = mn ? tp4 : tq4;
                     acc = drw && u4 < t4;
                     if (SPEC != 2) acc = acc || (mn && a.p_always) || (mx && a.q_always);
                     draws += drw ? 1u : 0u;
@@ -322,7 +294,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
                         // words of its tail stream
                         const uint32_t gt = C::GSZ == 32 ? ties : (ties >> (gl * C::GSZ)) & ((1u << C::GSZ) - 1u);
                         const uint32_t nt = static_cast<uint32_t>(__popc(gt));
-                        uint32_t head = hd[c] & 0xFFFFu, end = hd[c] >> 16;
+                        uint32_t head = hd[c], end = gen[c];
                         uint32_t *const rg = ring + (static_cast<uint32_t>(c) * C::GPI + gl) * C::RING;
                         while (__any_sync(kFull, head + nt > end)) {
                             // one block per lane of the group, as many as fit above the live words
@@ -342,7 +314,8 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
                             // (word >> 4) < (P32 mod 2^28)
                             acc = rg[at & (C::RING - 1u)] < (mn ? low_p : low_q);
                         }
-                        hd[c] = (head + nt) | (end << 16);
+                        hd[c] = head + nt;
+                        gen[c] = end;
                         __syncwarp();  // a later refill overwrites words read here
                     }
                 }
@@ -355,6 +328,43 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
             }
         }
         __syncwarp();
+    };
+    const uint32_t site_stride = 4u * q.ngw, lvl_stride = 4u * q.ngw;  // words between blocks of steps
+    uint4 setw = make_uint4(0u, 0u, 0u, 0u);
+    for (uint32_t s0 = 0; s0 < static_cast<uint32_t>(S::STEPS); s0 += C::P) {
+        if ((s0 & 63u) == 0u) setw = philox4x32_10(t, a.k | ((s0 >> 6) << 2), T, kTagSet << 28, a.k0, a.k1);
+        // the draws of the next P steps, one Philox block per lane at a time
+        const uint32_t n_site = (C::P / S::SPW) * q.ngw, n_all = n_site + (RANDOM ? (C::P / S::SPL) * q.ngw : 0u);
+        for (uint32_t v = lane; v < n_all; v += 32u) {
+            const bool lv = v >= n_site;
+            const uint32_t vv = lv ? v - n_site : v, blk = vv / q.ngw, gw = vv % q.ngw;
+            const uint2 tg = tab[gw];
+            const uint32_t index = lv ? (s0 / S::SPL + blk) * 8u : s0 / S::SPW + blk;
+            const uint4 B = philox4x32_10(t, a.k | (index << 2), tg.x, ((lv ? kTagAcc : kTagSite) << 28) | tg.y, a.k0,
+                                          a.k1);
+            if (lv) {
+                uint32_t pre[4];
+                transpose_nibbles(make_uint4(B.w, B.z, B.y, B.x), pre);
+                lvl_w[vv] = make_uint4(pre[0], pre[1], pre[2], pre[3]);
+            } else {
+                site_w[vv] = B;
+            }
+        }
+        __syncwarp();
+        uint32_t sets = word_of(setw, (s0 >> 4) & 3u) >> (2u * (s0 & 15u));
+        if (q.pk == 1u) sets = __shfl_sync(kFull, sets, 0);
+        const uint32_t *sw = reinterpret_cast<const uint32_t *>(site_w + gl) + m;
+        const uint32_t *lw = reinterpret_cast<const uint32_t *>(lvl_w + gl) + m;
+        for (int i0 = 0; i0 < C::P; i0 += S::SPL) {
+#pragma unroll
+            for (int e = 0; e < S::SPL; ++e) {  // the steps of one level block
+                step(sw + (e / S::SPW) * site_stride, (e % S::SPW) * (CX / S::SPW), lw, 4u * (e * S::TPB), sets & 1u,
+                     (sets >> 1) & 1u);
+                sets >>= 2;
+            }
+            sw += (S::SPL / S::SPW) * site_stride;
+            lw += lvl_stride;
+        }
     }
     for (uint32_t sg = 0; sg < q.pk; ++sg) {
         const int src = static_cast<int>(sg * q.ngp * C::GSZ);
@@ -398,9 +408,9 @@ cudaError_t launch_lane_cells(const StepArgs &a, const LaneSplit &q, cudaStream_
 // attempts, with GX * GY of 32 lanes at work.  One MCS at L=8192, p=0.95, q=0.05
 // (us, bit-parallel and lane per cell):
 //   256x64 sub-tiles (32 groups): 8x8 281, 585; 16x8 487, 629; 32x8 773, 634;
-//                                 16x16 906, 637; 32x16 1503, 744
-//   64x64 (8 groups):             8x4 504, 525; 16x4 716, 443; 8x8 847, 461;
-//                                 16x16 2332, 561; 32x16 3850, 780
+//                                 16x16 906, 575; 32x16 1503, 744
+//   64x64 (8 groups):             8x4 504, 525; 16x4 716, 443; 8x8 847, 429;
+//                                 16x8 1263, 421; 16x16 2332, 476; 32x16 3850, 660
 //   32x32 (2 groups):             8x4 1684, 700; 8x8 2832, 591; 16x16 7900, 863
 // so the line lies at cx cy 32 / groups = 256.  Cells four columns wide (half
 // rows of two sites) and sub-tiles whose last group row is so incomplete that
