@@ -339,7 +339,7 @@ int oct_run_mcs(oct_sim *s, int64_t n) {
     if (n < 0) return fail(OCT_EINVAL, "n must be >= 0");
     if (s->t + static_cast<uint64_t>(n) > 0xFFFFFFFFull) return fail(OCT_EINVAL, "MCS counter would pass 2^32-1");
     OCT_CUDA(cudaSetDevice(s->device));
-    if (!s->timing && oct::rows_take(s->args) && oct::rows_fit_cluster(s->args)) {
+    if (!s->timing && oct::rows_take(s->args) && oct::rows_fit_block(s->args)) {
         // whole MCS in one launch (which advances the counter), at most kRunMcs each
         s->args.dt = 0;
         for (int64_t left = n; left > 0; left -= kRunMcs)

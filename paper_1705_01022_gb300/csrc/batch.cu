@@ -132,9 +132,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
 // share the launch (two forms of the step: deposition only, and the general
 // one), so that no replica waits for another's kernel, and there is no graph to
 // capture after every membership change.  Latency bound like rowlanes.cuh: 16
-// MCS and the W^2 of 64 replicas of L = 64..512 take
-// 0.74 ms; at kRowWarpsMax both are level (24 replicas of L=2048, 6144 warps: 2.44
-// ms with the graph).
+// MCS and the W^2 of 64 replicas of L = 64..512 take 0.74 ms.
 template <bool RANDOM, int SPEC, bool ONE>
 __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDesc &wd, uint32_t T, bool held, uint32_t t,
                                                uint32_t k, uint32_t *sm) {
@@ -181,19 +179,24 @@ __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDe
     }
 }
 
-__global__ void __launch_bounds__(kBatchWarps * 32)
-    batch_row_kernel(const ReplicaDev *reps, const BatchItem *items, const WarpDesc *descs, uint32_t n_descs,
-                     const uint32_t *t_of, uint32_t dt, uint32_t k) {
-    __shared__ __align__(16) uint32_t smem[kBatchWarps * row_smem_words<true>()];
-    const uint32_t di = blockIdx.x * kBatchWarps + (threadIdx.x >> 5);
-    if (di >= n_descs) return;  // the whole warp leaves together
-    const WarpDesc wd = descs[di];
+// Larger batches take the graph's branches, whose lanes of four TC rows need
+// fewer instructions per attempt (16 MCS and the W^2 of n replicas of L=2048, 256
+// warps each, ms in row lanes and with the graph: n=20 1.78, 2.38; 24 2.11, 2.44;
+// 32 2.71, 2.86; 48 3.91, 3.05).
+constexpr uint32_t kBatchRowWarpsMax = 152u * 54u;
+
+// One warp per block, so that the blocks spread evenly over the schedulers (16
+// replicas of L=2048, 16 MCS and their W^2: 1.57 ms, 1.78 with four).
+__global__ void __launch_bounds__(32)
+    batch_row_kernel(const ReplicaDev *reps, const BatchItem *items, const WarpDesc *descs, const uint32_t *t_of,
+                     uint32_t dt, uint32_t k) {
+    __shared__ __align__(16) uint32_t sm[row_smem_words<true>()];
+    const WarpDesc wd = descs[blockIdx.x];
     const uint32_t slot = (threadIdx.x & 31u) / wd.G;
     const bool held = slot < wd.n;
     const BatchItem it = items[wd.first + (held ? slot : 0u)];
     const ReplicaDev R = reps[it.rep];
     const uint32_t t = t_of[it.rep] + dt;
-    uint32_t *const sm = smem + (threadIdx.x >> 5) * row_smem_words<true>();
     if (wd.G == 32u) {
         if (wd.kpz)
             batch_row_item<false, 1, true>(R, wd, it.T, held, t, k, sm);
@@ -492,7 +495,7 @@ cudaError_t grow_slots(oct_batch *b, size_t need) {
 }
 
 // The batch in row lanes, if every sub-tile fits a warp that way and a device
-// step has at most kRowWarpsMax warps: items of one form and lane layout
+// step has at most kBatchRowWarpsMax warps: items of one form and lane layout
 // packed into descriptors.  Leaves the lists empty otherwise.
 void row_lists(const std::vector<oct::ReplicaDev> &rd, const std::vector<uint32_t> &active,
                std::vector<oct::BatchItem> &items, std::vector<oct::WarpDesc> &descs) {
@@ -502,7 +505,7 @@ void row_lists(const std::vector<oct::ReplicaDev> &rd, const std::vector<uint32_
         if (D.GX * (D.By / 4u) > 32u) return;
         lanes += static_cast<uint64_t>(D.tiles_x) * D.tiles_y * oct::row_segment(D.GX, D.By);
     }
-    if (lanes > 32ull * oct::kRowWarpsMax) return;
+    if (lanes > 32ull * oct::kBatchRowWarpsMax) return;
     std::vector<oct::BatchItem> bucket[2][6][6];  // form, log2 of GX, of the lanes per sub-tile
     for (uint32_t slot : active) {
         const oct::ReplicaDev &D = rd[slot];
@@ -681,9 +684,8 @@ cudaError_t enqueue_branch_step(oct_batch *b, uint32_t k, int br, cudaStream_t s
 // overlap: its head may run during the tail of the step enqueued before it.
 cudaError_t enqueue_row_step(oct_batch *b, uint32_t dt, uint32_t k, bool overlap, cudaStream_t st) {
     const oct::WorkBuf &w = b->wb[b->cur];
-    const dim3 grid((b->row_descs + oct::kBatchWarps - 1) / oct::kBatchWarps), block(oct::kBatchWarps * 32);
-    return oct::launch_overlapped(oct::batch_row_kernel, grid, block, overlap, st, w.reps, w.items, w.descs,
-                                  b->row_descs, b->d_t, dt, k);
+    return oct::launch_overlapped(oct::batch_row_kernel, dim3(b->row_descs), dim3(32), overlap, st, w.reps, w.items,
+                                  w.descs, b->d_t, dt, k);
 }
 
 // Enqueues device step k of the current MCS of every active replica, branch by branch.

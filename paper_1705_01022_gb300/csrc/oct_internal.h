@@ -48,9 +48,9 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, 
 
 // The device step with one TC row per lane (rowlanes.cu), for lattices too small
 // to fill the chip: whether it takes a step, one step, and n MCS in one launch
-// for lattices that fit a cluster.
+// for lattices that fit a block.
 bool rows_take(const StepArgs &a);
-bool rows_fit_cluster(const StepArgs &a);
+bool rows_fit_block(const StepArgs &a);
 cudaError_t launch_row_step(const StepArgs &a, bool any_random, bool overlap, cudaStream_t st);
 cudaError_t launch_row_run(const StepArgs &a, bool any_random, uint32_t *t_out, uint32_t n, cudaStream_t st);
 

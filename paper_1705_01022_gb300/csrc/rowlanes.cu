@@ -1,13 +1,12 @@
 // Launches of the row-lane device step (rowlanes.cuh).
 //
-// Three forms.  A lattice of at most kBlockWarps warps runs all its MCS in one
-// launch of one block, with the lattice in shared memory.  One of at most
-// kClusterWarps runs them in one launch of one thread-block cluster: the device
-// steps are separated by the hardware's cluster barrier instead of a launch,
-// and a warp draws the random words of the next step between its arrival and
-// its wait.  Larger ones take one launch per device step, each started while
-// the one before writes back (programmatic dependent launch): the draws, which
-// do not depend on the lattice, run before the wait for it.
+// Two forms.  A lattice of at most kBlockWarps warps runs all its MCS in one
+// launch of one block, with the lattice in shared memory.  Larger ones take one
+// launch per device step, each started while the one before writes back
+// (programmatic dependent launch): the draws, which do not depend on the lattice,
+// run before the wait for it.  A cluster of eight blocks for lattices in between
+// was slower than the launches (L=1024, p=0.95, q=0.05, 8 MCS and a W^2: 309 and
+// 253 us): its few SMs share more warps each.
 #include "oct_internal.h"
 
 #include "rowlanes.cuh"
@@ -16,15 +15,16 @@
 namespace oct {
 namespace {
 
-constexpr uint32_t kRowWarps = 4;      // warps per block of a device-step launch
-constexpr uint32_t kClusterCtas = 8;   // the portable limit
-constexpr uint32_t kClusterWarpsPerCta = 8;
-constexpr uint32_t kClusterWarps = kClusterCtas * kClusterWarpsPerCta;
-constexpr uint32_t kBlockWarps = 8;               // of a lattice in one block
-constexpr uint32_t kBlockLattice = 64u * 1024u;  // bytes of its lattice at most (L = 512)
-
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// Warps per block of a device-step launch: one while they still find free
+// places, so that the blocks spread evenly over the schedulers, else four (8
+// MCS and a W^2, us with one and with four: L=1536 257, 274; L=4096 316, 352; 4 MCS
+// at L=6144 (2304 warps) 239, 253; L=8192 (4096 warps) 391, 343).
+constexpr uint32_t kRowWarps = 4;
+constexpr uint32_t kRowSingleMax = 152u * 20u;   // warps of a step in one-warp blocks
+// One block up to a warp per scheduler: 8 MCS and a W^2 at L=256 KPZ 135 us,
+// 149 with launches.
+constexpr uint32_t kBlockWarps = 4;
+constexpr uint32_t kBlockLattice = 64u * 1024u;  // bytes of its lattice at most
 
 template <bool RANDOM, int SPEC, bool ONE, bool SHARED = false, class Ready, class Done>
 __device__ __forceinline__ void row_step(const StepArgs &a, uint32_t *lat, uint32_t warp, uint32_t t, uint32_t k, uint32_t *sm,
@@ -77,46 +77,16 @@ __device__ __forceinline__ void row_counters(const StepArgs &a, uint32_t warp, i
     }
 }
 
-template <bool RANDOM, int SPEC, bool ONE>
-__global__ void __launch_bounds__(kRowWarps * 32) row_step_kernel(const __grid_constant__ StepArgs a) {
-    __shared__ __align__(16) uint32_t sm[kRowWarps * row_smem_words<RANDOM>()];
+template <bool RANDOM, int SPEC, bool ONE, uint32_t WARPS>
+__global__ void __launch_bounds__(WARPS * 32) row_step_kernel(const __grid_constant__ StepArgs a) {
+    __shared__ __align__(16) uint32_t sm[WARPS * row_smem_words<RANDOM>()];
     const uint32_t S = ONE ? 32u : row_segment(a.GX, a.By);
-    const uint32_t warp = blockIdx.x * kRowWarps + (threadIdx.x >> 5);
+    const uint32_t warp = blockIdx.x * WARPS + (threadIdx.x >> 5);
     if (warp * (32u / S) >= work_tiles(a)) return;  // the whole warp leaves together
     int net = 0, draws = 0, tails = 0;
     row_step<RANDOM, SPEC, ONE>(a, a.lat, warp, *a.t_ptr + a.dt, a.k, sm + (threadIdx.x >> 5) * row_smem_words<RANDOM>(), net,
                                 draws, tails, [] { wait_for_previous_grid(); }, [] { launch_dependents(); });
     row_counters<RANDOM>(a, warp, net, draws, tails);
-}
-
-// n MCS of a lattice whose warps fit one cluster (the grid is the cluster).
-template <bool RANDOM, int SPEC, bool ONE>
-__global__ void __launch_bounds__(kClusterWarpsPerCta * 32)
-    row_run_kernel(const __grid_constant__ StepArgs a, uint32_t *t_out, uint32_t n) {
-    __shared__ __align__(16) uint32_t sm[kClusterWarpsPerCta * row_smem_words<RANDOM>()];
-    const uint32_t S = ONE ? 32u : row_segment(a.GX, a.By);
-    const uint32_t warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const bool work = warp * (32u / S) < work_tiles(a);  // a warp without work still keeps the barriers
-    const uint32_t t0 = *a.t_ptr;
-    int net = 0, draws = 0, tails = 0;
-    bool first = true;
-    for (uint32_t i = 0; i < n; ++i)
-        for (uint32_t k = 0; k < 4u; ++k) {
-            const bool wait = !first;
-            if (work)
-                row_step<RANDOM, SPEC, ONE>(a, a.lat, warp, t0 + i, k, sm + (threadIdx.x >> 5) * row_smem_words<RANDOM>(), net,
-                                            draws, tails, [wait] {
-                                                if (wait) cluster_wait();
-                                            },
-                                            [] {});
-            else if (wait)
-                cluster_wait();
-            cluster_arrive();
-            first = false;
-        }
-    cluster_wait();
-    if (warp == 0u && threadIdx.x == 0u) *t_out = t0 + n;
-    if (work) row_counters<RANDOM>(a, warp, net, draws, tails);
 }
 
 // n MCS of a lattice that one block holds in shared memory.
@@ -149,37 +119,21 @@ uint32_t row_warps(const StepArgs &a) {
 
 template <bool RANDOM, int SPEC, bool ONE>
 cudaError_t launch_row_step_as(const StepArgs &a, bool overlap, cudaStream_t st) {
-    const dim3 grid((row_warps(a) + kRowWarps - 1u) / kRowWarps), block(kRowWarps * 32u);
-    return launch_overlapped(row_step_kernel<RANDOM, SPEC, ONE>, grid, block, overlap, st, a);
+    const uint32_t warps = row_warps(a);
+    if (warps <= kRowSingleMax)
+        return launch_overlapped(row_step_kernel<RANDOM, SPEC, ONE, 1u>, dim3(warps), dim3(32u), overlap, st, a);
+    return launch_overlapped(row_step_kernel<RANDOM, SPEC, ONE, kRowWarps>, dim3((warps + kRowWarps - 1u) / kRowWarps),
+                             dim3(kRowWarps * 32u), overlap, st, a);
 }
 
 template <bool RANDOM, int SPEC, bool ONE>
 cudaError_t launch_row_run_as(const StepArgs &a, uint32_t *t_out, uint32_t n, cudaStream_t st) {
-    const uint32_t warps = row_warps(a), bytes = a.L * a.wpr * 8u;
-    if (warps <= kBlockWarps && bytes <= kBlockLattice) {
-        const uint32_t smem = bytes + warps * row_smem_words<RANDOM>() * 4u;
-        cudaError_t e = cudaFuncSetAttribute(row_block_kernel<RANDOM, SPEC, ONE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        row_block_kernel<RANDOM, SPEC, ONE><<<1, warps * 32u, smem, st>>>(a, t_out, n);
-        return cudaGetLastError();
-    }
-    // as few warps per scheduler as eight blocks allow
-    uint32_t per_cta = (warps + kClusterCtas - 1u) / kClusterCtas;
-    per_cta = per_cta < 4u ? (warps < 4u ? warps : 4u) : per_cta;
-    uint32_t ctas = 1u;
-    while (ctas * per_cta < warps) ctas <<= 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(per_cta * 32u);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1u;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, row_run_kernel<RANDOM, SPEC, ONE>, a, t_out, n);
+    const uint32_t warps = row_warps(a), smem = a.L * a.wpr * 8u + warps * row_smem_words<RANDOM>() * 4u;
+    cudaError_t e = cudaFuncSetAttribute(row_block_kernel<RANDOM, SPEC, ONE>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+    row_block_kernel<RANDOM, SPEC, ONE><<<1, warps * 32u, smem, st>>>(a, t_out, n);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -189,7 +143,7 @@ bool rows_take(const StepArgs &a) {
            row_warps(a) <= kRowWarpsMax;
 }
 
-bool rows_fit_cluster(const StepArgs &a) { return row_warps(a) <= kClusterWarps; }
+bool rows_fit_block(const StepArgs &a) { return row_warps(a) <= kBlockWarps && a.L * a.wpr * 8u <= kBlockLattice; }
 
 #define OCT_ROWS(FN, ...)                                                                                \
     do {                                                                                                 \

@@ -13,8 +13,8 @@
 // of repeating them: lane m generates every fourth block of the device step and
 // leaves it (of the acceptance draws, their comparison with P32) in shared
 // memory, before the step's first access to the lattice.  8 MCS and a W^2: L=256
-// KPZ 405 -> 144 us, L=3136 p=0.95 (32 x 16 sub-tiles) 640 -> 291 us, L=4096
-// p=q=0.5 667 -> 390 us.
+// KPZ 405 -> 136 us, L=3136 p=0.95 (32 x 16 sub-tiles) 640 -> 285 us, L=4096
+// p=q=0.5 667 -> 354 us.
 //
 // Lanes of a sub-tile: gx + GX * tr, TC row tr = 0 .. By/4 - 1 (group row tr/4,
 // m = tr % 4), a power-of-two number of band columns GX, at most 32 lanes.
@@ -154,8 +154,7 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
     const uint4 *const lvl = lvl_w + gw;
 
     // one collective step, rows of the set at ro2 = 0 or 2 (dy a constant when ONE)
-    auto step = [&](uint32_t s, uint32_t dx, bool dy) {
-        const uint32_t u = sw[(s >> 1) * (kRowGroups * 4u)] >> (2u * (s & 1u));
+    auto step = [&](uint32_t u, const uint4 &V, uint32_t dx, bool dy) {
         const uint32_t sh2 = 2u * dx, r0 = dy ? 2u : 0u;
         const uint32_t col = ((u & kNib) + kNib) << sh2;  // see step_candidates
         const uint32_t yoff = ((u >> 1) & kNib) * 0xFu;
@@ -178,7 +177,6 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
                 uint32_t pmin = ((cmn * 3u) >> (sh2 + 1u)) & kNib;
                 if (SPEC == 2) pmin &= ~pmax;
                 draws += __popc(pmin | pmax);
-                const uint4 V = lvl[s * kRowGroups];
                 const uint32_t mn = pmin << m, mx4 = pmax << m;  // bit 4j+m
                 acc = (mn & V.x) | (mx4 & V.z);
                 uint32_t und = (mn & V.y) | (mx4 & V.w);
@@ -279,16 +277,29 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
             if (has_b) D ^= vu;
         }
     };
-    for (uint32_t s = 0; s < 16u; ++s) {
-        uint32_t d = (setw.x >> (2u * s)) & 3u;
-        if (ONE) {
-            d = __shfl_sync(kFull, d, 0);  // warp-uniform to the compiler too
+    auto site_of = [&](uint32_t s) { return sw[(s >> 1) * (kRowGroups * 4u)] >> (2u * (s & 1u)); };
+    auto level_of = [&](uint32_t s) { return RANDOM ? lvl[s * kRowGroups] : make_uint4(0u, 0u, 0u, 0u); };
+    if (ONE) {
+        // the sets from lane 0: warp-uniform to the compiler too.  The next step's
+        // draws are read before this step's chain (L=256 KPZ, 8 MCS and a W^2: 145
+        // to 136 us).
+        const uint32_t sets = __shfl_sync(kFull, setw.x, 0);
+        uint32_t u = site_of(0u);
+        uint4 V = level_of(0u);
+        for (uint32_t s = 0; s < 16u; ++s) {
+            const uint32_t us = u, nx = (s + 1u) & 15u, d = (sets >> (2u * s)) & 3u;
+            const uint4 Vs = V;
+            u = site_of(nx);
+            V = level_of(nx);
             if (d & 2u)
-                step(s, d & 1u, true);
+                step(us, Vs, d & 1u, true);
             else
-                step(s, d & 1u, false);
-        } else {
-            step(s, d & 1u, (d & 2u) != 0u);
+                step(us, Vs, d & 1u, false);
+        }
+    } else {
+        for (uint32_t s = 0; s < 16u; ++s) {
+            const uint32_t d = (setw.x >> (2u * s)) & 3u;
+            step(site_of(s), level_of(s), d & 1u, (d & 2u) != 0u);
         }
     }
 

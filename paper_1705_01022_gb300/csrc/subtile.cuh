@@ -234,8 +234,9 @@ __device__ __forceinline__ void step_candidates(const uint32_t (&X)[16], const u
         const uint32_t yoff = dx ? (u & (kNib << 1)) * 6u : ((u >> 1) & kNib) * 3u;
         const int r0 = 4 * m + 2 * DY, r1 = r0 + 1;
         const uint32_t xa = X[r0], xb = X[r1];
-        const uint32_t xra = __funnelshift_r(xa, E >> r0, 1);
-        const uint32_t xrb = __funnelshift_r(xb, E >> r1, 1);
+        // (column 31 is a candidate's only for dx = 1)
+        const uint32_t xra = dx ? __funnelshift_r(xa, E >> r0, 1) : xa >> 1;
+        const uint32_t xrb = dx ? __funnelshift_r(xb, E >> r1, 1) : xb >> 1;
         const uint32_t ya = Y[r0], yb = Y[r1];
         const uint32_t yc = (r1 + 1 < 16) ? Y[(r1 + 1) & 15] : D;
         if (SPEC == 1) {
