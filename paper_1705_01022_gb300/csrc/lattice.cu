@@ -91,6 +91,7 @@ struct W2Lane {
     uint32_t M2, Mz;
     int SPw;
     uint32_t ext;
+    uint32_t St;  // sum of the words' S (see w2_word): the sums t2 are read off it once per chunk
 };
 
 // One 32-site word w.  With a_j the running step inside the word (j = 0..31)
@@ -125,14 +126,15 @@ __device__ __forceinline__ void w2_word(const unsigned char *tab, uint32_t slot,
     const uint32_t ext = min_u16x2(min_u16x2(e0.y, c1), min_u16x2(c2, c3));
     // S = sum .x + 512: Sl = sum 2 t1 + 512, bits 17..26 sum t2
     const uint32_t S = e0.x + e1.x + e2.x + e3.x + 512u;
-    const uint32_t Sl = S & 0x1FFFFu, T2 = (S >> 17) & 0x3FFu;
+    const uint32_t Sl = S & 0x1FFFFu;
+    a.St += S;
     const uint32_t SP = static_cast<uint32_t>(p1 + p2 + p3);
     const uint32_t tw = SP * 16u + Sl;  // 2 A1 + 512
     // lane sums: zp = 32 P + 2 A1 + 512, P zp + Vb + t2 = (word's square sum)
     // + 512 P + 2^16; the offsets are removed at the end of the chunk
     const uint32_t P = static_cast<uint32_t>(a.P);
     const uint32_t zp = P * 32u + tw;
-    a.M2 = zp * P + a.M2 + (acc2 & 0x1FFFFu) + T2;
+    a.M2 = zp * P + a.M2 + (acc2 & 0x1FFFFu);
     a.Mz += zp;
     a.SPw += a.P;
     a.ext = min_u16x2(a.ext, ext + P * 0xFFFF0001u);
@@ -193,7 +195,7 @@ __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
         const uint32_t ny = last ? y + stride : y, nc = last ? 0u : c + 1;
         if (ny < nrows)
             load_lane(lat + static_cast<size_t>(ny) * wpr, nc * kW2ChunkWords + kW2LaneWords * lane, wpr, vec_ok, vn);
-        W2Lane a{0, 0u, 0u, 0, 0xFFFFFFFFu};
+        W2Lane a{0, 0u, 0u, 0, 0xFFFFFFFFu, 0u};
         uint32_t nw = 0;
         if (w0 + kW2ChunkWords <= wpr) {
 #pragma unroll
@@ -209,7 +211,8 @@ __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
         }
         // lane-relative sums: sum q' and sum q'^2 over the lane's 32 nw sites
         // (|q'| <= 512, so both fit 32 bits), extremes and net step
-        const int M2 = static_cast<int>(a.M2 - 512u * static_cast<uint32_t>(a.SPw) - 65536u * nw);
+        const int M2 = static_cast<int>(a.M2 + ((a.St - (static_cast<uint32_t>(a.P) << 27)) >> 17) -
+                                        512u * static_cast<uint32_t>(a.SPw) - 65536u * nw);
         const int M1 = static_cast<int>(a.Mz + 32u * static_cast<uint32_t>(a.SPw) - 512u * nw) / 2;
         const int step = a.P;
         int incl = step;
@@ -503,7 +506,7 @@ __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
         const uint32_t nw = (y < nrows && w < wpr) ? min(lw, wpr - w) : 0u;
         const uint32_t *row = J->lat + static_cast<size_t>(min(y, nrows - 1u)) * wpr;
         const bool vec_ok = lw >= 4u && (wpr & 3u) == 0u && (reinterpret_cast<uintptr_t>(J->lat) & 15u) == 0u;
-        W2Lane a{0, 0u, 0u, 0, 0xFFFFFFFFu};
+        W2Lane a{0, 0u, 0u, 0, 0xFFFFFFFFu, 0u};
         uint32_t v[4], vn[4] = {0u, 0u, 0u, 0u};
         load_quad(row + w, 0u, nw, vec_ok, v);
         for (uint32_t j = 0; j < lw; j += 4u) {
@@ -515,7 +518,8 @@ __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
             for (int i = 0; i < 4; ++i) v[i] = vn[i];
         }
         // as in w2_rows_kernel: the lane's sums, lifted by the steps before it
-        const int M2 = static_cast<int>(a.M2 - 512u * static_cast<uint32_t>(a.SPw) - 65536u * nw);
+        const int M2 = static_cast<int>(a.M2 + ((a.St - (static_cast<uint32_t>(a.P) << 27)) >> 17) -
+                                        512u * static_cast<uint32_t>(a.SPw) - 65536u * nw);
         const int M1 = static_cast<int>(a.Mz + 32u * static_cast<uint32_t>(a.SPw) - 512u * nw) / 2;
         int incl = a.P;
         for (uint32_t o = 1; o < sl; o <<= 1) {

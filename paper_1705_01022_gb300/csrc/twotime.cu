@@ -84,7 +84,8 @@ constexpr int kAcTableBytes = 256 * 256;             // entry e of copy c at byt
 struct AcLane {
     int Bt, Bs;
     int Lt, Ls, Lc;
-    int nx, ny, yt, ys;
+    int ny, yt, ys;
+    uint32_t Sx, Sy;  // sums of the words' sx, sy fields (see ac_word)
 };
 
 // One word pair: sites x..x+31 of X_t (wt) and X_s (ws).  With a_t, a_s the
@@ -120,20 +121,21 @@ __device__ __forceinline__ void ac_word(const unsigned char *tab, uint32_t slot,
         pt = ac_mad_hi(e[k].y, 16, pt);
         ps = ac_mad_hi(e[k].x, 16, ps);
     }
-    uint32_t sx = 0x10000u, sy = 0x10000u;
+    uint32_t sx = 128u, sy = 128u;
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         sx += e[k].x;
         sy += e[k].y;
     }
-    const int At = 4 * spt + static_cast<int>(sy & 0x1FFFFu) - 0x10000;
-    const int As = 4 * sps + static_cast<int>(sx & 0x1FFFFu) - 0x10000;
-    const int C = static_cast<int>(acc & 0x1FFFFu) - 0x10000 + static_cast<int>((sx >> 17) & 0x1FFu) - 240;
+    const int At = 4 * spt + static_cast<int>(sy & 0x1FFFFu) - 128;
+    const int As = 4 * sps + static_cast<int>(sx & 0x1FFFFu) - 128;
+    const int C = static_cast<int>(acc & 0x1FFFFu);  // + 2^16; sum X is added once per chunk
     const int zs = 32 * a.Bs + As;
     a.Lt += 32 * a.Bt + At;
     a.Ls += zs;
     a.Lc += a.Bt * zs + a.Bs * At + C;
-    a.nx += static_cast<int>((sy >> 17) & 0x3Fu);
+    a.Sx += sx;
+    a.Sy += sy;
     a.Bt += pt;
     a.Bs += ps;
 }
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(kAcWarps * 32, kAcBlocksPerSM)
         if (ny_ < L)
             ac_load_chunk(lt, ls, plane, static_cast<size_t>(ny_) * wpr, nc * kAcChunkWords + kAcLaneWords * lane,
                           wpr, vec_ok, nxt);
-        AcLane a{0, 0, 0, 0, 0, 0, 0, 0, 0};
+        AcLane a{0, 0, 0, 0, 0, 0, 0, 0, 0u, 0u};
         uint32_t nw = 0;
         if (w0 + kAcChunkWords <= wpr) {
 #pragma unroll
@@ -225,10 +227,14 @@ __global__ void __launch_bounds__(kAcWarps * 32, kAcBlocksPerSM)
                 }
         }
         const int nbits = 32 * static_cast<int>(nw);
+        // the words' fields above the sums of t1: sum (X + 30), resp. sum c, once the
+        // constants and net steps above them are taken off
+        a.Lc += static_cast<int>((a.Sx - (nw << 30) - (static_cast<uint32_t>(a.Bs) << 28)) >> 17) -
+                static_cast<int>(nw) * (240 + 0x10000);
+        nx += static_cast<int>((a.Sy - (nw << 30) - (static_cast<uint32_t>(a.Bt) << 28)) >> 17);
         // X popcounts from the net steps: popc = (net + bits) / 2
         mt += (a.Bt + nbits) / 2 + a.yt;
         ms += (a.Bs + nbits) / 2 + a.ys;
-        nx += a.nx;
         ny += a.ny;
         // step counts of both lattices in one scan: |prefix| <= 8192 fits the
         // low 16 bits of a two's-complement packed word
