@@ -154,18 +154,10 @@ __device__ __forceinline__ uint4 level_words(uint32_t s, const Ctx &c) {
 
 // PRE: tail words the lane reads at once for its first ties (0: one word per
 // tie in the loop); the fastest choice differs between the block layers.
+// und: the tied candidates (of them, pmin: minima); returns acc with those that
+// their tail words accept.
 template <int PRE, class Ctx>
-__device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pmax, const uint4 &W,
-                                                      const Ctx &c, TailPool &tp) {
-    const uint32_t lw[4] = {W.x, W.y, W.z, W.w};
-    uint32_t acc = 0, und = pmin | pmax;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const uint32_t bit = 31u - static_cast<uint32_t>(i);
-        const uint32_t tb = (((c.thr_p >> bit) & 1u) ? pmin : 0u) | (((c.thr_q >> bit) & 1u) ? pmax : 0u);
-        acc |= und & tb & ~lw[i];
-        und &= ~(tb ^ lw[i]);
-    }
+__device__ __forceinline__ uint32_t resolve_ties(uint32_t acc, uint32_t und, uint32_t pmin, const Ctx &c, TailPool &tp) {
     // Skip the tail stage only when no lane of the warp needs it: every lane
     // takes part in the refill rounds.
     if (__all_sync(kFull, und == 0u)) return acc;
@@ -199,6 +191,22 @@ __device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pm
     }
     tp.head = h + nt;
     return acc;
+}
+
+// The packed candidates against P32 on the four levels, then the ties.
+template <int PRE, class Ctx>
+__device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pmax, const uint4 &W,
+                                                      const Ctx &c, TailPool &tp) {
+    const uint32_t lw[4] = {W.x, W.y, W.z, W.w};
+    uint32_t acc = 0, und = pmin | pmax;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const uint32_t bit = 31u - static_cast<uint32_t>(i);
+        const uint32_t tb = (((c.thr_p >> bit) & 1u) ? pmin : 0u) | (((c.thr_q >> bit) & 1u) ? pmax : 0u);
+        acc |= und & tb & ~lw[i];
+        und &= ~(tb ^ lw[i]);
+    }
+    return resolve_ties<PRE>(acc, und, pmin, c, tp);
 }
 
 // A collective step runs in three phases: the candidates of every thread
@@ -472,6 +480,13 @@ __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[1
     if (c.gy < c.GY - 1) D ^= vu;
 }
 
+// The column 1 << x of every cell's DB site (bits 4j, 4j+1 of the site word u).
+__device__ __forceinline__ uint32_t db_column(uint32_t u) {
+    const uint32_t base = (u & kNib) + kNib;                // 1 << (x & 1)
+    const uint32_t high = base & (((u >> 1) & kNib) * 3u);  // the cells with x >= 2
+    return high * 3u + base;
+}
+
 // One-hot row masks of a DB step: sel[4m + r] holds, for every cell of TC row m
 // whose site lies in its row r, the site's column (site word m: bits 4j, 4j+1
 // = x offset, 4j+2, 4j+3 = y offset of cell j).
@@ -480,9 +495,7 @@ __device__ __forceinline__ void db_select(const uint4 &site, uint32_t (&sel)[16]
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         const uint32_t u = sw[m];
-        const uint32_t base = (u & kNib) + kNib;              // 1 << (x & 1)
-        const uint32_t high = base & (((u >> 1) & kNib) * 3u);  // the cells with x >= 2
-        const uint32_t col = high * 3u + base;                  // 1 << x
+        const uint32_t col = db_column(u);
         const uint32_t C = ((u >> 2) & kNib) * 0xFu, Dd = ((u >> 3) & kNib) * 0xFu;
         sel[4 * m + 0] = col & ~C & ~Dd;
         sel[4 * m + 1] = col & C & ~Dd;
@@ -579,6 +592,32 @@ __device__ __forceinline__ void db_step(uint32_t (&X)[16], uint32_t (&Y)[16], ui
     db_apply(X, Y, E, D, f, c);
 }
 
+// The four leading bits of every cell's uniform against P32's, for p and for q:
+// below (lt) and equal (eq), from the last level up.
+struct LevelCmp {
+    uint32_t ltp, eqp, ltq, eqq;
+};
+template <class Ctx>
+__device__ __forceinline__ LevelCmp level_compare(const uint4 &W, const Ctx &c) {
+    const uint32_t lw[4] = {W.x, W.y, W.z, W.w};
+    LevelCmp v{0u, kFull, 0u, kFull};
+#pragma unroll
+    for (int i = 3; i >= 0; --i) {
+        const uint32_t tp = (c.thr_p >> (31 - i)) & 1u ? kFull : 0u, tq = (c.thr_q >> (31 - i)) & 1u ? kFull : 0u;
+        v.ltp = (tp & ~lw[i]) | (~(tp ^ lw[i]) & v.ltp);
+        v.eqp &= ~(tp ^ lw[i]);
+        v.ltq = (tq & ~lw[i]) | (~(tq ^ lw[i]) & v.ltq);
+        v.eqq &= ~(tq ^ lw[i]);
+    }
+    return v;
+}
+
+// Bitwise v[2 d + c].
+__device__ __forceinline__ uint32_t mux4(uint32_t c, uint32_t d, uint32_t v0, uint32_t v1, uint32_t v2, uint32_t v3) {
+    const uint32_t lo = (c & v1) | (~c & v0), hi = (c & v3) | (~c & v2);
+    return (d & hi) | (~d & lo);
+}
+
 // Four words holding one value bit per cell of TC row m in nibble j (at most
 // one bit set, at any of its four places; a zero nibble is 0): packed to bit
 // 4j+m.  The words are folded in pairs, so that a fold serves two of them.
@@ -625,27 +664,37 @@ __device__ __forceinline__ void transpose_nibbles(const uint4 &site, uint32_t (&
 // shuffles too (8 instead of 12).  Bound by the integer pipe on large
 // lattices and by latency where a step has few warps per scheduler: 2 MCS of
 // L=12288 (256x64, p=0.95, q=0.05; 3.8 warps per scheduler) went from 628 to
-// 511 us.
+// 511 us, and from 465 to 437 us when the attempt's row is picked by bit masks
+// (three selects per quantity instead of an and-or per row) and one comparison
+// of the level words serves the three phases.
 template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                                 const uint4 &site, uint32_t s, const Ctx &c, TailPool &tp,
                                                 int &net, int &draws) {
-    uint32_t sel[16];
-    db_select(site, sel);
+    const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
+    uint32_t col[4], C[4], Dd[4];  // the site's column, one-hot; its row's bits, over the cell
     uint32_t a[4], b[4], lo[4], hi[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        a[m] = b[m] = lo[m] = hi[m] = 0u;
+        const uint32_t u = sw[m];
+        col[m] = db_column(u);
+        C[m] = ((u >> 2) & kNib) * 0xFu;
+        Dd[m] = ((u >> 3) & kNib) * 0xFu;
+        uint32_t x[4], xr[4], y[5];
 #pragma unroll
         for (int r = 0; r < 4; ++r) {
             const int R = 4 * m + r;
-            const uint32_t x = X[R], xr = __funnelshift_r(x, E >> R, 1);
-            const uint32_t y = Y[R], yd = (R < 15) ? Y[(R + 1) & 15] : D;
-            a[m] |= sel[R] & (x ^ xr);
-            b[m] |= sel[R] & (y ^ yd);
-            lo[m] |= sel[R] & ~x & ~y;
-            hi[m] |= sel[R] & x & y;
+            x[r] = X[R];
+            xr[r] = __funnelshift_r(x[r], E >> R, 1);
+            y[r] = Y[R];
         }
+        y[4] = m < 3 ? Y[(4 * m + 4) & 15] : D;
+        const uint32_t xs = mux4(C[m], Dd[m], x[0], x[1], x[2], x[3]), xn = mux4(C[m], Dd[m], xr[0], xr[1], xr[2], xr[3]);
+        const uint32_t ys = mux4(C[m], Dd[m], y[0], y[1], y[2], y[3]), yn = mux4(C[m], Dd[m], y[1], y[2], y[3], y[4]);
+        a[m] = col[m] & (xs ^ xn);
+        b[m] = col[m] & (ys ^ yn);
+        lo[m] = col[m] & ~xs & ~ys;
+        hi[m] = col[m] & xs & ys;
     }
     uint32_t A = pack_cells(a[0], a[1], a[2], a[3]), B = pack_cells(b[0], b[1], b[2], b[3]);
     const uint32_t LO = pack_cells(lo[0], lo[1], lo[2], lo[3]);  // X(s) = Y(s) = 0: a minimum where a and b
@@ -654,21 +703,21 @@ __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)
     transpose_nibbles(site, q);
     const uint32_t x0 = q[0], x1 = q[1], y0 = q[2], y1 = q[3];  // site coordinates in the cell
     const uint32_t xlast = x0 & x1, ylast = y0 & y1;
-    uint4 W = make_uint4(0u, 0u, 0u, 0u);
-    if (RANDOM) W = level_words(s, c);
+    LevelCmp lv{0u, 0u, 0u, 0u};
+    if (RANDOM) lv = level_compare(level_words(s, c), c);
+    uint32_t dmin = 0u, dmax = 0u, dacc = 0u;  // candidates decided by draws, and those accepted
 
     // accepted flips of one phase (cls: its cells)
     auto phase = [&](uint32_t cls) {
         const uint32_t can = A & B & cls, mn = can & LO, mx = can & HI;
-        if (!RANDOM) {
-            const uint32_t fn = mn & c.p_always, fx = mx & c.q_always;
-            net += __popc(fn) - __popc(fx);
-            return fn | fx;
+        uint32_t f = 0u;
+        if (RANDOM) {
+            const uint32_t pmin = SPEC == 2 ? mn : mn & c.p_random, pmax = SPEC == 2 ? mx : mx & c.q_random;
+            f = resolve_ties<kPreDb>((pmin & lv.ltp) | (pmax & lv.ltq), (pmin & lv.eqp) | (pmax & lv.eqq), pmin, c, tp);
+            dmin |= pmin;
+            dmax |= pmax;
+            dacc |= f;
         }
-        const uint32_t pmin = SPEC == 2 ? mn : mn & c.p_random, pmax = SPEC == 2 ? mx : mx & c.q_random;
-        draws += __popc(pmin | pmax);
-        uint32_t f = accept_candidates<kPreDb>(pmin, pmax, W, c, tp);
-        net += random_net(f, pmin, pmax);
         if (SPEC != 2) {
             const uint32_t fn = mn & c.p_always, fx = mx & c.q_always;
             net += __popc(fn) - __popc(fx);
@@ -703,9 +752,20 @@ __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)
         B ^= below(gt, pb);
     }
     F |= F2 | phase(xlast & ylast);  // corners
+    if (RANDOM) {
+        draws += __popc(dmin | dmax);
+        net += random_net(dacc, dmin, dmax);
+    }
+    uint32_t f[16];
 #pragma unroll
-    for (int R = 0; R < 16; ++R) sel[R] &= ((F >> (R >> 2)) & kNib) * 0xFu;
-    db_apply(X, Y, E, D, sel, c);
+    for (int m = 0; m < 4; ++m) {
+        const uint32_t fc = col[m] & (((F >> m) & kNib) * 0xFu);
+        f[4 * m + 0] = fc & ~C[m] & ~Dd[m];
+        f[4 * m + 1] = fc & C[m] & ~Dd[m];
+        f[4 * m + 2] = fc & ~C[m] & Dd[m];
+        f[4 * m + 3] = fc & C[m] & Dd[m];
+    }
+    db_apply(X, Y, E, D, f, c);
 }
 
 // A collective step of DTrDTr (Sec. 4.1.2): DT whose
