@@ -69,15 +69,16 @@ __device__ __forceinline__ uint32_t word_of(const uint4 &w, uint32_t m) {
     return pick4(m, w.x, w.y, w.z, w.w);
 }
 
-// One word per row of the active half cell: the columns of the cells whose site
-// lies in that row.  u holds the cells' offsets from bit cx*j on (x offset,
-// then y offset); all cells are built together, an offset bit at a time: the
-// column 1 << rx by moving the bits of the cells with offset bit b up by 2^b
-// columns, then split by the bits of the row.  (A cell at a time this was a fifth
-// of a step's instructions; with the blocks shared by a group's lanes, one MCS of
-// 8x8 cells at L=16384, 256x64, p=0.95, q=0.05 went from 872 to 730 us.)
+// The sites of a TC row's cells.  u holds the cells' offsets from bit cx*j on (x
+// offset, then y offset); all cells are built together, an offset bit at a
+// time: the column 1 << rx by moving the bits of the cells with offset bit b up
+// by 2^b columns; hi[b] covers the cells with bit b of the row set.  (A cell at a
+// time this was a fifth of a step's instructions; with the blocks shared by a
+// group's lanes, one MCS of 8x8 cells at L=16384, 256x64, p=0.95, q=0.05 went from
+// 872 to 730 us, and to 691 us with each cell's bits picked by row instead of a
+// test of every row.)
 template <int CX, int CY>
-__device__ __forceinline__ void cells_select(uint32_t u, uint32_t dx, uint32_t (&M)[CY / 2]) {
+__device__ __forceinline__ uint32_t cells_select(uint32_t u, uint32_t dx, uint32_t (&hi)[CellShape<CX, CY>::BYB]) {
     using S = CellShape<CX, CY>;
     constexpr uint32_t kOne = CX == 4 ? 0x11111111u : CX == 8 ? 0x01010101u : CX == 16 ? 0x00010001u : 1u;
     uint32_t col = kOne;
@@ -86,29 +87,56 @@ __device__ __forceinline__ void cells_select(uint32_t u, uint32_t dx, uint32_t (
         const uint32_t span = (1u << (1 << b)) - 1u;  // columns [0, 2^b), one of them set
         col += (col & (((u >> b) & kOne) * span)) * span;
     }
-    M[0] = col << (dx * S::UX);
 #pragma unroll
-    for (int b = S::BYB - 1; b >= 0; --b) {
-        const uint32_t hi = ((u >> (S::BXB + b)) & kOne) * S::CMASK;  // cells with this bit of ry
-#pragma unroll
-        for (int v = S::UY - (2 << b); v >= 0; v -= 2 << b) {
-            M[v + (1 << b)] = M[v] & hi;
-            M[v] &= ~hi;
-        }
-    }
+    for (int b = 0; b < S::BYB; ++b) hi[b] = ((u >> (S::BXB + b)) & kOne) * S::CMASK;
+    return col << (dx * S::UX);
 }
 
+// Splits F[0] by row into F.
+template <int BYB>
+__device__ __forceinline__ void split_rows(const uint32_t (&hi)[BYB], uint32_t (&F)[1 << BYB]) {
+#pragma unroll
+    for (int b = BYB - 1; b >= 0; --b)
+#pragma unroll
+        for (int v = (1 << BYB) - (2 << b); v >= 0; v -= 2 << b) {
+            F[v + (1 << b)] = F[v] & hi[b];
+            F[v] &= ~hi[b];
+        }
+}
+
+// Bitwise v[row], row given by hi.
+template <int BYB>
+__device__ __forceinline__ uint32_t pick_row(const uint32_t (&hi)[BYB], const uint32_t *v) {
+    uint32_t w[1 << BYB];
+#pragma unroll
+    for (int i = 0; i < (1 << BYB); ++i) w[i] = v[i];
+#pragma unroll
+    for (int b = 0; b < BYB; ++b)
+#pragma unroll
+        for (int i = 0; i < (1 << (BYB - 1 - b)); ++i) w[i] = (hi[b] & w[2 * i + 1]) | (~hi[b] & w[2 * i]);
+    return w[0];
+}
+
+// The candidates of a step: per TC row the columns, where X(s) = 0, and the bits
+// of the cells' rows (hi of cells_select).
+template <int CX, int CY>
+struct CellCand {
+    uint32_t cand[CellShape<CX, CY>::NTR], low[CellShape<CX, CY>::NTR];
+    uint32_t rows[CellShape<CX, CY>::NTR][CellShape<CX, CY>::BYB];
+    uint32_t flip[CellShape<CX, CY>::NTR * CellShape<CX, CY>::UY];  // deposition only: the flips of every active row
+};
+
 // Phase 1 with sub-cell set (dx, DY): every cell (j, TC row i) of the lane
-// attempts site (cx*j + dx*cx/2 + rx, i*cy + DY*cy/2 + ry) of the lane.  The
-// cells' sites are gathered into one column mask per row of the active
-// half (cand[i*UY + v] holds row i*cy + DY*UY + v); an attempt is eligible iff
-// X(s) != X(s+x), Y(s) != Y(s+y) and X(s) == Y(s) (Eq. (1)), the minimum
-// being X(s) = 0.  Candidates needing a draw are packed to bit 4j+m.
+// attempts site (cx*j + dx*cx/2 + rx, i*cy + DY*cy/2 + ry) of the lane.  Each
+// cell's four slope bits are picked from the rows of its active half by the
+// bits of ry; an attempt is eligible iff X(s) != X(s+x), Y(s) != Y(s+y) and X(s)
+// == Y(s) (Eq. (1)), the minimum being X(s) = 0.  Candidates needing a draw are
+// packed to bit 4j+m.
 template <int CX, int CY, int DY, bool RANDOM, int SPEC>
 __device__ __forceinline__ void cells_candidates(const uint32_t (&X)[16], const uint32_t (&Y)[16], uint32_t E,
                                                  uint32_t D, const uint32_t (&site)[CellShape<CX, CY>::NTR],
                                                  uint32_t s, uint32_t dx,
-                                                 const CellCtx &cc, uint32_t (&cand)[8], uint32_t &pmin,
+                                                 const CellCtx &cc, CellCand<CX, CY> &q, uint32_t &pmin,
                                                  uint32_t &pmax) {
     using S = CellShape<CX, CY>;
     const uint32_t sub = (s % S::SPW) * (CX / S::SPW);
@@ -117,27 +145,33 @@ __device__ __forceinline__ void cells_candidates(const uint32_t (&X)[16], const 
 #pragma unroll
     for (int i = 0; i < S::NTR; ++i) {
         const uint32_t m = cc.m0 + static_cast<uint32_t>(i);
-        uint32_t M[S::UY];
-        cells_select<CX, CY>(site[i] >> sub, dx, M);
-        uint32_t mn = 0u, mx = 0u;
+        const uint32_t col = cells_select<CX, CY>(site[i] >> sub, dx, q.rows[i]);
+        uint32_t x[S::UY], xr[S::UY], y[S::UY + 1];
 #pragma unroll
         for (int v = 0; v < S::UY; ++v) {
             const int r = i * CY + DY * S::UY + v;
-            const uint32_t x = X[r];
-            const uint32_t xr = __funnelshift_r(x, E >> r, 1);
-            const uint32_t y = Y[r];
-            const uint32_t yd = (r + 1 < 16) ? Y[(r + 1) & 15] : D;
-            uint32_t cd;
-            if (SPEC == 1)
-                cd = M[v] & ~x & xr & ~y & yd;  // deposition only: the minima
-            else
-                cd = M[v] & (x ^ xr) & (y ^ yd) & ~(x ^ y);
-            cand[i * S::UY + v] = cd;
-            if (RANDOM) {
-                mn |= cd & ~x;
-                mx |= cd & x;
-            }
+            x[v] = X[r];
+            xr[v] = __funnelshift_r(x[v], E >> r, 1);
+            y[v] = Y[r];
         }
+        constexpr int kHalf = DY * S::UY + S::UY;
+        y[S::UY] = (i * CY + kHalf < 16) ? Y[(i * CY + kHalf) & 15] : D;
+        if (SPEC == 1) {
+            // every minimum flips: nothing to pack, and a test per row is cheaper than
+            // picking four bits and splitting the flips again (8x8: 363 and 375 us)
+            uint32_t M[S::UY];
+            M[0] = col;
+            split_rows(q.rows[i], M);
+#pragma unroll
+            for (int v = 0; v < S::UY; ++v) q.flip[i * S::UY + v] = M[v] & ~x[v] & xr[v] & ~y[v] & y[v + 1];
+            continue;
+        }
+        const uint32_t xs = pick_row<S::BYB>(q.rows[i], x), xn = pick_row<S::BYB>(q.rows[i], xr);
+        const uint32_t ys = pick_row<S::BYB>(q.rows[i], y), yn = pick_row<S::BYB>(q.rows[i], y + 1);
+        const uint32_t cd = col & (xs ^ xn) & (ys ^ yn) & ~(xs ^ ys);
+        q.cand[i] = cd;
+        q.low[i] = ~xs;
+        uint32_t mn = cd & ~xs, mx = cd & xs;
         if (RANDOM) {
             if (SPEC != 2) {
                 mn &= cc.c.p_random;
@@ -208,7 +242,7 @@ __device__ __forceinline__ uint32_t cells_accept(uint32_t pmin, uint32_t pmax, c
 // 15 only for DY = 1 and row 0 only for DY = 0).
 template <int CX, int CY, int DY, bool RANDOM, int SPEC>
 __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
-                                            uint32_t dx, uint32_t acc, const uint32_t (&cand)[8], const CellCtx &cc,
+                                            uint32_t dx, uint32_t acc, const CellCand<CX, CY> &q, const CellCtx &cc,
                                             int &net) {
     using S = CellShape<CX, CY>;
     const LaneCtx<KeysConst> &c = cc.c;
@@ -229,21 +263,23 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
         }
         const uint32_t amin = c.p_always | (spread & c.p_random);
         const uint32_t amax = c.q_always | (spread & c.q_random);
+        uint32_t F[S::UY];  // the TC row's flips, by row of the active half
+        if (SPEC == 1) {
+            uint32_t any = 0u;
+#pragma unroll
+            for (int v = 0; v < S::UY; ++v) any |= F[v] = q.flip[i * S::UY + v];
+            net += __popc(any);  // one flip per cell
+        } else if (SPEC == 2) {
+            F[0] = q.cand[i] & spread;
+        } else {
+            F[0] = q.cand[i] & ((q.low[i] & amin) | (~q.low[i] & amax));
+            net += always_net<RANDOM>(F[0], ~q.low[i], c);
+        }
+        if (SPEC != 1) split_rows(q.rows[i], F);
 #pragma unroll
         for (int v = 0; v < S::UY; ++v) {
             const int r = i * CY + DY * S::UY + v;
-            const uint32_t x = X[r];
-            const uint32_t cd = cand[i * S::UY + v];
-            uint32_t f;
-            if (SPEC == 1) {
-                f = cd;
-                net += __popc(f);
-            } else if (SPEC == 2) {
-                f = cd & spread;
-            } else {
-                f = cd & ((~x & amin) | (x & amax));
-                net += always_net<RANDOM>(f, x, c);
-            }
+            const uint32_t x = X[r], f = F[v];
             X[r] = x ^ (f * 3u);  // f ^ (f << 1): one flip per cell, cells at least cx columns apart
             Y[r] ^= f;
             if (r + 1 < 16)
@@ -336,7 +372,8 @@ __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uin
         const uint32_t *const sw = reinterpret_cast<const uint32_t *>(site_w + (s % S::DRAW) / S::SPW * 32 + g_at) + cc.m0;
 #pragma unroll
         for (int i = 0; i < S::NTR; ++i) site[i] = sw[i];
-        uint32_t cand[8], pmin, pmax;
+        CellCand<CX, CY> cand;
+        uint32_t pmin, pmax;
         if (d & 2u)
             cells_candidates<CX, CY, 1, RANDOM, SPEC>(X, Y, E, D, site, s, d & 1u, cc, cand, pmin, pmax);
         else
