@@ -247,6 +247,7 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
     using S = CellShape<CX, CY>;
     const LaneCtx<KeysConst> &c = cc.c;
     uint32_t dE = 0u, dB0 = 0u, dD = 0u, dY0 = 0u;
+    uint32_t all[16] = {};  // the flips by row
 #pragma unroll
     for (int i = 0; i < S::NTR; ++i) {
         const uint32_t m = cc.m0 + static_cast<uint32_t>(i);
@@ -286,14 +287,14 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
                 Y[(r + 1) & 15] ^= f;
             else
                 D ^= f;
-            dE |= (f >> 31) << r;
-            dB0 |= (f & 1u) << r;
+            all[r] = f;
             if (r == 15) dD = f;
             if (r == 0) dY0 = f;
         }
     }
     if (dx) {
         // flips at bit 31 changed column 0 of the right neighbour (this lane's E)
+        dE = gather_msb(all);
         E ^= dE;
         const uint32_t vr = __shfl_up_sync(kFull, dE, 1);
         if (c.gx > 0) {
@@ -307,6 +308,7 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
         }
     } else {
         // flips at bit 0 changed this lane's column 0, mirrored by the left neighbour's E
+        dB0 = gather_lsb(all);
         const uint32_t vl = __shfl_down_sync(kFull, dB0, 1);
         if (c.gx < c.GX - 1) E ^= vl;
     }
