@@ -23,6 +23,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <utility>
 #include <vector>
 
@@ -91,7 +92,8 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
         if (x0 >= L) x0 -= L;
         uint32_t y0 = __umulhi(M.y, L) + R.By * (2u * ty + (sigma >> 1));
         if (y0 >= L) y0 -= L;
-        LaneCtx<KeysWeyl> c;
+        using Keys = std::conditional_t<SCHEME == 4, KeysWeyl, KeysFma>;
+        LaneCtx<Keys> c;
         c.GX = static_cast<int>(wd.GX);
         c.GY = G / c.GX;
         c.gx = sub % c.GX;
@@ -102,7 +104,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
         c.k = k;
         c.T = it.T;
         c.g = static_cast<uint32_t>(sub);
-        c.key = KeysWeyl{R.k0, R.k1};
+        c.key = Keys(R.k0, R.k1);
         c.first_round();
         c.thr_p = R.thr_p;
         c.thr_q = R.thr_q;
@@ -158,7 +160,7 @@ __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDe
     c.T = T;
     c.g = (static_cast<uint32_t>(rl.tr) >> 2) * wd.GX + static_cast<uint32_t>(rl.gx);
     rl.gw = seg * (S / 4u) + c.g;
-    c.key = KeysWeyl{R.k0, R.k1};
+    c.key = KeysWeyl(R.k0, R.k1);
     c.first_round();
     c.thr_p = R.thr_p;
     c.thr_q = R.thr_q;

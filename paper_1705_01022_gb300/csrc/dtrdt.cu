@@ -86,11 +86,9 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     const TilePlace pl = place_tile(a, w < n_tiles ? w : 0u, t, a.k);
     const uint32_t T = pl.T, x0 = pl.x0, y0 = pl.y0;
 
-    // Deposition only draws one block per two steps: there the key additions are
-    // cheaper than the constant operands (127.6 and 135.0 us for one MCS at L=16384,
-    // 256x64); with draws the constants win (L=2^17, 1024x16, p=0.95: see subtile.cuh).
-    constexpr bool kWeyl = SCHEME == 4;
-    LaneCtx<std::conditional_t<kWeyl, KeysWeyl, KeysConst>> c;
+    // round keys: see KeysConst
+    using Keys = std::conditional_t<SCHEME == 4, KeysWeyl, std::conditional_t<SCHEME == 0 || SCHEME == 5, KeysFma, KeysConst>>;
+    LaneCtx<Keys> c;
     c.GX = static_cast<int>(a.GX);
     c.GY = static_cast<int>(a.GY);
     c.gx = static_cast<int>(sub) % c.GX;
@@ -102,10 +100,10 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     c.k = a.k;
     c.T = T;
     c.g = sub;
-    if constexpr (kWeyl)
-        c.key = KeysWeyl{a.k0, a.k1};
-    else
+    if constexpr (std::is_same_v<Keys, KeysConst>)
         c.key.a = &a;
+    else
+        c.key = Keys(a.k0, a.k1);
     c.first_round();
     c.thr_p = a.thr_p;
     c.thr_q = a.thr_q;

@@ -36,17 +36,36 @@ __device__ __forceinline__ void reduce_bits(uint32_t *w, uint32_t v, uint32_t ma
     atomicOr(w, v & mask);
 }
 
-// Round keys of Philox: from the launch's arguments (constant memory, so that
-// they cost neither registers nor additions) or from the key itself.  With the
-// first round's products kept per sub-tile, one MCS at L=2^17 (1024x16, p=0.95,
-// q=0.05) takes 1.4 % less.
+// A 1 that the compiler does not know: one * c + x is then a multiply-add on the
+// FMA pipe, where x + c would run on the integer pipe that binds the step.
+__device__ __forceinline__ uint32_t opaque_one() {
+    uint32_t v;
+    asm volatile("mov.u32 %0, 1;" : "=r"(v));
+    return v;
+}
+
+// Round keys of Philox: from the launch's arguments (constant memory, neither
+// registers nor additions), by multiply-adds, or by plain additions.  One MCS at
+// L=2^17 (1024x16, p=0.95, q=0.05) 9.57, 9.45 and 9.8 ms, at L=32768 KPZ (which
+// draws one block in two steps) additions 355 us, multiply-adds 357 us; DTrDB at
+// L=12288 constants 437 us, multiply-adds 446 us; DTrDTr at L=8192 270, 275 us.
 struct KeysConst {
     const StepArgs *a;
     __device__ __forceinline__ uint32_t lo(int r) const { return a->rk0[r]; }
     __device__ __forceinline__ uint32_t hi(int r) const { return a->rk1[r]; }
 };
+struct KeysFma {
+    uint32_t k0, k1, one;
+    __device__ __forceinline__ KeysFma() {}
+    __device__ __forceinline__ KeysFma(uint32_t lo_word, uint32_t hi_word)
+        : k0(lo_word), k1(hi_word), one(opaque_one()) {}
+    __device__ __forceinline__ uint32_t lo(int r) const { return one * (static_cast<uint32_t>(r) * 0x9E3779B9u) + k0; }
+    __device__ __forceinline__ uint32_t hi(int r) const { return one * (static_cast<uint32_t>(r) * 0xBB67AE85u) + k1; }
+};
 struct KeysWeyl {
     uint32_t k0, k1;
+    __device__ __forceinline__ KeysWeyl() {}
+    __device__ __forceinline__ KeysWeyl(uint32_t lo_word, uint32_t hi_word) : k0(lo_word), k1(hi_word) {}
     __device__ __forceinline__ uint32_t lo(int r) const { return k0 + static_cast<uint32_t>(r) * 0x9E3779B9u; }
     __device__ __forceinline__ uint32_t hi(int r) const { return k1 + static_cast<uint32_t>(r) * 0xBB67AE85u; }
 };
