@@ -411,6 +411,9 @@ int oct_batch_measure_slot(oct_batch *b, int64_t slot, oct_w2 *out);
  * this way without stalling the device (Sec. 2.1, Eq. (3); the scheduling is
  * this library's, the paper has no counterpart). */
 int oct_batch_measure_async(oct_batch *b, int64_t slot, int64_t *ticket);
+/* The same for n replicas (at most 1024; a slot may be named more than once) in
+ * as few launches as they need; tickets[i] belongs to slots[i]. */
+int oct_batch_measure_slots_async(oct_batch *b, const int64_t *slots, int64_t n, int64_t *tickets);
 int oct_batch_poll(oct_batch *b, int64_t ticket, oct_w2 *out, int *ready);
 int oct_batch_wait(oct_batch *b, int64_t ticket, oct_w2 *out);
 

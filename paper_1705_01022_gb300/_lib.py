@@ -130,6 +130,8 @@ _SIGNATURES = [
     ("oct_batch_run", [_H, ctypes.c_int64], ctypes.c_int),
     ("oct_batch_measure_slot", [_H, ctypes.c_int64, ctypes.POINTER(oct_w2)], ctypes.c_int),
     ("oct_batch_measure_async", [_H, ctypes.c_int64, ctypes.POINTER(ctypes.c_int64)], ctypes.c_int),
+    ("oct_batch_measure_slots_async", [_H, ctypes.POINTER(ctypes.c_int64), ctypes.c_int64,
+                                       ctypes.POINTER(ctypes.c_int64)], ctypes.c_int),
     ("oct_batch_poll", [_H, ctypes.c_int64, ctypes.POINTER(oct_w2), ctypes.POINTER(ctypes.c_int)], ctypes.c_int),
     ("oct_batch_wait", [_H, ctypes.c_int64, ctypes.POINTER(oct_w2)], ctypes.c_int),
     ("oct_batch_measure_w2", [_H, ctypes.POINTER(oct_w2), ctypes.c_int64], ctypes.c_int),
@@ -365,6 +367,13 @@ def oct_batch_measure_async(h: int, slot: int) -> int:
     t = ctypes.c_int64()
     _check(load().oct_batch_measure_async(h, slot, ctypes.byref(t)), "oct_batch_measure_async")
     return t.value
+
+
+def oct_batch_measure_slots_async(h: int, slots) -> list[int]:
+    n = len(slots)
+    t = (ctypes.c_int64 * n)()
+    _check(load().oct_batch_measure_slots_async(h, (ctypes.c_int64 * n)(*slots), n, t), "oct_batch_measure_slots_async")
+    return list(t)
 
 
 def oct_batch_poll(h: int, ticket: int):

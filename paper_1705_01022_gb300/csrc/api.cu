@@ -507,7 +507,7 @@ int enqueue_w2(oct_sim *s) {
         j.cnt = s->d_net;
         j.cnt_n = j.cnt_off = oct::kNetSlots;
         j.cnt_out = reinterpret_cast<long long *>(static_cast<char *>(s->h_small) + 128);
-        OCT_CUDA(oct::launch_w2_small_one(j, s->d_rows, s->stream));
+        OCT_CUDA(oct::launch_w2_small_pack(&j, 1, s->d_rows, s->stream));
         s->w2_pending = true;
         s->w2_t = s->t;
         return OCT_OK;

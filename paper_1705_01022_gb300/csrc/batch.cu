@@ -214,6 +214,8 @@ __global__ void __launch_bounds__(32)
 
 // Adds n to the MCS counter of every active replica.
 __global__ void batch_advance_kernel(uint32_t *t_of, const uint32_t *active, uint32_t n_active, uint32_t n) {
+    launch_dependents();
+    wait_for_previous_grid();
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_active; i += gridDim.x * blockDim.x)
         t_of[active[i]] += n;
 }
@@ -279,6 +281,9 @@ struct MeasureRecord {
 // records); larger batches take several launches.
 constexpr uint64_t kMeasureRows = uint64_t{1} << 20;
 constexpr int kMeasureRing = 1024;
+// Rows one launch of an asynchronous measurement takes beyond its first
+// replica: the batch's scratch grows to at most 3 MB for it.
+constexpr int64_t kPackRows = 65536;
 constexpr int kMarkRing = 64;
 constexpr int kGraphMcs = 4;  // MCS in the batch's longer captured graph
 
@@ -345,6 +350,7 @@ struct oct_batch {
     oct::MeasureRecord *h_req = nullptr;
     std::vector<cudaEvent_t> req_ev;
     std::vector<int64_t> req_L;
+    std::vector<int> req_at;  // ring index of the event recorded behind the ticket's launches
     int64_t req_next = 0;  // tickets handed out so far
     // stream marks (oct_batch_mark): a ring of events
     std::vector<cudaEvent_t> mark_ev;
@@ -704,8 +710,9 @@ cudaError_t enqueue_step(oct_batch *b, uint32_t k, cudaStream_t st) {
 cudaError_t enqueue_advance(oct_batch *b, uint32_t n, cudaStream_t st) {
     if (b->n_active == 0) return cudaSuccess;
     const int blocks = static_cast<int>(std::min<uint32_t>(1024u, (b->n_active + 255u) / 256u));
-    oct::batch_advance_kernel<<<blocks, 256, 0, st>>>(b->d_t, b->wb[b->cur].active, b->n_active, n);
-    return cudaGetLastError();
+    const uint32_t *active = b->wb[b->cur].active;
+    return oct::launch_overlapped(oct::batch_advance_kernel, dim3(blocks), dim3(256), true, st, b->d_t, active,
+                                  b->n_active, n);
 }
 
 // Advances the MCS counters of the replicas of one branch.
@@ -858,7 +865,8 @@ int measure_slot(oct_batch *b, int64_t slot, oct_w2 *out) {
     int rc = ensure_rows(b, b->reps[slot].L);
     if (rc) return rc;
     auto *m = static_cast<oct::MeasureRecord *>(b->h_small);
-    BATCH_CUDA(oct::launch_w2_small_one(replica_job(b, slot, m), b->d_rows, b->stream));
+    oct::W2Job j = replica_job(b, slot, m);
+    BATCH_CUDA(oct::launch_w2_small_pack(&j, 1, b->d_rows, b->stream));
     BATCH_CUDA(cudaStreamSynchronize(b->stream));
     record_to_w2(*m, b->reps[slot].L, out);
     return OCT_OK;
@@ -921,26 +929,48 @@ int ticket_index(oct_batch *b, int64_t ticket, int *idx) {
 extern "C" {
 
 int oct_batch_measure_async(oct_batch *b, int64_t slot, int64_t *ticket) {
-    if (!b || !ticket || !valid_slot(b, slot)) return bfail(OCT_EINVAL, "no replica in that slot");
+    return oct_batch_measure_slots_async(b, &slot, 1, ticket);
+}
+
+int oct_batch_measure_slots_async(oct_batch *b, const int64_t *slots, int64_t n, int64_t *tickets) {
+    if (!b || n < 0 || n > oct::kMeasureRing || (n > 0 && (!slots || !tickets)))
+        return bfail(OCT_EINVAL, "bad slot list");
+    for (int64_t i = 0; i < n; ++i)
+        if (!valid_slot(b, slots[i])) return bfail(OCT_EINVAL, "no replica in that slot");
+    if (n == 0) return OCT_OK;
     BATCH_CUDA(cudaSetDevice(b->device));
-    const int64_t L = b->reps[slot].L;
     if (!b->h_req) {
-        BATCH_CUDA(cudaMallocHost(&b->h_req, sizeof(oct::MeasureRecord) * oct::kMeasureRing));
         b->req_ev.assign(oct::kMeasureRing, nullptr);
         b->req_L.assign(oct::kMeasureRing, 0);
+        b->req_at.assign(oct::kMeasureRing, 0);
+        BATCH_CUDA(cudaMallocHost(&b->h_req, sizeof(oct::MeasureRecord) * oct::kMeasureRing));
     }
-    const int i = static_cast<int>(b->req_next % oct::kMeasureRing);
-    if (b->req_ev[i]) {
-        BATCH_CUDA(cudaEventSynchronize(b->req_ev[i]));  // the ring wrapped: the oldest record is done
-    } else {
-        BATCH_CUDA(cudaEventCreateWithFlags(&b->req_ev[i], cudaEventDisableTiming));
+    for (int64_t first = 0; first < n;) {
+        oct::W2Job jobs[oct::kW2PackJobs];
+        uint32_t m = 0;
+        int64_t rows = 0;
+        while (first + m < n && m < oct::kW2PackJobs) {
+            const int64_t slot = slots[first + m], L = b->reps[slot].L, ticket = b->req_next + m;
+            if (m > 0 && rows + L > oct::kPackRows) break;
+            const int i = static_cast<int>(ticket % oct::kMeasureRing);
+            if (ticket >= oct::kMeasureRing)  // the ring wrapped: the oldest record is done
+                BATCH_CUDA(cudaEventSynchronize(b->req_ev[b->req_at[i]]));
+            jobs[m++] = replica_job(b, slot, b->h_req + i);
+            rows += L;
+        }
+        const int at = static_cast<int>((b->req_next + m - 1) % oct::kMeasureRing);
+        if (!b->req_ev[at]) BATCH_CUDA(cudaEventCreateWithFlags(&b->req_ev[at], cudaEventDisableTiming));
+        int rc = ensure_rows(b, rows);
+        if (rc) return rc;
+        BATCH_CUDA(oct::launch_w2_small_pack(jobs, m, b->d_rows, b->stream));
+        BATCH_CUDA(cudaEventRecord(b->req_ev[at], b->stream));
+        for (uint32_t i = 0; i < m; ++i) {
+            const int r = static_cast<int>(b->req_next % oct::kMeasureRing);
+            b->req_L[r] = b->reps[slots[first]].L;
+            b->req_at[r] = at;
+            tickets[first++] = b->req_next++;
+        }
     }
-    int rc = ensure_rows(b, L);
-    if (rc) return rc;
-    BATCH_CUDA(oct::launch_w2_small_one(replica_job(b, slot, b->h_req + i), b->d_rows, b->stream));
-    BATCH_CUDA(cudaEventRecord(b->req_ev[i], b->stream));
-    b->req_L[i] = L;
-    *ticket = b->req_next++;
     return OCT_OK;
 }
 
@@ -950,7 +980,7 @@ int oct_batch_poll(oct_batch *b, int64_t ticket, oct_w2 *out, int *ready) {
     int rc = ticket_index(b, ticket, &i);
     if (rc) return rc;
     BATCH_CUDA(cudaSetDevice(b->device));
-    const cudaError_t e = cudaEventQuery(b->req_ev[i]);
+    const cudaError_t e = cudaEventQuery(b->req_ev[b->req_at[i]]);
     if (e == cudaErrorNotReady) {
         (void)cudaGetLastError();  // "not ready" is an answer, not an error: do not leave it behind
         *ready = 0;
@@ -968,7 +998,7 @@ int oct_batch_wait(oct_batch *b, int64_t ticket, oct_w2 *out) {
     int rc = ticket_index(b, ticket, &i);
     if (rc) return rc;
     BATCH_CUDA(cudaSetDevice(b->device));
-    BATCH_CUDA(cudaEventSynchronize(b->req_ev[i]));
+    BATCH_CUDA(cudaEventSynchronize(b->req_ev[b->req_at[i]]));
     record_to_w2(b->h_req[i], b->req_L[i], out);
     return OCT_OK;
 }

@@ -135,7 +135,11 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     }
 }
 
-__global__ void advance_t_kernel(uint32_t *t_ptr, uint32_t n) { *t_ptr += n; }
+__global__ void advance_t_kernel(uint32_t *t_ptr, uint32_t n) {
+    launch_dependents();
+    wait_for_previous_grid();
+    *t_ptr += n;
+}
 
 }  // namespace
 
@@ -206,8 +210,7 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, 
 }
 
 cudaError_t launch_advance_t(uint32_t *t_ptr, uint32_t n, cudaStream_t st) {
-    advance_t_kernel<<<1, 1, 0, st>>>(t_ptr, n);
-    return cudaGetLastError();
+    return launch_overlapped(advance_t_kernel, dim3(1), dim3(1), true, st, t_ptr, n);
 }
 
 }  // namespace oct

@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "oct_internal.h"
+#include "overlap.cuh"
 
 namespace oct {
 namespace {
@@ -461,7 +462,9 @@ __global__ void __launch_bounds__(kW2CombineThreads)
 // Bound by launches and latency, not by work: one W^2 of L=256 went from four
 // kernels and two copies (33 us with the wait) to two kernels (17 us), and the
 // W^2 of 256 replicas (L = 64..2048, 375 M sites) from 256 such calls (8.3 ms)
-// to 0.5 ms.
+// to 0.5 ms.  Both launches overlap the one before them: the tables are
+// filled during the last device step (8 MCS of L=256 and their W^2: 132 to
+// 128 us).
 constexpr int kW2SmallThreads = 512;  // of the second launch
 
 // Words j .. j+3 of the lane's nw, as one 16-byte load where allowed.
@@ -479,8 +482,21 @@ __device__ __forceinline__ void load_quad(const uint32_t *row, uint32_t j, uint3
     }
 }
 
+// A job list passed by value; the kernels read it where no list in device
+// memory is given.  Asynchronous measurements take it: a copy to the device
+// would need staging that outlives the call.  Up to 32 lattices (2.8 KB of the
+// 4 KB of arguments) share two launches; one by one the device idled in each:
+// 24 served jobs with 192 W^2 went from 8.75 to 6.9 ms.
+template <uint32_t N>
+struct W2Pack {
+    W2Job j[N];
+};
+
+template <uint32_t N>
 __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
-    w2_small_rows_kernel(const __grid_constant__ W2Job one, const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows) {
+    w2_small_rows_kernel(const __grid_constant__ W2Pack<N> pack, const W2Job *jobs, uint32_t n, uint32_t n_tasks,
+                         W2RowSums *rows) {
+    launch_dependents();
     extern __shared__ __align__(16) unsigned char w2_table[];
     for (int i = threadIdx.x; i < 256; i += blockDim.x) {
         const uint2 e = byte_entry(static_cast<uint32_t>(i));
@@ -488,18 +504,17 @@ __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
         for (int c = 0; c < 16; ++c) *reinterpret_cast<uint2 *>(w2_table + 256 * i + 8 * c) = e;
     }
     __syncthreads();
+    wait_for_previous_grid();  // the table needs nothing of it
+    const W2Job *list = jobs ? jobs : pack.j;
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t slot = 8u * (lane & 15u);
     for (uint32_t task = blockIdx.x * kW2Warps + (threadIdx.x >> 5); task < n_tasks; task += gridDim.x * kW2Warps) {
-        const W2Job *J = &one;
-        if (jobs) {  // the last job whose first task is not past this one
-            uint32_t a = 0, b = n;
-            while (b - a > 1u) {
-                const uint32_t m = (a + b) >> 1;
-                if (jobs[m].task_first <= task) a = m; else b = m;
-            }
-            J = jobs + a;
+        uint32_t a0 = 0, b0 = n;  // the last job whose first task is not past this one
+        while (b0 - a0 > 1u) {
+            const uint32_t m = (a0 + b0) >> 1;
+            if (list[m].task_first <= task) a0 = m; else b0 = m;
         }
+        const W2Job *J = list + a0;
         const uint32_t wpr = J->L >> 5, nrows = J->nrows, lw = 1u << J->lw_log, sl = 1u << J->sl_log;
         const uint32_t y = ((task - J->task_first) << (5u - J->sl_log)) + (lane >> J->sl_log);
         const uint32_t li = lane & (sl - 1u), w = li * lw;
@@ -555,13 +570,15 @@ __global__ void __launch_bounds__(kW2Warps * 32, kW2BlocksPerSM)
 }
 
 // Pass 2: one block per lattice, a run of consecutive rows per thread.
+template <uint32_t N>
 __global__ void __launch_bounds__(kW2SmallThreads)
-    w2_small_finish_kernel(const __grid_constant__ W2Job one, const W2Job *jobs, const W2RowSums *all_rows) {
+    w2_small_finish_kernel(const __grid_constant__ W2Pack<N> pack, const W2Job *jobs, const W2RowSums *all_rows) {
+    wait_for_previous_grid();
     constexpr int kWarps = kW2SmallThreads / 32;
     __shared__ int wsum[kWarps];
     __shared__ long long red[6][kWarps];
     __shared__ long long last_h;
-    const W2Job &J = jobs ? jobs[blockIdx.x] : one;
+    const W2Job &J = (jobs ? jobs : pack.j)[N > 1u || jobs ? blockIdx.x : 0u];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t nrows = J.nrows;
     const W2RowSums *rows = all_rows + J.row_first;
@@ -718,7 +735,7 @@ __global__ void __launch_bounds__(kNetSlots)
 cudaError_t table_kernel_setup(const void *kernel, int which, int *sm_count) {
     constexpr int kMaxDevices = 64;
     static int sms[kMaxDevices] = {};
-    static bool smem_set[2][kMaxDevices] = {};
+    static bool smem_set[3][kMaxDevices] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -736,17 +753,18 @@ cudaError_t table_kernel_setup(const void *kernel, int which, int *sm_count) {
     return cudaSuccess;
 }
 
-cudaError_t w2_small(const W2Job &one, const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows,
+template <uint32_t N>
+cudaError_t w2_small(const W2Pack<N> &pack, const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows,
                      cudaStream_t st) {
     int sms = 0;
-    cudaError_t e = table_kernel_setup(reinterpret_cast<const void *>(w2_small_rows_kernel), 1, &sms);
+    cudaError_t e = table_kernel_setup(reinterpret_cast<const void *>(w2_small_rows_kernel<N>), N > 1u ? 2 : 1, &sms);
     if (e != cudaSuccess) return e;
     const uint32_t want = (n_tasks + kW2Warps - 1) / kW2Warps, wave = static_cast<uint32_t>(sms) * kW2BlocksPerSM;
-    w2_small_rows_kernel<<<std::min(want, wave), kW2Warps * 32, kW2TableBytes, st>>>(one, jobs, n, n_tasks, rows);
-    e = cudaGetLastError();
+    e = launch_overlapped_smem(w2_small_rows_kernel<N>, dim3(std::min(want, wave)), dim3(kW2Warps * 32), kW2TableBytes,
+                               true, st, pack, jobs, n, n_tasks, rows);
     if (e != cudaSuccess) return e;
-    w2_small_finish_kernel<<<n, kW2SmallThreads, 0, st>>>(one, jobs, rows);
-    return cudaGetLastError();
+    return launch_overlapped(w2_small_finish_kernel<N>, dim3(n), dim3(kW2SmallThreads), true, st, pack, jobs,
+                             static_cast<const W2RowSums *>(rows));
 }
 
 int grid_for(uint64_t n, int threads) {
@@ -781,7 +799,7 @@ cudaError_t launch_w2_rows(const uint32_t *lat, uint32_t L, uint32_t nrows, uint
         j.nrows = nrows;
         j.plane_rows = plane_rows;
         j.res = out;
-        return launch_w2_small_one(j, rows, st);
+        return launch_w2_small_pack(&j, 1, rows, st);
     }
     // one wave of resident blocks (64 KB of table each), rows taken grid-stride
     int sms = 0;
@@ -827,12 +845,17 @@ uint32_t w2_small_split(W2Job *jobs, uint32_t n) {
 }
 
 cudaError_t launch_w2_small(const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows, cudaStream_t st) {
-    return w2_small(W2Job{}, jobs, n, n_tasks, rows, st);
+    return w2_small(W2Pack<1>{}, jobs, n, n_tasks, rows, st);
 }
 
-cudaError_t launch_w2_small_one(W2Job job, W2RowSums *rows, cudaStream_t st) {
-    const uint32_t n_tasks = w2_small_split(&job, 1);
-    return w2_small(job, nullptr, 1, n_tasks, rows, st);
+cudaError_t launch_w2_small_pack(W2Job *jobs, uint32_t n, W2RowSums *rows, cudaStream_t st) {
+    if (n == 0 || n > kW2PackJobs) return cudaErrorInvalidValue;
+    const uint32_t n_tasks = w2_small_split(jobs, n);
+    const W2Job *none = nullptr;
+    if (n == 1) return w2_small(W2Pack<1>{{jobs[0]}}, none, 1, n_tasks, rows, st);
+    W2Pack<kW2PackJobs> pack{};
+    std::copy(jobs, jobs + n, pack.j);
+    return w2_small(pack, none, n, n_tasks, rows, st);
 }
 
 cudaError_t launch_pack_canonical(const uint32_t *lat, uint32_t L, uint32_t cy0, uint32_t ncy,

@@ -108,8 +108,9 @@ uint32_t w2_small_split(W2Job *jobs, uint32_t n);
 // The exact sums of n lattices (sides up to kW2SmallL) in two launches.
 // jobs: the same list in device memory; rows: one record per row of them all.
 cudaError_t launch_w2_small(const W2Job *jobs, uint32_t n, uint32_t n_tasks, W2RowSums *rows, cudaStream_t st);
-// The same for one lattice, passed by value.
-cudaError_t launch_w2_small_one(W2Job job, W2RowSums *rows, cudaStream_t st);
+// The same for a list in host memory, passed by value (n <= kW2PackJobs); fills its split.
+constexpr uint32_t kW2PackJobs = 32;
+cudaError_t launch_w2_small_pack(W2Job *jobs, uint32_t n, W2RowSums *rows, cudaStream_t st);
 
 cudaError_t launch_w2(const uint32_t *lat, uint32_t L, W2RowSums *rows, W2Result *out,
                       cudaStream_t st);

@@ -12,11 +12,12 @@ __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontr
 __device__ __forceinline__ void wait_for_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <class... Params, class... Args>
-cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, bool overlap, cudaStream_t st,
-                              const Args &...args) {
+cudaError_t launch_overlapped_smem(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, bool overlap,
+                                   cudaStream_t st, const Args &...args) {
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = grid;
     cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -24,6 +25,12 @@ cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, 
     cfg.attrs = attr;
     cfg.numAttrs = overlap ? 1u : 0u;
     return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <class... Params, class... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, bool overlap, cudaStream_t st,
+                              const Args &...args) {
+    return launch_overlapped_smem(kernel, grid, block, 0, overlap, st, args...);
 }
 
 }  // namespace oct

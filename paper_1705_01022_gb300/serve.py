@@ -16,7 +16,8 @@ job, since it is part of the job's dynamics):
   fewest running sites), so their launches overlap too;
 * at a job's measurement times its exact W^2 is computed on the device and
   handed to the ``on_result`` callback (streamed back).  With a batch that
-  measures asynchronously (``measure_async`` / ``poll``), the reduction is
+  measures asynchronously (``measure_async`` / ``poll``; ``measure_async_many``
+  takes all the jobs due at a tick in one call), the reduction is
   enqueued behind the job's MCS and the result delivered when it is done, so
   the host never waits for the device between ticks;
 * a job that reaches t_max leaves the batch and returns its memory; its
@@ -221,17 +222,24 @@ class ServingEngine:
         n = self._chunk(bi)
         batch.run(n)
         self.ticks += 1
+        if self.async_measure:
+            # the measurements due now, together: a W^2 of a few rows leaves the device nearly idle
+            due = [(job, slot) for (b, slot), job in self.running.items()
+                   if b == bi and job.t + n in job.measure_at]
+            slots = [slot for _, slot in due]
+            if hasattr(batch, "measure_async_many"):
+                tickets = batch.measure_async_many(slots)
+            else:
+                tickets = [batch.measure_async(slot) for slot in slots]
+            self.pending.extend((job, bi, ticket) for (job, _), ticket in zip(due, tickets))
         for (b, slot), job in list(self.running.items()):
             if b != bi:
                 continue
             job.t += n
             self.mcs_attempts += n * job.L * job.L
             last = job.t >= job.t_max
-            if job.t in job.measure_at:
-                if self.async_measure:
-                    self.pending.append((job, bi, batch.measure_async(slot)))
-                else:
-                    self._deliver_one(job, batch.measure(slot), now)
+            if job.t in job.measure_at and not self.async_measure:
+                self._deliver_one(job, batch.measure(slot), now)
             if last:
                 batch.remove(slot)
                 del self.running[(bi, slot)]
@@ -376,6 +384,11 @@ class GpuBatch:
 
     def measure_async(self, slot: int) -> int:
         return self._lib.oct_batch_measure_async(self.h, slot)
+
+    def measure_async_many(self, slots) -> list:
+        # a call takes at most 1024 (_lib's ring of tickets)
+        return [t for i in range(0, len(slots), 1024)
+                for t in self._lib.oct_batch_measure_slots_async(self.h, slots[i:i + 1024])]
 
     def mark(self) -> int:
         return self._lib.oct_batch_mark(self.h)
