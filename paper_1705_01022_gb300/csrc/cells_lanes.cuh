@@ -386,18 +386,14 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
 template <int CX, int CY, bool RANDOM, int SPEC>
 cudaError_t launch_lane_cells(const StepArgs &a, const LaneSplit &q, cudaStream_t st) {
     const uint32_t warps = (work_tiles(a) + q.pk - 1u) / q.pk, smem = kStepWarpsPerBlock * q.bytes;
-    constexpr int kMaxDevices = 64;
-    static uint32_t limit[kMaxDevices] = {};  // dynamic shared memory allowed so far
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
+    // The limit is that of the largest sub-tile for every launch: threads that
+    // run different sub-tiles may pass here at the same time.
+    using C = LaneCells<CX, CY>;
+    const uint32_t most = kStepWarpsPerBlock * lane_split<CX, CY, RANDOM>(1u, C::NCMAX * C::GPI * 4u * CY).bytes;
+    if (smem > most) return cudaErrorInvalidValue;
+    cudaError_t e = cudaFuncSetAttribute(lane_cells_kernel<CX, CY, RANDOM, SPEC>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
     if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    if (smem > limit[dev]) {
-        e = cudaFuncSetAttribute(lane_cells_kernel<CX, CY, RANDOM, SPEC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-        limit[dev] = smem;
-    }
     lane_cells_kernel<CX, CY, RANDOM, SPEC><<<(warps + kStepWarpsPerBlock - 1) / kStepWarpsPerBlock,
                                               kStepWarpsPerBlock * 32, smem, st>>>(a, q);
     return cudaSuccess;

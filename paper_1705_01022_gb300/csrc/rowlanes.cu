@@ -129,8 +129,10 @@ cudaError_t launch_row_step_as(const StepArgs &a, bool overlap, cudaStream_t st)
 template <bool RANDOM, int SPEC, bool ONE>
 cudaError_t launch_row_run_as(const StepArgs &a, uint32_t *t_out, uint32_t n, cudaStream_t st) {
     const uint32_t warps = row_warps(a), smem = a.L * a.wpr * 8u + warps * row_smem_words<RANDOM>() * 4u;
+    // the same limit for every launch: threads that run other sizes may pass here at the same time
+    constexpr uint32_t kMost = kBlockLattice + kBlockWarps * row_smem_words<RANDOM>() * 4u;
     cudaError_t e = cudaFuncSetAttribute(row_block_kernel<RANDOM, SPEC, ONE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMost));
     if (e != cudaSuccess) return e;
     row_block_kernel<RANDOM, SPEC, ONE><<<1, warps * 32u, smem, st>>>(a, t_out, n);
     return cudaGetLastError();

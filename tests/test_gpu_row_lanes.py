@@ -1,6 +1,5 @@
 """The device step of small lattices (one TC row per lane) against the oracle's
-replay: lattices held by one block, by a cluster and stepped by overlapping
-launches; sub-tiles that share a warp or fill it, with one and several band
+replay: lattices held by one block and stepped by overlapping launches; sub-tiles that share a warp or fill it, with one and several band
 columns, and a ragged last warp; draws on both, one or no rate."""
 import numpy as np
 import pytest
@@ -16,8 +15,8 @@ def g():
 
 
 SHAPES = [(64, 32, 16), (128, 64, 64), (192, 32, 32), (256, 64, 64), (384, 64, 16), (448, 32, 16),  # one block
-          (576, 32, 32), (640, 64, 64), (1024, 32, 128), (1024, 128, 32),                           # a cluster
-          (1088, 32, 16), (1152, 64, 64), (1088, 32, 32), (1280, 64, 32)]                           # launches
+          (576, 32, 32), (640, 64, 64), (1024, 32, 128), (1024, 128, 32),                           # launches of one-warp blocks
+          (1088, 32, 16), (1152, 64, 64), (1088, 32, 32), (1280, 64, 32)]
 
 
 @pytest.mark.parametrize("p,q", [(0.95, 0.05), (1.0, 0.0), (0.6, 0.0), (1.0, 0.5), (1.0, 1.0)])
@@ -83,3 +82,36 @@ def test_device_steps_equal_a_run(g):
             _lib.oct_end_mcs(b.h)
         assert np.array_equal(a.planes(), b.planes())
         assert a.measure().net_flips == b.measure().net_flips
+
+
+def test_threads_with_different_sizes(g):
+    """Threads on streams of their own, whose sizes and cells need different
+    shared memory of the same kernels, get what each gets alone."""
+    import threading
+
+    import torch
+    cases = [(64, 4, 4), (256, 4, 4), (512, 4, 4), (128, 8, 8), (512, 8, 8), (1024, 8, 8)]
+
+    def once(L, cx, cy):
+        with g.Simulation(L, 0.95, 0.05, L, cx=cx, cy=cy, stream=torch.cuda.Stream()) as sim:
+            for _ in range(4):
+                sim.run(1)
+            return np.array(sim.lattice())
+
+    want = [once(*c) for c in cases]
+    bad = []
+
+    def loop(i):
+        try:
+            for _ in range(10):
+                if not np.array_equal(once(*cases[i]), want[i]):
+                    bad.append(cases[i])
+        except Exception as e:
+            bad.append((cases[i], e))
+
+    threads = [threading.Thread(target=loop, args=(i,)) for i in range(len(cases))]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    assert not bad
