@@ -266,6 +266,48 @@ __device__ __forceinline__ uint32_t gather_lsb(const uint32_t (&f)[16]) {
     return v >> 16;
 }
 
+// Constants that the compiler does not know (see opaque_one), for the additive
+// flips of a step.
+struct FlipConsts {
+    uint32_t one, neg, c16;
+    __device__ __forceinline__ FlipConsts() : one(opaque_one()) {
+        neg = 0u - one;
+        asm volatile("mov.u32 %0, 16;" : "=r"(c16));
+    }
+};
+// floor(a b / 2^32) + c
+__device__ __forceinline__ uint32_t mad_hi_signed(uint32_t a, uint32_t b, uint32_t c) {
+    int r;
+    asm("mad.hi.s32 %0, %1, %2, %3;"
+        : "=r"(r)
+        : "r"(static_cast<int>(a)), "r"(static_cast<int>(b)), "r"(static_cast<int>(c)));
+    return static_cast<uint32_t>(r);
+}
+// Signed flips of a row: a candidate f has X(s) != X(s+x), Y(s) != Y(s+y) and
+// X(s) == Y(s), so a minimum (X(s) = 0) takes 2^s from the row's X, adds it to Y(s)
+// and takes it from Y(s+y), and a maximum does the opposite: with h = +-f a flip is
+// a few multiply-adds, where exclusive ors would run on the integer pipe that binds
+// the step (77 % of its rate on packed warps, the FMA pipe 20 %), and a row offset per lane
+// is a factor 0 or 1 in place of masks.  Column 31 works modulo 2^32.  One MCS at L=19456 in
+// 64 x 64 sub-tiles, p=0.95, q=0.05: 326 to 308 us, KPZ 201 to 178 us (with the
+// candidates' columns and packed bits by multiply-adds too, 2.8 and 1.7 % of it); on full
+// warps KPZ at L=32768 350 to 343 us, L=2^17 with draws 9.45 to 9.36 ms.
+template <int SPEC>
+__device__ __forceinline__ uint32_t signed_flips(uint32_t f, uint32_t x) {
+    return SPEC == 1 ? f : f - 2u * (f & x);
+}
+// The changes that flips at column 31 of the left lane make to column 0: v has
+// their bits at 4m + I (m: TC row), e0 the column's own bits there.  Field m
+// of the word, 4 bits from bit 4m + I on, is -1 or +1 (0 without a flip);
+// column_fields moves field m to the top (m = 3 first), and mad_hi_signed of it
+// with 16 adds it.
+template <int SPEC, int I, bool NEGATE>
+__device__ __forceinline__ uint32_t column_fields(uint32_t v, uint32_t e0) {
+    const uint32_t b = v & (0x1111u << I);
+    const uint32_t w = SPEC == 1 ? (NEGATE ? b : b * 15u) : b + 14u * (NEGATE ? b & ~e0 : b & e0);
+    return w << (16 - I);
+}
+
 // A collective step runs in three phases: the candidates of every thread
 // cell of the lane (specialised on the set's row offset dy), the acceptance
 // draws (one copy of the code, shared by both offsets), and the flips with
@@ -335,7 +377,7 @@ __device__ __forceinline__ void step_candidates(const uint32_t (&X)[16], const u
 template <int DY, bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_apply(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                            uint32_t dx, uint32_t acc, const uint32_t (&cnd0)[4],
-                                           const uint32_t (&cnd1)[4], const Ctx &c, int &net) {
+                                           const uint32_t (&cnd1)[4], const Ctx &c, const FlipConsts &k, int &net) {
     uint32_t f0s[4], f1s[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -361,16 +403,15 @@ __device__ __forceinline__ void step_apply(uint32_t (&X)[16], uint32_t (&Y)[16],
             f1 = cnd1[m] & ((~xb & amin) | (xb & amax));
             net += always_net<RANDOM>(f0, xa, c) + always_net<RANDOM>(f1, xb, c);
         }
-        // f ^ (f << 1) = 3f: a cell flips at most one site, so flips are at
-        // least three columns apart and the sum has no carries (FMA pipe)
-        X[r0] = xa ^ (f0 * 3u);
-        X[r1] = xb ^ (f1 * 3u);
-        Y[r0] ^= f0;
-        Y[r1] ^= f0 ^ f1;
+        const uint32_t h0 = signed_flips<SPEC>(f0, xa), h1 = signed_flips<SPEC>(f1, xb);
+        X[r0] = h0 * k.neg + xa;
+        X[r1] = h1 * k.neg + xb;
+        Y[r0] = h0 * k.one + Y[r0];
+        Y[r1] = h1 * k.one + (h0 * k.neg + Y[r1]);
         if (r1 + 1 < 16)
-            Y[(r1 + 1) & 15] ^= f1;
+            Y[(r1 + 1) & 15] = h1 * k.neg + Y[(r1 + 1) & 15];
         else
-            D ^= f1;
+            D = h1 * k.neg + D;
         f0s[m] = f0;
         f1s[m] = f1;
     }
@@ -380,8 +421,19 @@ __device__ __forceinline__ void step_apply(uint32_t (&X)[16], uint32_t (&Y)[16],
         // Flips at bit 31 changed column 0 of the right neighbour (this lane's E).
         const uint32_t dE = gather_msb_pairs(f0s, f1s) >> (DY ? 0 : 2);
         E ^= dE;
-        const uint32_t v = __shfl_up_sync(kFull, dE, 1);
-        if (c.gx > 0) {
+        uint32_t v = __shfl_up_sync(kFull, dE, 1);
+        if (SPEC == 1) {
+            v = c.gx > 0 ? v >> (2 * DY) : 0u;
+            uint32_t w0 = column_fields<1, 0, false>(v, 0u), w1 = column_fields<1, 1, false>(v, 0u);
+#pragma unroll
+            for (int m = 3; m >= 0; --m) {
+                const int r0 = 4 * m + 2 * DY, r1 = r0 + 1;
+                X[r0] = mad_hi_signed(w0, k.c16, X[r0]);
+                X[r1] = mad_hi_signed(w1, k.c16, X[r1]);
+                w0 *= k.c16;
+                w1 *= k.c16;
+            }
+        } else if (c.gx > 0) {  // the signs cost more here than the multiply-adds save
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
                 const int r0 = 4 * m + 2 * DY, r1 = r0 + 1;
@@ -416,24 +468,25 @@ __device__ __forceinline__ void step_candidates_rt(const uint32_t (&X)[16], cons
                                                    uint32_t dx, uint32_t dy, const Ctx &c,
                                                    uint32_t (&cnd0)[4], uint32_t (&cnd1)[4],
                                                    uint32_t &pmin, uint32_t &pmax) {
-    const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
-    const uint32_t sh2 = 2u * dx;  // site words: shifted to the step's field by run_subtile
-    const uint32_t ro = 2u * dy;
+    const uint32_t sw[4] = {site.x, site.y, site.z, site.w};  // shifted to the step's field by run_subtile
+    // column factor of the set, and the one that brings a candidate's cell to bit 4j+3
+    // (the cell's one candidate lies at bit 4j + 2dx + xoff; no carries)
+    const uint32_t cs = dx ? 4u : 1u, ps = dx ? 3u : 12u, kc = dx ? kNib * 4u : kNib;
+    const uint32_t Es = E >> (2u * dy);
     pmin = 0u;
     pmax = 0u;
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         const uint32_t u = sw[m];
-        const uint32_t col = ((u & kNib) + kNib) << sh2;  // 1 + xoff: one-hot, no carries
+        const uint32_t col = (u & kNib) * cs + kc;  // 1 + xoff: one-hot, no carries
         const uint32_t yoff = ((u >> 1) & kNib) * 0xFu;
         const uint32_t xa = dy ? X[4 * m + 2] : X[4 * m];
         const uint32_t xb = dy ? X[4 * m + 3] : X[4 * m + 1];
         const uint32_t ya = dy ? Y[4 * m + 2] : Y[4 * m];
         const uint32_t yb = dy ? Y[4 * m + 3] : Y[4 * m + 1];
         const uint32_t yc = dy ? (m < 3 ? Y[(4 * m + 4) & 15] : D) : Y[4 * m + 2];
-        const uint32_t r0 = 4u * m + ro;
-        const uint32_t xra = __funnelshift_r(xa, E >> r0, 1);
-        const uint32_t xrb = __funnelshift_r(xb, E >> (r0 + 1u), 1);
+        const uint32_t xra = __funnelshift_r(xa, Es >> (4 * m), 1);
+        const uint32_t xrb = __funnelshift_r(xb, Es >> (4 * m + 1), 1);
         if (SPEC == 1) {
             cnd0[m] = col & ~yoff & ~xa & xra & ~ya & yb;  // the minima
             cnd1[m] = col & yoff & ~xb & xrb & ~yb & yc;
@@ -442,22 +495,24 @@ __device__ __forceinline__ void step_candidates_rt(const uint32_t (&X)[16], cons
         cnd0[m] = col & ~yoff & (xa ^ xra) & (ya ^ yb) & ~(xa ^ ya);
         cnd1[m] = col & yoff & (xb ^ xrb) & (yb ^ yc) & ~(xb ^ yb);
         if (RANDOM) {
-            const uint32_t mn = (cnd0[m] & ~xa) | (cnd1[m] & ~xb);
             const uint32_t mx = (cnd0[m] & xa) | (cnd1[m] & xb);
+            const uint32_t mn = SPEC == 2 ? cnd0[m] | cnd1[m] : (cnd0[m] & ~xa) | (cnd1[m] & ~xb);
             const uint32_t cmn = SPEC == 2 ? mn : mn & c.p_random, cmx = SPEC == 2 ? mx : mx & c.q_random;
-            pmin |= (((cmn * 3u) >> (sh2 + 1u)) & kNib) << m;  // see step_candidates
-            pmax |= (((cmx * 3u) >> (sh2 + 1u)) & kNib) << m;
+            pmin = ((cmn * ps) & (kNib << 3)) | (pmin >> 1);
+            pmax = ((cmx * ps) & (kNib << 3)) | (pmax >> 1);
         }
     }
+    if (RANDOM && SPEC == 2) pmin &= ~pmax;  // pmin held every candidate: keep the minima
 }
 
 template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                               uint32_t dy, uint32_t acc, const uint32_t (&cnd0)[4],
-                                              const uint32_t (&cnd1)[4], const Ctx &c, int &net) {
+                                              const uint32_t (&cnd1)[4], const Ctx &c, const FlipConsts &k, uint32_t &E0,
+                                              int &net) {
     const uint32_t ro = 2u * dy;
-    const uint32_t dym = dy ? 0xFFFFFFFFu : 0u;
-    uint32_t dD = 0, dY0 = 0;
+    // the factors with which a flip counts in the rows of one offset and the other
+    const uint32_t B = dy, A = 1u - dy, nB = 0u - B, nA = 0u - A;
     uint32_t g0[4], g1[4], f0s[4], f1s[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
@@ -467,7 +522,11 @@ __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[1
             amin |= spread & c.p_random;
             amax |= spread & c.q_random;
         }
-        uint32_t f0, f1;
+        uint32_t f0, f1, xa = 0u, xb = 0u;
+        if (SPEC != 1) {
+            xa = dy ? X[4 * m + 2] : X[4 * m];
+            xb = dy ? X[4 * m + 3] : X[4 * m + 1];
+        }
         if (SPEC == 1) {
             f0 = cnd0[m];
             f1 = cnd1[m];
@@ -476,28 +535,26 @@ __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[1
             f0 = cnd0[m] & spread;
             f1 = cnd1[m] & spread;
         } else {
-            const uint32_t xa = dy ? X[4 * m + 2] : X[4 * m];
-            const uint32_t xb = dy ? X[4 * m + 3] : X[4 * m + 1];
             f0 = cnd0[m] & ((~xa & amin) | (xa & amax));
             f1 = cnd1[m] & ((~xb & amin) | (xb & amax));
             net += always_net<RANDOM>(f0, xa, c) + always_net<RANDOM>(f1, xb, c);
         }
-        g0[m] = f0 * 3u;  // 3f = f ^ (f << 1), see step_apply; applied after the exchange
-        g1[m] = f1 * 3u;
-        const uint32_t f01 = f0 ^ f1;
-        Y[4 * m] ^= f0 & ~dym;
-        Y[4 * m + 1] ^= f01 & ~dym;
-        Y[4 * m + 2] ^= (f0 & dym) | (f1 & ~dym);
-        Y[4 * m + 3] ^= f01 & dym;
+        const uint32_t h0 = signed_flips<SPEC>(f0, xa), h1 = signed_flips<SPEC>(f1, xb);
+        const uint32_t h = h0 * k.neg + h1;
+        Y[4 * m] = h0 * A + Y[4 * m];
+        Y[4 * m + 1] = h * A + Y[4 * m + 1];
+        Y[4 * m + 2] = h0 * B + (h1 * nA + Y[4 * m + 2]);
+        Y[4 * m + 3] = h * B + Y[4 * m + 3];
         if (m < 3)
-            Y[(4 * m + 4) & 15] ^= f1 & dym;
+            Y[(4 * m + 4) & 15] = h1 * nB + Y[(4 * m + 4) & 15];
         else
-            D ^= f1 & dym;
+            D = h1 * nB + D;
+        g0[m] = h0;  // the changes of X are applied after the exchange
+        g1[m] = h1;
         f0s[m] = f0;
         f1s[m] = f1;
-        if (m == 3) dD = f1 & dym;
-        if (m == 0) dY0 = f0 & ~dym;
     }
+    const uint32_t dD = f1s[3] * B, dY0 = f0s[0] * A;
     uint32_t dE = gather_msb_pairs(f0s, f1s) >> 2;
     if (c.GX > 1) {  // warp-uniform: every sub-tile of a warp has the same shape
         dE <<= ro;
@@ -505,11 +562,16 @@ __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[1
         E ^= dE;
         uint32_t vr = __shfl_up_sync(kFull, dE, 1);
         const uint32_t vl = __shfl_down_sync(kFull, dB0, 1);
-        vr = c.gx > 0 ? (vr >> ro) : 0u;  // the left lane is in the same sub-tile: same row offset
+        vr = c.gx > 0 ? vr : 0u;  // the left lane is in the same sub-tile: same row offset
+        const uint32_t vs = vr >> ro, es = E0 >> ro;
+        uint32_t w0 = column_fields<SPEC, 0, true>(vs, es), w1 = column_fields<SPEC, 1, true>(vs, es);
+        if (SPEC != 1) E0 ^= vr ^ dB0;
 #pragma unroll
-        for (int m = 0; m < 4; ++m) {
-            g0[m] ^= (vr >> (4 * m)) & 1u;
-            g1[m] ^= (vr >> (4 * m + 1)) & 1u;
+        for (int m = 3; m >= 0; --m) {
+            g0[m] = mad_hi_signed(w0, k.c16, g0[m]);
+            g1[m] = mad_hi_signed(w1, k.c16, g1[m]);
+            w0 *= k.c16;
+            w1 *= k.c16;
         }
         if (c.gx < c.GX - 1) E ^= vl;
     } else {
@@ -517,10 +579,10 @@ __device__ __forceinline__ void step_apply_rt(uint32_t (&X)[16], uint32_t (&Y)[1
     }
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
-        X[4 * m] ^= g0[m] & ~dym;
-        X[4 * m + 1] ^= g1[m] & ~dym;
-        X[4 * m + 2] ^= g0[m] & dym;
-        X[4 * m + 3] ^= g1[m] & dym;
+        X[4 * m] = g0[m] * nA + X[4 * m];
+        X[4 * m + 1] = g1[m] * nA + X[4 * m + 1];
+        X[4 * m + 2] = g0[m] * nB + X[4 * m + 2];
+        X[4 * m + 3] = g1[m] * nB + X[4 * m + 3];
     }
     const uint32_t vd = __shfl_up_sync(kFull, dD, c.GX);
     const uint32_t vu = __shfl_down_sync(kFull, dY0, c.GX);
@@ -1290,6 +1352,10 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
     const bool straight = lane_straight(q, L, active);
     stage_lane(q, L, wpr, straight, active, X, Y, E, D);
 
+    const FlipConsts flips;
+    uint32_t E0 = 0u;  // X bits of the lane's own column 0 (for column_fields)
+    if (LANE_SETS && (SCHEME == 0 || SCHEME == 5)) E0 = gather_lsb(X);
+
     // Block layer: 16 single-hit collective steps.
     const uint4 setw = c.draw(c.k, kTagSet << 28);
     uint4 site = make_uint4(0u, 0u, 0u, 0u);
@@ -1360,11 +1426,11 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             net += random_net(acc, pmin, pmax);
         }
         if (LANE_SETS)
-            step_apply_rt<RANDOM, kSpec>(X, Y, E, D, d >> 1, acc, cnd0, cnd1, c, net);
+            step_apply_rt<RANDOM, kSpec>(X, Y, E, D, d >> 1, acc, cnd0, cnd1, c, flips, E0, net);
         else if (d & 2u)
-            step_apply<1, RANDOM, kSpec>(X, Y, E, D, d & 1u, acc, cnd0, cnd1, c, net);
+            step_apply<1, RANDOM, kSpec>(X, Y, E, D, d & 1u, acc, cnd0, cnd1, c, flips, net);
         else
-            step_apply<0, RANDOM, kSpec>(X, Y, E, D, d & 1u, acc, cnd0, cnd1, c, net);
+            step_apply<0, RANDOM, kSpec>(X, Y, E, D, d & 1u, acc, cnd0, cnd1, c, flips, net);
     }
 
     launch_dependents();  // the next step's head overlaps this one's write-back
