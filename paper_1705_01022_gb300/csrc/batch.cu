@@ -63,7 +63,7 @@ constexpr int kBatchBlocksPerSM = 4;
 // LANE_SETS: the warp holds several sub-tiles (fewer than 32 groups each), each
 // with its own set draws; otherwise one sub-tile fills the warp and the step
 // takes the uniform row-offset path of the plain kernel.
-// SCHEME: 0 DTrDT, 4 with deposition only (p = 1, q = 0), 5 with both rates
+// SCHEME: 0 DTrDT, 4 with deposition only (p = 1, q = 0), 10 with both rates
 // strictly inside (0, 1) (the step variants of the plain kernel).
 template <bool RANDOM, bool LANE_SETS, int SCHEME>
 __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
@@ -203,12 +203,12 @@ __global__ void __launch_bounds__(32)
         if (wd.kpz)
             batch_row_item<false, 1, true>(R, wd, it.T, held, t, k, sm);
         else
-            batch_row_item<true, 0, true>(R, wd, it.T, held, t, k, sm);
+            batch_row_item<true, -1, true>(R, wd, it.T, held, t, k, sm);
     } else {
         if (wd.kpz)
             batch_row_item<false, 1, false>(R, wd, it.T, held, t, k, sm);
         else
-            batch_row_item<true, 0, false>(R, wd, it.T, held, t, k, sm);
+            batch_row_item<true, -1, false>(R, wd, it.T, held, t, k, sm);
     }
 }
 
@@ -679,8 +679,8 @@ cudaError_t enqueue_branch_step(oct_batch *b, uint32_t k, int br, cudaStream_t s
         case 1: OCT_BATCH(false, false, 0); break;
         case 2: OCT_BATCH(true, true, 0); break;
         case 3: OCT_BATCH(true, false, 0); break;
-        case 4: OCT_BATCH(true, true, 5); break;
-        case 5: OCT_BATCH(true, false, 5); break;
+        case 4: OCT_BATCH(true, true, 10); break;
+        case 5: OCT_BATCH(true, false, 10); break;
         case 6: OCT_BATCH(false, true, 4); break;
         default: OCT_BATCH(false, false, 4); break;
     }

@@ -173,7 +173,7 @@ __device__ __forceinline__ void cells_candidates(const uint32_t (&X)[16], const 
         q.low[i] = ~xs;
         uint32_t mn = cd & ~xs, mx = cd & xs;
         if (RANDOM) {
-            if (SPEC != 2) {
+            if (SPEC < 2) {
                 mn &= cc.c.p_random;
                 mx &= cc.c.q_random;
             }
@@ -191,7 +191,7 @@ __device__ __forceinline__ void cells_candidates(const uint32_t (&X)[16], const 
 // Phase 2: acceptance of the lane's packed candidates (bit 4j+m), as in
 // accept_candidates, for groups that span GS lane rows: a tied candidate's
 // word in its group's tail stream is ranked among the ties of the whole group.
-template <int GS>
+template <int GS, int TIES>
 __device__ __forceinline__ uint32_t cells_accept(uint32_t pmin, uint32_t pmax, const uint4 &W, const CellCtx &cc,
                                                  TailPool &tp) {
     const LaneCtx<KeysConst> &c = cc.c;
@@ -204,6 +204,7 @@ __device__ __forceinline__ uint32_t cells_accept(uint32_t pmin, uint32_t pmax, c
         acc |= und & tb & ~lw[i];
         und &= ~(tb ^ lw[i]);
     }
+    if (TIES == kTiesRefused) return acc;
     // ties of the lane's whole group (its GS lane rows)
     uint32_t gund = und;
     if (GS > 1) {
@@ -220,7 +221,7 @@ __device__ __forceinline__ uint32_t cells_accept(uint32_t pmin, uint32_t pmax, c
     // The group's ties take the next words of its tail stream in order of
     // position; every lane of the group keeps the group's stream in its own
     // slot, so that it finds the words of its own ties there.
-    if (__all_sync(kFull, gund == 0u)) return acc;
+    if (__all_sync(kFull, gund == 0u || (TIES == kTiesAsk && !ties_matter(c.thr_p, c.thr_q)))) return acc;
     const uint32_t ng = static_cast<uint32_t>(__popc(gund));
     tail_refill(ng, c.g, c, tp);
     // (w >> 4) < (P32 mod 2^28)  <=>  w < 16 (P32 mod 2^28)
@@ -270,7 +271,7 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
 #pragma unroll
             for (int v = 0; v < S::UY; ++v) any |= F[v] = q.flip[i * S::UY + v];
             net += __popc(any);  // one flip per cell
-        } else if (SPEC == 2) {
+        } else if (SPEC >= 2) {
             F[0] = q.cand[i] & spread;
         } else {
             F[0] = q.cand[i] & ((q.low[i] & amin) | (~q.low[i] & amax));
@@ -386,7 +387,7 @@ __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uin
             const uint4 lvl = lvl_w[(s % S::DRAW) / S::SPL * 32 + g_at];
             const uint32_t sh = (s % S::SPL) * 4u * S::TPB;  // this step's positions
             const uint4 W = make_uint4(lvl.x >> sh, lvl.y >> sh, lvl.z >> sh, lvl.w >> sh);
-            acc = cells_accept<S::GS>(pmin, pmax, W, cc, tp);
+            acc = cells_accept<S::GS, SPEC == 2 ? kTiesCount : SPEC == 3 ? kTiesRefused : kTiesAsk>(pmin, pmax, W, cc, tp);
             net += random_net(acc, pmin, pmax);
         }
         if (d & 2u)

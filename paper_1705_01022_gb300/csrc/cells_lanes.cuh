@@ -240,6 +240,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
 
     int net = 0;
     uint32_t draws = 0u, tails = 0u;
+    const uint32_t tie_mask = ties_matter(a.thr_p, a.thr_q) ? kFull : 0u;
     const uint32_t tp4 = a.thr_p >> 28, tq4 = a.thr_q >> 28, low_p = a.thr_p << 4, low_q = a.thr_q << 4;
     constexpr uint32_t kM = 1u | (1u << C::UX);  // X(s) and Y(s) of a half row, at the site's place
     constexpr int U = C::NCMAX < 4 ? C::NCMAX : 4;  // turns in flight
@@ -282,13 +283,13 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32) lane_cells_kernel(con
                 } else if (!RANDOM) {
                     acc = (mn && a.p_always) || (mx && a.q_always);
                 } else {
-                    const bool drw = SPEC == 2 ? mn || mx : (mn && a.p_random) || (mx && a.q_random);
+                    const bool drw = SPEC >= 2 ? mn || mx : (mn && a.p_random) || (mx && a.q_random);
                     const uint32_t u4 = (lw[c * C::GPI * 4] >> (4u * j) >> lev) & 15u, t4 = mn ? tp4 : tq4;
                     acc = drw && u4 < t4;
-                    if (SPEC != 2) acc = acc || (mn && a.p_always) || (mx && a.q_always);
+                    if (SPEC < 2) acc = acc || (mn && a.p_always) || (mx && a.q_always);
                     draws += drw ? 1u : 0u;
                     const bool tie = drw && u4 == t4;
-                    const uint32_t ties = __ballot_sync(kFull, tie);
+                    const uint32_t ties = SPEC == 3 ? 0u : SPEC == 2 ? __ballot_sync(kFull, tie) : __ballot_sync(kFull, tie) & tie_mask;
                     if (ties) {
                         // the ties of the lane's group, in order of position, take the next
                         // words of its tail stream
@@ -428,6 +429,8 @@ template <int CX, int CY>
 cudaError_t launch_cells_shape(const StepArgs &a, bool any_random, cudaStream_t st) {
     if (!any_random && a.p_always == 0xFFFFFFFFu && a.q_always == 0u)
         return launch_cells_variant<CX, CY, false, 1>(a, st);  // deposition only (p = 1, q = 0)
+    if (any_random && a.p_random && a.q_random && !ties_matter(a.thr_p, a.thr_q))
+        return launch_cells_variant<CX, CY, true, 3>(a, st);   // both inside, every tie refused
     if (any_random && a.p_random && a.q_random)
         return launch_cells_variant<CX, CY, true, 2>(a, st);   // both rates inside (0, 1)
     if (any_random) return launch_cells_variant<CX, CY, true, 0>(a, st);

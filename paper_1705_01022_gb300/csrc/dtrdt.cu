@@ -63,7 +63,7 @@ __host__ __device__ inline uint32_t segment_lanes(uint32_t groups) {
 // and DTrDTr with acceptance draws) spill at the 96 registers of five blocks;
 // at four blocks they do not, and run 3-4 % faster despite the lower occupancy.
 constexpr int step_min_blocks(int scheme, bool packed) {
-    return (packed || scheme == 2 || scheme == 3 || scheme == 7) ? kStepBlocksPerSMPacked : kStepBlocksPerSM;
+    return (packed || scheme == 2 || scheme == 3 || scheme == 7 || scheme == 9) ? kStepBlocksPerSMPacked : kStepBlocksPerSM;
 }
 
 template <bool RANDOM, int SCHEME, bool PACKED>
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
     const uint32_t T = pl.T, x0 = pl.x0, y0 = pl.y0;
 
     // round keys: see KeysConst
-    using Keys = std::conditional_t<SCHEME == 4, KeysWeyl, std::conditional_t<SCHEME == 0 || SCHEME == 5, KeysFma, KeysConst>>;
+    using Keys = std::conditional_t<SCHEME == 4, KeysWeyl, std::conditional_t<SCHEME == 0 || SCHEME == 5 || SCHEME == 8, KeysFma, KeysConst>>;
     LaneCtx<Keys> c;
     c.GX = static_cast<int>(a.GX);
     c.GY = static_cast<int>(a.GY);
@@ -152,6 +152,7 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, 
     const uint32_t per_block = kStepWarpsPerBlock * (packed ? 32u / S : 1u);
     const uint32_t blocks = (n_tiles + per_block - 1) / per_block;
     const dim3 grid(blocks), block(kStepWarpsPerBlock * 32);
+    const bool ties = ties_matter(a.thr_p, a.thr_q);
     cudaError_t e = cudaSuccess;
 #define OCT_LAUNCH(SCHEME, PACKED)                                                   \
     do {                                                                             \
@@ -173,7 +174,8 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, 
             if (packed)
                 OCT_LAUNCH(2, true);
             else if (a.p_random && a.q_random)
-                e = launch_overlapped(dtrdt_step_kernel<true, 7, false>, grid, block, overlap, st, a);  // both rates random
+                e = ties ? launch_overlapped(dtrdt_step_kernel<true, 7, false>, grid, block, overlap, st, a)  // both rates random
+                         : launch_overlapped(dtrdt_step_kernel<true, 9, false>, grid, block, overlap, st, a);
             else
                 OCT_LAUNCH(2, false);
             break;
@@ -196,9 +198,11 @@ cudaError_t launch_dtrdt_step(const StepArgs &a, bool any_random, bool overlap, 
             } else if (any_random && a.p_random && a.q_random) {
                 // both rates strictly inside (0, 1): every candidate is decided by its draw
                 if (packed)
-                    e = launch_overlapped(dtrdt_step_kernel<true, 5, true>, grid, block, overlap, st, a);
+                    e = ties ? launch_overlapped(dtrdt_step_kernel<true, 5, true>, grid, block, overlap, st, a)
+                             : launch_overlapped(dtrdt_step_kernel<true, 8, true>, grid, block, overlap, st, a);
                 else
-                    e = launch_overlapped(dtrdt_step_kernel<true, 5, false>, grid, block, overlap, st, a);
+                    e = ties ? launch_overlapped(dtrdt_step_kernel<true, 5, false>, grid, block, overlap, st, a)
+                             : launch_overlapped(dtrdt_step_kernel<true, 8, false>, grid, block, overlap, st, a);
             } else if (packed) {
                 OCT_LAUNCH(0, true);
             } else {

@@ -152,6 +152,8 @@ bool rows_fit_block(const StepArgs &a) { return row_warps(a) <= kBlockWarps && a
         const bool one = row_segment(a.GX, a.By) == 32u;                                                 \
         if (!any_random && a.p_always == 0xFFFFFFFFu && a.q_always == 0u)                                \
             return one ? FN<false, 1, true>(__VA_ARGS__) : FN<false, 1, false>(__VA_ARGS__);             \
+        if (any_random && a.p_random && a.q_random && !ties_matter(a.thr_p, a.thr_q))                    \
+            return one ? FN<true, 3, true>(__VA_ARGS__) : FN<true, 3, false>(__VA_ARGS__);               \
         if (any_random && a.p_random && a.q_random)                                                      \
             return one ? FN<true, 2, true>(__VA_ARGS__) : FN<true, 2, false>(__VA_ARGS__);               \
         if (any_random) return one ? FN<true, 0, true>(__VA_ARGS__) : FN<true, 0, false>(__VA_ARGS__);   \

@@ -14,7 +14,7 @@
 // leaves it (of the acceptance draws, their comparison with P32) in shared
 // memory, before the step's first access to the lattice.  8 MCS and a W^2: L=256
 // KPZ 405 -> 136 us, L=3136 p=0.95 (32 x 16 sub-tiles) 640 -> 285 us, L=4096
-// p=q=0.5 667 -> 354 us.
+// p=q=0.5 667 -> 350 us, then 256 us without its ties (ties_matter).
 //
 // Lanes of a sub-tile: gx + GX * tr, TC row tr = 0 .. By/4 - 1 (group row tr/4,
 // m = tr % 4), a power-of-two number of band columns GX, at most 32 lanes.
@@ -75,6 +75,8 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
         site_w[b * kRowGroups + gw] = c.draw(c.k | (b << 2), (kTagSite << 28) | c.g);
     }
     uint32_t head = 0u, end = 0u;  // words of the group's tail stream used, generated
+    // see ties_matter: with SPEC 3 none does, with SPEC -1 (general) the replica's rates say
+    const bool ties_count = SPEC == 0 || SPEC == 2 || (SPEC == -1 && __any_sync(kFull, ties_matter(c.thr_p, c.thr_q)));
     if (RANDOM) {
 #pragma unroll
         for (uint32_t i = 0; i < 4u; ++i) {
@@ -94,9 +96,11 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
             }
             lvl_w[s * kRowGroups + gw] = v;
         }
-        *reinterpret_cast<uint4 *>(ring + 4u * m) = c.draw(c.k | (m << 2), (kTagTail << 28) | c.g);
-        end = 16u;
-        ++tails;
+        if (ties_count) {
+            *reinterpret_cast<uint4 *>(ring + 4u * m) = c.draw(c.k | (m << 2), (kTagTail << 28) | c.g);
+            end = 16u;
+            ++tails;
+        }
     }
     __syncwarp();
     ready();
@@ -172,41 +176,43 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
             uint32_t acc = 0u;
             if (RANDOM) {
                 const uint32_t cc = f0 | f1, mx = (f0 & xa) | (f1 & xb);
-                const uint32_t cmx = SPEC == 2 ? mx : mx & c.q_random, cmn = SPEC == 2 ? cc : (cc & ~mx) & c.p_random;
+                const uint32_t cmx = SPEC >= 2 ? mx : mx & c.q_random, cmn = SPEC >= 2 ? cc : (cc & ~mx) & c.p_random;
                 const uint32_t pmax = ((cmx * 3u) >> (sh2 + 1u)) & kNib;
                 uint32_t pmin = ((cmn * 3u) >> (sh2 + 1u)) & kNib;
-                if (SPEC == 2) pmin &= ~pmax;
+                if (SPEC >= 2) pmin &= ~pmax;
                 draws += __popc(pmin | pmax);
                 const uint32_t mn = pmin << m, mx4 = pmax << m;  // bit 4j+m
                 acc = (mn & V.x) | (mx4 & V.z);
-                uint32_t und = (mn & V.y) | (mx4 & V.w);
-                // ties of the whole group, so that a tie's place in the tail stream is the
-                // number of lower ones
-                uint32_t gt = und;
-                gt |= __shfl_xor_sync(kFull, gt, rl.GX);
-                gt |= __shfl_xor_sync(kFull, gt, 2 * rl.GX);
-                const uint32_t nt = static_cast<uint32_t>(__popc(gt));
-                while (__any_sync(kFull, end - head < nt)) {
-                    __syncwarp();  // the words about to be overwritten have been read
-                    const uint4 B = c.draw(c.k | (((end >> 2) + m) << 2), (kTagTail << 28) | c.g);
-                    if (end - head <= kRowRing - 16u) {
-                        *reinterpret_cast<uint4 *>(ring + ((end + 4u * m) & (kRowRing - 1u))) = B;
-                        end += 16u;
-                        ++tails;
+                if (ties_count) {
+                    uint32_t und = (mn & V.y) | (mx4 & V.w);
+                    // ties of the whole group, so that a tie's place in the tail stream is the
+                    // number of lower ones
+                    uint32_t gt = und;
+                    gt |= __shfl_xor_sync(kFull, gt, rl.GX);
+                    gt |= __shfl_xor_sync(kFull, gt, 2 * rl.GX);
+                    const uint32_t nt = static_cast<uint32_t>(__popc(gt));
+                    while (__any_sync(kFull, end - head < nt)) {
+                        __syncwarp();  // the words about to be overwritten have been read
+                        const uint4 B = c.draw(c.k | (((end >> 2) + m) << 2), (kTagTail << 28) | c.g);
+                        if (end - head <= kRowRing - 16u) {
+                            *reinterpret_cast<uint4 *>(ring + ((end + 4u * m) & (kRowRing - 1u))) = B;
+                            end += 16u;
+                            ++tails;
+                        }
+                        __syncwarp();
                     }
-                    __syncwarp();
+                    while (und) {
+                        const uint32_t bit = und & (0u - und);
+                        und ^= bit;
+                        const uint32_t at = head + static_cast<uint32_t>(__popc(gt & (bit - 1u)));
+                        acc |= (ring[at & (kRowRing - 1u)] < ((mn & bit) ? low_p : low_q)) ? bit : 0u;
+                    }
+                    head += nt;
                 }
-                while (und) {
-                    const uint32_t bit = und & (0u - und);
-                    und ^= bit;
-                    const uint32_t at = head + static_cast<uint32_t>(__popc(gt & (bit - 1u)));
-                    acc |= (ring[at & (kRowRing - 1u)] < ((mn & bit) ? low_p : low_q)) ? bit : 0u;
-                }
-                head += nt;
                 acc = (acc >> m) & kNib;
                 net += random_net(acc, pmin, pmax);
             }
-            if (SPEC == 2) {
+            if (SPEC >= 2) {
                 const uint32_t spread = acc * 0xFu;
                 f0 &= spread;
                 f1 &= spread;

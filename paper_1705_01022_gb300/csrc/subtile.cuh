@@ -156,6 +156,17 @@ __device__ __forceinline__ void tail_refill(uint32_t need, uint32_t g, const Ctx
     }
 }
 
+// Whether a tied candidate can be accepted: with rates that are multiples of 1/16
+// (among them 1/2) the bits after the first four are below no threshold, so every
+// tie is refused and the tail stream need not be read.  p=q=1/2: 8 MCS and the W^2 of
+// L=4096 349 to 256 us; two MCS at L=32768 (1024x16) 1.25 to 1.03 ms, at L=8192 with 8 x 8
+// cells 868 to 656 us, in DTrDTr 268 to 230 us.
+__host__ __device__ __forceinline__ bool ties_matter(uint32_t thr_p, uint32_t thr_q) {
+    return ((thr_p | thr_q) << 4) != 0u;
+}
+// What a step knows of it when it is compiled (the question costs the others 0.3 to 3 %).
+constexpr int kTiesAsk = 0, kTiesCount = 1, kTiesRefused = 2;
+
 // Acceptance of the packed candidates (bit 4j+m = thread cell column j, TC
 // row m).  The uniform u of a candidate, most significant bit first:
 //  * bits 31..28 come from the four level words of the lane's group (bit
@@ -175,11 +186,12 @@ __device__ __forceinline__ uint4 level_words(uint32_t s, const Ctx &c) {
 // tie in the loop); the fastest choice differs between the block layers.
 // und: the tied candidates (of them, pmin: minima); returns acc with those that
 // their tail words accept.
-template <int PRE, class Ctx>
+template <int PRE, int TIES, class Ctx>
 __device__ __forceinline__ uint32_t resolve_ties(uint32_t acc, uint32_t und, uint32_t pmin, const Ctx &c, TailPool &tp) {
     // Skip the tail stage only when no lane of the warp needs it: every lane
     // takes part in the refill rounds.
-    if (__all_sync(kFull, und == 0u)) return acc;
+    if (TIES == kTiesRefused) return acc;
+    if (__all_sync(kFull, und == 0u || (TIES == kTiesAsk && !ties_matter(c.thr_p, c.thr_q)))) return acc;
     const uint32_t nt = static_cast<uint32_t>(__popc(und));
     tail_refill(nt, c.g, c, tp);
     // (w >> 4) < (P32 mod 2^28)  <=>  w < 16 (P32 mod 2^28)
@@ -213,7 +225,7 @@ __device__ __forceinline__ uint32_t resolve_ties(uint32_t acc, uint32_t und, uin
 }
 
 // The packed candidates against P32 on the four levels, then the ties.
-template <int PRE, class Ctx>
+template <int PRE, int TIES = kTiesAsk, class Ctx>
 __device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pmax, const uint4 &W,
                                                       const Ctx &c, TailPool &tp) {
     const uint32_t lw[4] = {W.x, W.y, W.z, W.w};
@@ -225,7 +237,7 @@ __device__ __forceinline__ uint32_t accept_candidates(uint32_t pmin, uint32_t pm
         acc |= und & tb & ~lw[i];
         und &= ~(tb ^ lw[i]);
     }
-    return resolve_ties<PRE>(acc, und, pmin, c, tp);
+    return resolve_ties<PRE, TIES>(acc, und, pmin, c, tp);
 }
 
 // A lane's flips at column 31, or 0, gathered by row with one funnel shift per row
@@ -775,7 +787,7 @@ __device__ __forceinline__ void transpose_nibbles(const uint4 &site, uint32_t (&
 // 511 us, and from 465 to 437 us when the attempt's row is picked by bit masks
 // (three selects per quantity instead of an and-or per row) and one comparison
 // of the level words serves the three phases.
-template <bool RANDOM, int SPEC = 0, class Ctx>
+template <bool RANDOM, int SPEC = 0, int TIES = kTiesAsk, class Ctx>
 __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)[16], uint32_t &E, uint32_t &D,
                                                 const uint4 &site, uint32_t s, const Ctx &c, TailPool &tp,
                                                 int &net, int &draws) {
@@ -821,7 +833,7 @@ __device__ __forceinline__ void db_step_delayed(uint32_t (&X)[16], uint32_t (&Y)
         uint32_t f = 0u;
         if (RANDOM) {
             const uint32_t pmin = SPEC == 2 ? mn : mn & c.p_random, pmax = SPEC == 2 ? mx : mx & c.q_random;
-            f = resolve_ties<kPreDb>((pmin & lv.ltp) | (pmax & lv.ltq), (pmin & lv.eqp) | (pmax & lv.eqq), pmin, c, tp);
+            f = resolve_ties<kPreDb, TIES>((pmin & lv.ltp) | (pmax & lv.ltq), (pmin & lv.eqp) | (pmax & lv.eqq), pmin, c, tp);
             dmin |= pmin;
             dmax |= pmax;
             dacc |= f;
@@ -1335,7 +1347,8 @@ __device__ __forceinline__ void write_back(const LaneGeom &q, uint32_t L, uint32
 // SCHEME: 0 DTrDT, 1 DTrDB with all attempts of a step together, 2 DTrDB with
 // delayed borders, 3 DTrDTr, 4 DTrDT with deposition only (p = 1, q = 0),
 // 5 DTrDT with both rates strictly inside (0, 1), 6 DTrDB with deposition only,
-// 7 DTrDB with delayed borders and both rates random.
+// 7 DTrDB with delayed borders and both rates random, 8 and 9 as 5 and 7 with
+// rates for which every tie is refused, 10 as 5 for rates of either kind.
 template <bool RANDOM, bool LANE_SETS, int SCHEME = 0, class Ctx>
 __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t plane_rows, uint32_t wpr,
                                             uint32_t Bx, uint32_t By, uint32_t x0, uint32_t y0, bool active,
@@ -1354,7 +1367,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
 
     const FlipConsts flips;
     uint32_t E0 = 0u;  // X bits of the lane's own column 0 (for column_fields)
-    if (LANE_SETS && (SCHEME == 0 || SCHEME == 5)) E0 = gather_lsb(X);
+    if (LANE_SETS && (SCHEME == 0 || SCHEME == 5 || SCHEME == 8 || SCHEME == 10)) E0 = gather_lsb(X);
 
     // Block layer: 16 single-hit collective steps.
     const uint4 setw = c.draw(c.k, kTagSet << 28);
@@ -1383,13 +1396,15 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
             dtr_apply<RANDOM, LANE_SETS>(X, Y, E, D, c0, r0, acc, ca, cb, c, n, net);
             continue;
         }
-        if (SCHEME == 1 || SCHEME == 2 || SCHEME == 6 || SCHEME == 7) {
+        if (SCHEME == 1 || SCHEME == 2 || SCHEME == 6 || SCHEME == 7 || SCHEME == 9) {
             // DB: one site word per TC row and step, 4 bits per cell
             site = c.draw(c.k | (s << 2), (kTagSiteDb << 28) | c.g);
             if (SCHEME == 2)
                 db_step_delayed<RANDOM>(X, Y, E, D, site, s, c, tp, net, draws);
             else if (SCHEME == 7)
-                db_step_delayed<RANDOM, 2>(X, Y, E, D, site, s, c, tp, net, draws);
+                db_step_delayed<RANDOM, 2, kTiesCount>(X, Y, E, D, site, s, c, tp, net, draws);
+            else if (SCHEME == 9)
+                db_step_delayed<RANDOM, 2, kTiesRefused>(X, Y, E, D, site, s, c, tp, net, draws);
             else if (SCHEME == 6)
                 db_step<RANDOM, 1>(X, Y, E, D, site, s, c, tp, net, draws);
             else
@@ -1405,7 +1420,8 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
         const uint32_t d_own = (setw.x >> (2u * s)) & 3u;
         const uint32_t d = LANE_SETS ? d_own : __shfl_sync(kFull, d_own, 0);
         uint32_t cnd0[4], cnd1[4], pmin, pmax;
-        constexpr int kSpec = SCHEME == 4 ? 1 : SCHEME == 5 ? 2 : 0;
+        constexpr int kSpec = SCHEME == 4 ? 1 : (SCHEME == 5 || SCHEME == 8 || SCHEME == 10) ? 2 : 0;
+        constexpr int kTies = (SCHEME == 0 || SCHEME == 5) ? kTiesCount : SCHEME == 8 ? kTiesRefused : kTiesAsk;
         if (LANE_SETS)
             step_candidates_rt<RANDOM, kSpec>(X, Y, E, D, site, s, d & 1u, d >> 1, c, cnd0, cnd1, pmin, pmax);
         // the candidate phase with the set's column offset as a constant as well
@@ -1422,7 +1438,7 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
         uint32_t acc = 0u;
         if (RANDOM) {
             draws += __popc(pmin | pmax);
-            acc = accept_candidates<SCHEME == 3 ? kPreDtr : (LANE_SETS ? kPrePacked : kPreDt)>(pmin, pmax, level_words(s, c), c, tp);
+            acc = accept_candidates<LANE_SETS ? kPrePacked : kPreDt, kTies>(pmin, pmax, level_words(s, c), c, tp);
             net += random_net(acc, pmin, pmax);
         }
         if (LANE_SETS)
