@@ -1169,7 +1169,13 @@ int oct_batch_measure_w2(oct_batch *b, oct_w2 *out, int64_t n) {
     for (size_t i = 0; i < b->job_ranges.size(); ++i) {
         const uint32_t first = b->job_ranges[i].first;
         const uint32_t end = i + 1 < b->job_ranges.size() ? b->job_ranges[i + 1].first : b->n_jobs;
-        BATCH_CUDA(oct::launch_w2_small(b->d_jobs + first, end - first, b->job_ranges[i].second, b->d_rows, b->stream));
+        if (end - first == 1u) {
+            oct::W2Job j = b->h_jobs[first];
+            BATCH_CUDA(oct::launch_w2_small_pack(&j, 1, b->d_rows, b->stream));
+        } else {
+            BATCH_CUDA(
+                oct::launch_w2_small(b->d_jobs + first, end - first, b->job_ranges[i].second, b->d_rows, b->stream));
+        }
     }
     BATCH_CUDA(cudaStreamSynchronize(b->stream));
     for (int64_t slot = 0; slot < n; ++slot) {

@@ -466,6 +466,10 @@ __global__ void __launch_bounds__(kW2CombineThreads)
 // filled during the last device step (8 MCS of L=256 and their W^2: 132 to
 // 128 us).
 constexpr int kW2SmallThreads = 512;  // of the second launch
+// Rows of one lattice that a single block may finish; a lattice alone with more
+// takes the large passes, whose second one has a block per 256 rows (W^2 in two
+// launches and in four, us: L=8192 41, 41; 12288 59, 44; 16384 70, 46).
+constexpr uint32_t kW2FinishRows = 8192;
 
 // Words j .. j+3 of the lane's nw, as one 16-byte load where allowed.
 __device__ __forceinline__ void load_quad(const uint32_t *row, uint32_t j, uint32_t nw, bool vec_ok,
@@ -584,9 +588,21 @@ __global__ void __launch_bounds__(kW2SmallThreads)
     const W2RowSums *rows = all_rows + J.row_first;
     const uint32_t per = (nrows + kW2SmallThreads - 1) / kW2SmallThreads;
     const uint32_t y0 = min(nrows, tid * per), y1 = min(nrows, y0 + per);
-    int rise = 0;  // of the column heights over the thread's rows
-    for (uint32_t y = y0; y < y1; ++y) rise += y == 0 ? 0 : rows[y].c ? 1 : -1;
-    int incl = rise;
+    // one pass over the thread's rows, relative to the height before its first one;
+    // several rows' records are in flight at a time
+    const long long Ll = J.L;
+    long long v[4] = {0, 0, 0, 0};  // S1, S2, counters
+    int hl = 0, rlo = 1 << 30, rhi = -(1 << 30);
+#pragma unroll 8
+    for (uint32_t y = y0; y < y1; ++y) {
+        const W2RowSums r = rows[y];
+        hl += y == 0 ? 0 : r.c ? 1 : -1;
+        v[0] += Ll * hl + r.r1;
+        v[1] += Ll * hl * hl + 2 * hl * r.r1 + r.r2;
+        rlo = min(rlo, hl + r.rmin);
+        rhi = max(rhi, hl + r.rmax);
+    }
+    int incl = hl;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int x = __shfl_up_sync(kFull, incl, o);
@@ -594,20 +610,17 @@ __global__ void __launch_bounds__(kW2SmallThreads)
     }
     if (lane == 31) wsum[warp] = incl;
     __syncthreads();
-    long long h = incl - rise;
+    long long h = incl - hl;  // before the thread's first row
     for (int w = 0; w < warp; ++w) h += wsum[w];
-    const long long Ll = J.L;
-    long long v[4] = {0, 0, 0, 0};  // S1, S2, counters
+    const long long n = y1 - y0;
+    v[1] += 2 * h * v[0] + Ll * n * h * h;
+    v[0] += Ll * n * h;
     long long lo = 1ll << 40, hi = -(1ll << 40);
-    for (uint32_t y = y0; y < y1; ++y) {
-        const W2RowSums r = rows[y];
-        h += y == 0 ? 0 : r.c ? 1 : -1;
-        v[0] += Ll * h + r.r1;
-        v[1] += Ll * h * h + 2 * h * r.r1 + r.r2;
-        lo = min(lo, h + r.rmin);
-        hi = max(hi, h + r.rmax);
+    if (n > 0) {
+        lo = h + rlo;
+        hi = h + rhi;
     }
-    if (y0 < y1 && y1 == nrows) last_h = h;
+    if (y0 < y1 && y1 == nrows) last_h = h + hl;
     if (J.cnt)
         for (uint32_t i = tid; i < J.cnt_n; i += kW2SmallThreads) {
             v[2] += static_cast<long long>(J.cnt[i]);
@@ -650,6 +663,32 @@ __global__ void __launch_bounds__(kW2SmallThreads)
         }
         if (J.t) *J.t_out = *J.t;
     }
+}
+
+// The counters and the time of a job whose sums the large passes took.
+__global__ void w2_counters_kernel(const __grid_constant__ W2Job J) {
+    __shared__ unsigned long long sum[2];
+    if (threadIdx.x < 2u) sum[threadIdx.x] = 0ull;
+    __syncthreads();
+    if (J.cnt) {
+        unsigned long long a = 0, b = 0;
+        for (uint32_t i = threadIdx.x; i < J.cnt_n; i += blockDim.x) {
+            a += J.cnt[i];
+            b += J.cnt[J.cnt_off + i];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            a += __shfl_down_sync(kFull, a, o);
+            b += __shfl_down_sync(kFull, b, o);
+        }
+        if ((threadIdx.x & 31u) == 0u) {
+            atomicAdd(&sum[0], a);
+            atomicAdd(&sum[1], b);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 2u && J.cnt) J.cnt_out[threadIdx.x] = static_cast<long long>(sum[threadIdx.x]);
+    if (threadIdx.x == 0u && J.t) *J.t_out = *J.t;
 }
 
 // Interleave two 4-bit values: a0 b0 a1 b1 a2 b2 a3 b3 (LSB first).
@@ -767,6 +806,27 @@ cudaError_t w2_small(const W2Pack<N> &pack, const W2Job *jobs, uint32_t n, uint3
                              static_cast<const W2RowSums *>(rows));
 }
 
+// One lattice in the passes for large ones: a warp per row, then a block per
+// kW2BlockRows rows, then one block.
+cudaError_t w2_large(const uint32_t *lat, uint32_t L, uint32_t nrows, uint32_t plane_rows, W2RowSums *rows,
+                     W2Result *out, cudaStream_t st) {
+    // one wave of resident blocks (64 KB of table each), rows taken grid-stride
+    int sms = 0;
+    cudaError_t e = table_kernel_setup(reinterpret_cast<const void *>(w2_rows_kernel), 0, &sms);
+    if (e != cudaSuccess) return e;
+    const uint64_t want = (static_cast<uint64_t>(nrows) + kW2Warps - 1) / kW2Warps;
+    const uint64_t wave = static_cast<uint64_t>(sms) * kW2BlocksPerSM;
+    const int blocks = static_cast<int>(want < wave ? want : wave);
+    w2_rows_kernel<<<blocks, kW2Warps * 32, kW2TableBytes, st>>>(lat, L, nrows, plane_rows, rows);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    w2_block_kernel<<<(nrows + kW2BlockRows - 1) / kW2BlockRows, kW2BlockRows, 0, st>>>(rows, L, nrows);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    w2_combine_kernel<<<1, kW2CombineThreads, 0, st>>>(rows, L, nrows, out);
+    return cudaGetLastError();
+}
+
 int grid_for(uint64_t n, int threads) {
     const uint64_t b = (n + threads - 1) / threads;
     return static_cast<int>(b < 152ull * 32 ? (b ? b : 1) : 152ull * 32);
@@ -801,21 +861,7 @@ cudaError_t launch_w2_rows(const uint32_t *lat, uint32_t L, uint32_t nrows, uint
         j.res = out;
         return launch_w2_small_pack(&j, 1, rows, st);
     }
-    // one wave of resident blocks (64 KB of table each), rows taken grid-stride
-    int sms = 0;
-    cudaError_t e = table_kernel_setup(reinterpret_cast<const void *>(w2_rows_kernel), 0, &sms);
-    if (e != cudaSuccess) return e;
-    const uint64_t want = (static_cast<uint64_t>(nrows) + kW2Warps - 1) / kW2Warps;
-    const uint64_t wave = static_cast<uint64_t>(sms) * kW2BlocksPerSM;
-    const int blocks = static_cast<int>(want < wave ? want : wave);
-    w2_rows_kernel<<<blocks, kW2Warps * 32, kW2TableBytes, st>>>(lat, L, nrows, plane_rows, rows);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    w2_block_kernel<<<(nrows + kW2BlockRows - 1) / kW2BlockRows, kW2BlockRows, 0, st>>>(rows, L, nrows);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    w2_combine_kernel<<<1, kW2CombineThreads, 0, st>>>(rows, L, nrows, out);
-    return cudaGetLastError();
+    return w2_large(lat, L, nrows, plane_rows, rows, out, st);
 }
 
 uint32_t w2_small_split(W2Job *jobs, uint32_t n) {
@@ -852,6 +898,13 @@ cudaError_t launch_w2_small_pack(W2Job *jobs, uint32_t n, W2RowSums *rows, cudaS
     if (n == 0 || n > kW2PackJobs) return cudaErrorInvalidValue;
     const uint32_t n_tasks = w2_small_split(jobs, n);
     const W2Job *none = nullptr;
+    if (n == 1 && jobs[0].nrows > kW2FinishRows) {
+        const W2Job &j = jobs[0];
+        const cudaError_t e = w2_large(j.lat, j.L, j.nrows, j.plane_rows, rows, j.res, st);
+        if (e != cudaSuccess || !(j.cnt || j.t)) return e;
+        w2_counters_kernel<<<1, j.cnt_n > 256u ? 512 : 32, 0, st>>>(j);
+        return cudaGetLastError();
+    }
     if (n == 1) return w2_small(W2Pack<1>{{jobs[0]}}, none, 1, n_tasks, rows, st);
     W2Pack<kW2PackJobs> pack{};
     std::copy(jobs, jobs + n, pack.j);

@@ -40,3 +40,25 @@ def test_lists_equal_single_measurements(sizes):
         with pytest.raises(_lib.OctError):
             _lib.oct_batch_wait(b.h, before + 1)
         assert _lib.oct_batch_measure_slots_async(b.h, []) == []
+
+
+@pytest.mark.parametrize("L", [8192, 8256])
+def test_one_large_replica(L):
+    """The last size one block finishes and the first it does not: alone, listed
+    with another, and as a simulation."""
+    import paper_1705_01022_gb300 as g
+    from paper_1705_01022_gb300 import _lib
+    g.build()
+    with g.Simulation(L, 0.95, 0.05, 5, Bx=32, By=32) as sim:
+        sim.run(2)
+        m = sim.measure()
+        want = tuple(getattr(m, f) for f in FIELDS)
+    rep = (L, 0.95, 0.05, 5, 32, 32)
+    with g.Batch([rep]) as b, g.Batch([rep, rep]) as two:
+        for x in (b, two):
+            x.run(2)
+        got = [_values(m) for m in b.measure() + two.measure()]
+        got += [_values(_lib.oct_batch_measure_slot(b.h, 0))]
+        got += [_values(_lib.oct_batch_wait(x.h, t)) for x in (b, two)
+                for t in _lib.oct_batch_measure_slots_async(x.h, list(range(len(x))))]
+    assert got == [want] * 7
