@@ -977,7 +977,7 @@ def main():
             "warmup": a.warmup, "ms_per_step": ms_max / a.steps, "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None, "dtype": "u32", "data": "synthetic",
             "config": workload(a), "clocks": clk.summary(), "roofline": roofline,
-            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": 5 * a.steps, "autotune": tuning, "dtrdb": dtrdb, "dtrdtr": dtrdtr, "cells": cells, "w2": w2_leg, "two_time": two_time, "batched": batched, "serving": serving,
+            "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": 4 * a.steps + 1, "autotune": tuning, "dtrdb": dtrdb, "dtrdtr": dtrdtr, "cells": cells, "w2": w2_leg, "two_time": two_time, "batched": batched, "serving": serving,
             "probe": {"lop3_per_clk_per_sm": lop3, "imad_per_clk_per_sm": imad, "probe_mhz": probe_mhz},
         }
         print(json.dumps(out), flush=True)

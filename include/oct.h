@@ -253,7 +253,8 @@ int oct_get_timing(oct_sim *s, double *step_ms, int64_t *step_launches, double *
  * needed an acceptance draw (counted only when p or q lies strictly inside
  * (0,1)), tail_blocks = Philox blocks the plain device-step kernels generated
  * for the tail stream of tied acceptance uniforms (counted over the lanes that
- * store them; zero without acceptance draws).  Synchronises. */
+ * store them; zero without acceptance draws, and where the rates are multiples
+ * of 1/16, whose ties are all refused).  Synchronises. */
 typedef struct {
     int64_t t;
     int64_t net_flips;
@@ -352,8 +353,8 @@ int oct_two_time_planes(const void *lat_t, const void *lat_s, int64_t L, void *s
  * Batched replicas.  Many independent realizations (each its own L, p, q and
  * key; every one the same DTrDT dynamics as a single handle, bit for bit) are
  * advanced together: every device step of every replica runs in one launch
- * per acceptance mode, and one MCS is captured once in a CUDA graph and
- * replayed.  Replica lattices are device-resident, planar layout.
+ * (small batches) or one per acceptance mode, warp packing and part, captured
+ * once in CUDA graphs and replayed.  Replica lattices are device-resident, planar layout.
  * ------------------------------------------------------------------------- */
 typedef struct oct_batch oct_batch;
 
@@ -387,7 +388,7 @@ int oct_batch_add(oct_batch *b, const oct_replica *r, int64_t *slot);
 int oct_batch_remove(oct_batch *b, int64_t slot);
 
 /* Enqueues n MCS for every replica in the batch (asynchronous); each replica
- * advances its own time t.  The work list and graph are rebuilt first if
+ * advances its own time t.  The work list (and graph) is rebuilt first if
  * replicas were added or removed; the rebuild copies the new work list in
  * stream order and does not wait for the device. */
 int oct_batch_run(oct_batch *b, int64_t n);
