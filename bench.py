@@ -385,16 +385,16 @@ def batched_leg(a, g, _lib, torch, stream, peak_tops):
         kms, klaunch = _lib.oct_batch_get_timing(b.h)
         _lib.oct_batch_set_timing(b.h, False)
         f_draw = draws / (sites * a.batch_steps)
-        # The batched kernel keeps no tail-block count: ties are 1/16 of the draws in
-        # expectation and a block holds four tail words, so about draws/64 blocks.
-        acct = alu_accounting("DT", 4, 4, True, 1.0, f_draw / 64.0, f_draw, 256)
+        # The batched kernel keeps no tail-block count, and its replicas at p = q = 1/2,
+        # whose ties are all refused, generate none: no tail block is credited.
+        acct = alu_accounting("DT", 4, 4, True, 1.0, 0.0, f_draw, 256)
         ops = acct["generated"]["ops_per_attempt"]
         achieved = ops * sites / 4 / (kms / klaunch * 1e-3) / 1e12
         survey = acct["survey"]["ops_per_attempt"] * sites / 4 / (kms / klaunch * 1e-3) / 1e12
         out["roofline"] = {"bound": "alu", "achieved": achieved, "peak": peak_tops, "unit": "Tops/s",
                            "frac": achieved / peak_tops, "kernel": "batch_step_kernel",
                            "device_step_ms": kms / klaunch, "draw_fraction": f_draw, "ops_per_attempt": ops,
-                           "accounting": "generated bits; tail blocks estimated as draws/64",
+                           "accounting": "generated bits, without the tail blocks (not counted)",
                            "survey_accounting": {"ops_per_attempt": acct["survey"]["ops_per_attempt"],
                                                  "achieved": survey, "frac": survey / peak_tops}}
     # the same replicas, one plain handle each, launched one after another

@@ -20,12 +20,13 @@
 // (8 TCs across, 4 TC rows) as 16 X-row and 16 Y-row words in registers, so
 // a collective step is a handful of 32-bit logic operations per TC row:
 // selection masks from the site draw, the four-bit minimum/maximum pattern,
-// and XOR flips.  The neighbour bits the update rule needs at the group edge
+// and flips by multiply-adds (signed_flips).  The neighbour bits the update rule needs at the group edge
 // (the X column just right of the group, the Y row just below it) are kept
 // as copies (E, D) and refreshed by warp shuffles after every step.  Acceptance
 // draws for 0 < p, q < 1 compare all 32 TCs of a lane against P32 at once on
-// four random bit levels; the rare ties finish from a tail stream shared by the
-// sub-tile through a ring in shared memory.
+// four random bit levels; the rare ties finish from the group's tail stream, in
+// the lane's own slot of shared memory.  Launches of fewer than 32 warps per SM
+// take a TC row per lane instead (rowlanes.cuh).
 //
 // Random streams (Philox-4x32-10, key = seed):
 //   MCS draw  (t, 0, 0, MCS<<28): ox, oy, set permutation
@@ -35,7 +36,7 @@
 //   acceptance: bits 31..28 of the uniform of TC (j, m) are bit 4j+m of the
 //             four words of (t, k|(s*8)<<2, T, ACC<<28|g); bits 27..0, needed
 //             only when those tie with P32's, are the top of the next word of
-//             the sub-tile's tail stream (t, k|(i/4)<<2, T, TAIL<<28)
+//             the group's tail stream (t, k|(i/4)<<2, T, TAIL<<28|g)
 #include <type_traits>
 
 #include "oct_internal.h"
