@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
 // share the launch (two forms of the step: deposition only, and the general
 // one), so that no replica waits for another's kernel, and there is no graph to
 // capture after every membership change.  Latency bound like rowlanes.cuh: 16
-// MCS and the W^2 of 64 replicas of L = 64..512 take 0.74 ms.
+// MCS and the W^2 of 64 replicas of L = 64..512 take 0.72 ms.
 template <bool RANDOM, int SPEC, bool ONE>
 __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDesc &wd, uint32_t T, bool held, uint32_t t,
                                                uint32_t k, uint32_t *sm) {
@@ -183,8 +183,8 @@ __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDe
 
 // Larger batches take the graph's branches, whose lanes of four TC rows need
 // fewer instructions per attempt (16 MCS and the W^2 of n replicas of L=2048, 256
-// warps each, ms in row lanes and with the graph: n=20 1.78, 2.38; 24 2.11, 2.44;
-// 32 2.71, 2.86; 48 3.91, 3.05).
+// warps each, ms in row lanes and with the graph: n=16 1.38, 1.98; 24 2.00, 2.29;
+// 32 2.52, 2.69; 40 3.07, 2.93).
 constexpr uint32_t kBatchRowWarpsMax = 152u * 54u;
 
 // One warp per block, so that the blocks spread evenly over the schedulers (16
