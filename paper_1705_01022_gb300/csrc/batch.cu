@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "../../include/oct.h"
+#include "grow.h"
 #include "oct_internal.h"
 #include "overlap.cuh"
 #include "rowlanes.cuh"
@@ -319,7 +320,7 @@ struct oct_batch {
     uint32_t row_descs = 0;       // warps of a device step in row lanes; 0: the branches below carry the batch
     uint32_t *d_queue = nullptr;  // 4 * kBranches counters: (device step, branch)
     oct::W2RowSums *d_rows = nullptr;
-    int64_t rows_cap = 0;
+    size_t rows_cap = 0;
     void *h_small = nullptr;
     // measurement of all replicas: job list (device, and its pinned staging),
     // records by slot, and the launches' ranges; rebuilt after a membership change
@@ -457,20 +458,18 @@ oct::ReplicaDev replica_dev(const oct_batch *b, int64_t slot) {
     return D;
 }
 
+// Stream-ordered: work already enqueued may still read the old buffer.
+template <typename T>
+cudaError_t grow_async(T **p, size_t *cap, size_t n, cudaStream_t st) {
+    return oct::grow_buffer(
+        p, cap, n, [st](T **q, size_t k) { return cudaMallocAsync(reinterpret_cast<void **>(q), sizeof(T) * k, st); },
+        [st](T *old) { return cudaFreeAsync(old, st); });
+}
+
 template <typename T>
 cudaError_t ensure(T **p, size_t *cap, size_t need, cudaStream_t st) {
     if (need <= *cap) return cudaSuccess;
-    size_t n = std::max<size_t>(need, 2 * *cap);
-    // stream-ordered: work already enqueued may still read the old buffer
-    if (*p) {
-        cudaError_t e = cudaFreeAsync(*p, st);
-        if (e != cudaSuccess) return e;
-    }
-    *p = nullptr;
-    *cap = 0;
-    cudaError_t e = cudaMallocAsync(reinterpret_cast<void **>(p), sizeof(T) * n, st);
-    if (e == cudaSuccess) *cap = n;
-    return e;
+    return grow_async(p, cap, std::max<size_t>(need, 2 * *cap), st);
 }
 
 // Grows the per-slot tables, keeping the device-resident counters.
@@ -849,15 +848,11 @@ oct::W2Job replica_job(const oct_batch *b, int64_t slot, oct::MeasureRecord *m) 
     return j;
 }
 
-// Row records for `rows` rows; stream-ordered: an earlier measurement may
-// still use the old ones.
+// Row records for `rows` rows.  They never shrink, also when growing fails: the
+// built job list (build_jobs) relies on those that it asked for.
 int ensure_rows(oct_batch *b, int64_t rows) {
-    if (rows <= b->rows_cap) return OCT_OK;
-    if (b->d_rows) BATCH_CUDA(cudaFreeAsync(b->d_rows, b->stream));
-    b->d_rows = nullptr;
-    b->rows_cap = 0;
-    BATCH_CUDA(cudaMallocAsync(reinterpret_cast<void **>(&b->d_rows), sizeof(oct::W2RowSums) * rows, b->stream));
-    b->rows_cap = rows;
+    if (static_cast<size_t>(rows) > b->rows_cap)
+        BATCH_CUDA(grow_async(&b->d_rows, &b->rows_cap, static_cast<size_t>(rows), b->stream));
     return OCT_OK;
 }
 
