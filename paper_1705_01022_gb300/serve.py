@@ -143,7 +143,11 @@ class ServingEngine:
         self.waiting: deque[Job] = deque()
         self.running: dict[tuple, Job] = {}  # (batch index, slot) -> job
         self.finished: list[Job] = []
-        self.pending: deque = deque()  # (job, batch index, ticket) of asynchronous measurements
+        # asynchronous measurements not yet delivered, in the order they were enqueued:
+        # [job, batch index, ticket, result or None], and those of each batch whose
+        # result has not been read
+        self.pending: deque = deque()
+        self.unread = [deque() for _ in self.batches]
         self.async_measure = all(hasattr(b, "measure_async") for b in self.batches)
         self.ticks = 0
         self.mcs_attempts = 0
@@ -226,12 +230,7 @@ class ServingEngine:
             # the measurements due now, together: a W^2 of a few rows leaves the device nearly idle
             due = [(job, slot) for (b, slot), job in self.running.items()
                    if b == bi and job.t + n in job.measure_at]
-            slots = [slot for _, slot in due]
-            if hasattr(batch, "measure_async_many"):
-                tickets = batch.measure_async_many(slots)
-            else:
-                tickets = [batch.measure_async(slot) for slot in slots]
-            self.pending.extend((job, bi, ticket) for (job, _), ticket in zip(due, tickets))
+            self._measure(bi, due)
         for (b, slot), job in list(self.running.items()):
             if b != bi:
                 continue
@@ -250,6 +249,28 @@ class ServingEngine:
         if self.throttled:
             self.inflight[bi].append(batch.mark())
 
+    def _measure(self, bi: int, due) -> None:
+        """Enqueues the measurements of (job, slot) pairs.  A batch keeps the
+        results of its last ``measure_limit`` tickets only (no such attribute:
+        all of them), so before more than that are out the oldest ones are read,
+        waiting for them if need be; ``deliver`` hands them on in their turn."""
+        batch, unread = self.batches[bi], self.unread[bi]
+        limit = getattr(batch, "measure_limit", None)
+        step = max(1, limit // 2) if limit else max(1, len(due))
+        for i in range(0, len(due), step):
+            part = due[i:i + step]
+            while limit and unread and len(unread) + len(part) > limit:
+                m = unread.popleft()
+                m[3] = batch.wait(m[2])
+            slots = [slot for _, slot in part]
+            if hasattr(batch, "measure_async_many"):
+                tickets = batch.measure_async_many(slots)
+            else:
+                tickets = [batch.measure_async(slot) for slot in slots]
+            new = [[job, bi, ticket, None] for (job, _), ticket in zip(part, tickets)]
+            self.pending.extend(new)
+            unread.extend(new)
+
     def _deliver_one(self, job: Job, res, now=None) -> None:
         assert res[0] in job.measure_at, (res[0], job.measure_at)
         job.results.append(res)
@@ -265,10 +286,12 @@ class ServingEngine:
         number delivered."""
         n = 0
         while self.pending:
-            job, bi, ticket = self.pending[0]
-            res = self.batches[bi].wait(ticket) if block else self.batches[bi].poll(ticket)
+            job, bi, ticket, res = self.pending[0]
             if res is None:
-                break
+                res = self.batches[bi].wait(ticket) if block else self.batches[bi].poll(ticket)
+                if res is None:
+                    break
+                self.unread[bi].popleft()
             self.pending.popleft()
             self._deliver_one(job, res)
             n += 1
@@ -356,6 +379,8 @@ def summary(jobs, wall_s: float) -> dict:
 class GpuBatch:
     """Adapter from the engine's batch interface to the C ABI batch."""
 
+    measure_limit = 1024  # tickets whose results stay readable (oct_batch_measure_async)
+
     def __init__(self, stream=None):
         from . import _address, _lib
         self._lib = _lib
@@ -386,9 +411,8 @@ class GpuBatch:
         return self._lib.oct_batch_measure_async(self.h, slot)
 
     def measure_async_many(self, slots) -> list:
-        # a call takes at most 1024 (_lib's ring of tickets)
-        return [t for i in range(0, len(slots), 1024)
-                for t in self._lib.oct_batch_measure_slots_async(self.h, slots[i:i + 1024])]
+        # (a list longer than measure_limit is refused: its first tickets would be lost to its last)
+        return self._lib.oct_batch_measure_slots_async(self.h, slots)
 
     def mark(self) -> int:
         return self._lib.oct_batch_mark(self.h)
