@@ -387,8 +387,10 @@ int oct_batch_add(oct_batch *b, const oct_replica *r, int64_t *slot);
 /* Removes the replica in `slot` and returns its lattice to the pool. */
 int oct_batch_remove(oct_batch *b, int64_t slot);
 
-/* Enqueues n MCS for every replica in the batch (asynchronous); each replica
- * advances its own time t.  The work list (and graph) is rebuilt first if
+/* Enqueues n MCS for every replica in the batch (asynchronous; a caller that
+ * enqueues more than about a thousand launches or graph replays ahead of the
+ * device waits in the call for the driver's queue); each replica advances its
+ * own time t.  The work list (and graph) is rebuilt first if
  * replicas were added or removed; the rebuild copies the new work list in
  * stream order and does not wait for the device. */
 int oct_batch_run(oct_batch *b, int64_t n);

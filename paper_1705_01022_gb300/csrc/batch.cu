@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(kBatchWarps * 32, kBatchBlocksPerSM)
 // A batch too small to fill the chip: one device step of every replica in one
 // launch, a TC row per lane (rowlanes.cuh), a descriptor per warp.  All modes
 // share the launch (two forms of the step: deposition only, and the general
-// one), so that no replica waits for another's kernel, and there is no graph to
-// capture after every membership change.  Latency bound like rowlanes.cuh: 16
-// MCS and the W^2 of 64 replicas of L = 64..512 take 0.72 ms.
+// one), so that no replica waits for another's kernel, and a membership that
+// soon changes has no graph to capture (kRowLaunchMcs).  Latency bound like
+// rowlanes.cuh: 16 MCS and the W^2 of 64 replicas of L = 64..512 take 0.72 ms.
 template <bool RANDOM, int SPEC, bool ONE>
 __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDesc &wd, uint32_t T, bool held, uint32_t t,
                                                uint32_t k, uint32_t *sm) {
@@ -287,6 +287,17 @@ constexpr int kMeasureRing = 1024;
 constexpr int64_t kPackRows = 65536;
 constexpr int kMarkRing = 64;
 constexpr int kGraphMcs = 4;  // MCS in the batch's longer captured graph
+// A batch in row lanes takes four launches per MCS.  The driver queues about a
+// thousand launches; past that a call waits for the device, so a long run would
+// no longer return at once (3000 MCS of four small replicas: the call took 90 of
+// 99 ms, 1.2 of 97 with replays).  After kRowLaunchMcs MCS of one membership the
+// rest is replayed from graphs of kRowGraphMcs and kRowGraphShort MCS (a batch
+// whose replicas change sooner, as in serving, never pays for their capture).
+// Replays break the overlap of launches at their ends: us per MCS of that batch
+// launched, and in graphs of 4, 8, 16 and 32 MCS, 31.6, 32.2, 31.9, 31.7 and 31.6.
+constexpr int64_t kRowLaunchMcs = 128;
+constexpr int kRowGraphMcs = 32;
+constexpr int kRowGraphShort = 8;
 
 }  // namespace
 }  // namespace oct
@@ -317,6 +328,7 @@ struct oct_batch {
     // the active replicas ordered by branch: act_n[br] of them from act_first[br]
     uint32_t act_first[kBranches] = {};
     uint32_t act_n[kBranches] = {};
+    int64_t row_mcs = 0;          // MCS launched one by one in row lanes since the last rebuild
     uint32_t row_descs = 0;       // warps of a device step in row lanes; 0: the branches below carry the batch
     uint32_t *d_queue = nullptr;  // 4 * kBranches counters: (device step, branch)
     oct::W2RowSums *d_rows = nullptr;
@@ -340,9 +352,9 @@ struct oct_batch {
     uint64_t ticks = 0;  // MCS run by oct_batch_run
     int grid = 0;
     cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;        // one MCS
+    cudaGraphExec_t exec = nullptr;        // one MCS (kRowGraphShort in row lanes)
     cudaGraph_t graph_n = nullptr;
-    cudaGraphExec_t exec_n = nullptr;      // kGraphMcs MCS
+    cudaGraphExec_t exec_n = nullptr;      // kGraphMcs MCS (kRowGraphMcs)
     // side streams and events of the captured MCS: one branch per kind
     cudaStream_t side[kBranches] = {};
     cudaEvent_t fork_ev = nullptr;
@@ -578,6 +590,7 @@ cudaError_t rebuild(oct_batch *b) {
     for (int br = 0; br < kBranches; ++br) active.insert(active.end(), by_branch[br].begin(), by_branch[br].end());
     row_lists(rd, active, items, descs);
     b->row_descs = static_cast<uint32_t>(descs.size());
+    b->row_mcs = 0;
     active.clear();
     for (int br = 0; br < kBranches; ++br) {
         b->act_first[br] = static_cast<uint32_t>(active.size());
@@ -723,6 +736,16 @@ cudaError_t enqueue_advance_branch(oct_batch *b, int br, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+// nmcs MCS of a batch in row lanes: launch by launch, each overlapping the one
+// before; the counters advance at the end.
+cudaError_t enqueue_row_mcs(oct_batch *b, cudaStream_t st, uint32_t nmcs) {
+    cudaError_t e = cudaSuccess;
+    for (uint32_t i = 0; i < nmcs; ++i)
+        for (uint32_t k = 0; k < 4 && e == cudaSuccess; ++k) e = enqueue_row_step(b, i, k, i > 0 || k > 0, st);
+    if (e == cudaSuccess && nmcs > 0) e = enqueue_advance(b, nmcs, st);
+    return e;
+}
+
 // nmcs MCS for capture on st.  The replicas of different branches (kinds,
 // and parts of a kind) share no memory and no counter, so each branch's
 // device steps and its own MCS-counter advances form a branch of the graph
@@ -756,7 +779,7 @@ cudaError_t capture_mcs(oct_batch *b, int nmcs, cudaGraph_t *graph, cudaGraphExe
     if (e != cudaSuccess) return e;
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        const cudaError_t e2 = enqueue_mcs(b, cap, nmcs);
+        const cudaError_t e2 = b->row_descs ? enqueue_row_mcs(b, cap, static_cast<uint32_t>(nmcs)) : enqueue_mcs(b, cap, nmcs);
         e = cudaStreamEndCapture(cap, graph);
         if (e == cudaSuccess) e = e2;
     }
@@ -1119,15 +1142,29 @@ int oct_batch_run(oct_batch *b, int64_t n) {
             BATCH_CUDA(enqueue_advance(b, 1u, b->stream));
         }
     } else if (b->row_descs) {
-        // launch by launch, each overlapping the one before; the counters advance
-        // at the end (2^16 MCS at a time, far inside their range)
-        for (int64_t done = 0; done < n;) {
-            const uint32_t part = static_cast<uint32_t>(std::min<int64_t>(n - done, 1 << 16));
-            for (uint32_t i = 0; i < part; ++i)
-                for (uint32_t k = 0; k < 4; ++k)
-                    BATCH_CUDA(enqueue_row_step(b, i, k, i > 0 || k > 0, b->stream));
-            BATCH_CUDA(enqueue_advance(b, part, b->stream));
-            done += part;
+        // launch by launch at first, replays of graphs once the membership has
+        // lasted (see kRowLaunchMcs); they are captured behind the first launches,
+        // while the device works on them.  A caller's capture takes the launches.
+        cudaStreamCaptureStatus outer = cudaStreamCaptureStatusNone;
+        if (n >= oct::kRowGraphShort) BATCH_CUDA(cudaStreamIsCapturing(b->stream, &outer));
+        int64_t left = n;
+        while (left > 0) {
+            if (left >= oct::kRowGraphShort && b->row_mcs >= oct::kRowLaunchMcs && outer == cudaStreamCaptureStatusNone) {
+                const bool longer = left >= oct::kRowGraphMcs;
+                const int mcs = longer ? oct::kRowGraphMcs : oct::kRowGraphShort;
+                cudaGraphExec_t &exec = longer ? b->exec_n : b->exec;
+                if (!exec) {
+                    const cudaError_t e = capture_mcs(b, mcs, longer ? &b->graph_n : &b->graph, &exec);
+                    if (e != cudaSuccess) return bfail(OCT_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
+                }
+                BATCH_CUDA(cudaGraphLaunch(exec, b->stream));
+                left -= mcs;
+                continue;
+            }
+            const int64_t part = std::min<int64_t>(left, oct::kRowLaunchMcs);
+            BATCH_CUDA(enqueue_row_mcs(b, b->stream, static_cast<uint32_t>(part)));
+            b->row_mcs += part;
+            left -= part;
         }
     } else {
         // kGraphMcs MCS per graph launch while that many are left, then one
