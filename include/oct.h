@@ -253,8 +253,10 @@ int oct_get_timing(oct_sim *s, double *step_ms, int64_t *step_launches, double *
  * needed an acceptance draw (counted only when p or q lies strictly inside
  * (0,1)), tail_blocks = Philox blocks the plain device-step kernels generated
  * for the tail stream of tied acceptance uniforms (counted over the lanes that
- * store them; zero without acceptance draws, and where the rates are multiples
- * of 1/16, whose ties are all refused).  Synchronises. */
+ * store them; zero without acceptance draws, and where both rates lie strictly
+ * inside (0,1) and are multiples of 1/16, whose ties are all refused; with one
+ * such rate beside 0 or 1 the 4 x 4-cell DTrDT step still generates them).
+ * Synchronises. */
 typedef struct {
     int64_t t;
     int64_t net_flips;
