@@ -39,7 +39,8 @@ int cuda_fail(cudaError_t e, const char *what) {
 uint32_t threshold32(double p) { return static_cast<uint32_t>(std::floor(std::ldexp(p, 32))); }
 
 constexpr int kEventPairs = 256;
-constexpr int64_t kRunMcs = 1024;  // MCS of a small lattice in one launch (about 10 ms at most)
+// MCS of a small lattice in one launch (L=256: 15 ms KPZ, 31 ms with p=0.95, q=0.05)
+constexpr int64_t kRunMcs = 1024;
 
 }  // namespace
 

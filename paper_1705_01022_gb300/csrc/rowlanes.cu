@@ -24,7 +24,11 @@ constexpr uint32_t kRowSingleMax = 152u * 20u;   // warps of a step in one-warp 
 // One block up to a warp per scheduler: 8 MCS and a W^2 at L=256 KPZ 135 us,
 // 149 with launches.
 constexpr uint32_t kBlockWarps = 4;
-constexpr uint32_t kBlockLattice = 64u * 1024u;  // bytes of its lattice at most
+// Its lattice in bytes at most: a lane holds 128 sites, a step a quarter of the
+// sites, four sites a byte (L <= 256).  With the warps' own areas it stays below
+// the 48 KB that a launch may take without raising its limit.
+constexpr uint32_t kBlockLattice = kBlockWarps * 32u * 128u;
+static_assert(kBlockLattice + kBlockWarps * row_smem_words<true>() * 4u <= 48u * 1024u, "within the default limit");
 
 template <bool RANDOM, int SPEC, bool ONE, bool SHARED = false, class Ready, class Done>
 __device__ __forceinline__ void row_step(const StepArgs &a, uint32_t *lat, uint32_t warp, uint32_t t, uint32_t k, uint32_t *sm,
@@ -129,11 +133,6 @@ cudaError_t launch_row_step_as(const StepArgs &a, bool overlap, cudaStream_t st)
 template <bool RANDOM, int SPEC, bool ONE>
 cudaError_t launch_row_run_as(const StepArgs &a, uint32_t *t_out, uint32_t n, cudaStream_t st) {
     const uint32_t warps = row_warps(a), smem = a.L * a.wpr * 8u + warps * row_smem_words<RANDOM>() * 4u;
-    // the same limit for every launch: threads that run other sizes may pass here at the same time
-    constexpr uint32_t kMost = kBlockLattice + kBlockWarps * row_smem_words<RANDOM>() * 4u;
-    cudaError_t e = cudaFuncSetAttribute(row_block_kernel<RANDOM, SPEC, ONE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMost));
-    if (e != cudaSuccess) return e;
     row_block_kernel<RANDOM, SPEC, ONE><<<1, warps * 32u, smem, st>>>(a, t_out, n);
     return cudaGetLastError();
 }
@@ -145,7 +144,7 @@ bool rows_take(const StepArgs &a) {
            row_warps(a) <= kRowWarpsMax;
 }
 
-bool rows_fit_block(const StepArgs &a) { return row_warps(a) <= kBlockWarps && a.L * a.wpr * 8u <= kBlockLattice; }
+bool rows_fit_block(const StepArgs &a) { return row_warps(a) <= kBlockWarps; }
 
 #define OCT_ROWS(FN, ...)                                                                                \
     do {                                                                                                 \
