@@ -326,7 +326,6 @@ __device__ __forceinline__ void cells_apply(uint32_t (&X)[16], uint32_t (&Y)[16]
 // single-hit collective steps, write back.  One sub-tile per warp.
 template <int CX, int CY, bool RANDOM, int SPEC>
 __device__ __forceinline__ void run_subtile_cells(uint32_t *lat, uint32_t L, uint32_t plane_rows, uint32_t wpr,
-                                                  uint32_t Bx, uint32_t By,
                                                   uint32_t x0, uint32_t y0, bool active, const CellCtx &cc,
                                                   uint32_t *ring, uint32_t *draw_w, int &net, int &draws,
                                                   int &tails) {
@@ -450,7 +449,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, kStepBlocksPerSMPacke
     c.g = static_cast<uint32_t>(cc.gr * c.GX + c.gx);  // the lane's group
 
     int net = 0, draws = 0, tails = 0;
-    run_subtile_cells<CX, CY, RANDOM, SPEC>(a.lat, L, a.plane_rows, a.wpr, a.Bx, a.By, x0, y0, active, cc,
+    run_subtile_cells<CX, CY, RANDOM, SPEC>(a.lat, L, a.plane_rows, a.wpr, x0, y0, active, cc,
                                             ring + (RANDOM ? (threadIdx.x >> 5) * 32 * kRingWordsPerLane : 0u),
                                             draw_w + (threadIdx.x >> 5) * kDraws, net, draws, tails);
 

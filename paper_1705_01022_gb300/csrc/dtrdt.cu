@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kStepWarpsPerBlock * 32, step_min_blocks(SCHEM
 
     const uint32_t wpr = a.wpr;
     int net = 0, draws = 0, tails = 0;
-    run_subtile<RANDOM, PACKED, SCHEME>(a.lat, L, a.plane_rows, wpr, a.Bx, a.By, x0, y0, active, c,
+    run_subtile<RANDOM, PACKED, SCHEME>(a.lat, L, a.plane_rows, wpr, x0, y0, active, c,
                                         ring + ((threadIdx.x >> 5) * 32 + seg * S) * kRingWordsPerLane,
                                         net, draws, tails);
     // lanes that hold no group (a packed sub-tile of, say, six groups has eight

@@ -336,8 +336,8 @@ __device__ __forceinline__ uint32_t column_fields(uint32_t v, uint32_t e0) {
 // draw, so no always/never masks are applied.
 template <int DY, bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_candidates(const uint32_t (&X)[16], const uint32_t (&Y)[16],
-                                                uint32_t E, uint32_t D, const uint4 &site, uint32_t s,
-                                                uint32_t dx, const Ctx &c, uint32_t (&cnd0)[4],
+                                                uint32_t E, uint32_t D, const uint4 &site, uint32_t dx,
+                                                const Ctx &c, uint32_t (&cnd0)[4],
                                                 uint32_t (&cnd1)[4], uint32_t &pmin, uint32_t &pmax) {
     const uint32_t sw[4] = {site.x, site.y, site.z, site.w};
     const uint32_t sh2 = 2u * dx;
@@ -374,7 +374,7 @@ __device__ __forceinline__ void step_candidates(const uint32_t (&X)[16], const u
         } else if (RANDOM) {
             const uint32_t mn = (cnd0[m] & ~xa) | (cnd1[m] & ~xb);
             const uint32_t mx = (cnd0[m] & xa) | (cnd1[m] & xb);
-            const uint32_t cmn = SPEC == 2 ? mn : mn & c.p_random, cmx = SPEC == 2 ? mx : mx & c.q_random;
+            const uint32_t cmn = mn & c.p_random, cmx = mx & c.q_random;
             // a cell has at most one candidate, at bit 4j + sh2 + xoff: 3 cmn sets bit
             // 4j + sh2 + 1 for either xoff (no carries: candidates are >= 3 bits apart)
             pmin |= (((cmn * 3u) >> (sh2 + 1u)) & kNib) << m;
@@ -476,8 +476,8 @@ __device__ __forceinline__ void step_apply(uint32_t (&X)[16], uint32_t (&Y)[16],
 // runs unconditionally so that all 32 lanes take part.
 template <bool RANDOM, int SPEC = 0, class Ctx>
 __device__ __forceinline__ void step_candidates_rt(const uint32_t (&X)[16], const uint32_t (&Y)[16],
-                                                   uint32_t E, uint32_t D, const uint4 &site, uint32_t s,
-                                                   uint32_t dx, uint32_t dy, const Ctx &c,
+                                                   uint32_t E, uint32_t D, const uint4 &site, uint32_t dx,
+                                                   uint32_t dy, const Ctx &c,
                                                    uint32_t (&cnd0)[4], uint32_t (&cnd1)[4],
                                                    uint32_t &pmin, uint32_t &pmax) {
     const uint32_t sw[4] = {site.x, site.y, site.z, site.w};  // shifted to the step's field by run_subtile
@@ -1351,8 +1351,7 @@ __device__ __forceinline__ void write_back(const LaneGeom &q, uint32_t L, uint32
 // rates for which every tie is refused, 10 as 5 for rates of either kind.
 template <bool RANDOM, bool LANE_SETS, int SCHEME = 0, class Ctx>
 __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t plane_rows, uint32_t wpr,
-                                            uint32_t Bx, uint32_t By, uint32_t x0, uint32_t y0, bool active,
-                                            const Ctx &c, uint32_t *ring, int &net, int &draws,
+                                            uint32_t x0, uint32_t y0, bool active, const Ctx &c, uint32_t *ring, int &net, int &draws,
                                             int &tails) {
     TailPool tp;
     tp.ring = ring + static_cast<uint32_t>(kRingWordsPerLane) * c.g;  // the lane's own slot
@@ -1423,18 +1422,18 @@ __device__ __forceinline__ void run_subtile(uint32_t *lat, uint32_t L, uint32_t 
         constexpr int kSpec = SCHEME == 4 ? 1 : (SCHEME == 5 || SCHEME == 8 || SCHEME == 10) ? 2 : 0;
         constexpr int kTies = (SCHEME == 0 || SCHEME == 5) ? kTiesCount : SCHEME == 8 ? kTiesRefused : kTiesAsk;
         if (LANE_SETS)
-            step_candidates_rt<RANDOM, kSpec>(X, Y, E, D, site, s, d & 1u, d >> 1, c, cnd0, cnd1, pmin, pmax);
+            step_candidates_rt<RANDOM, kSpec>(X, Y, E, D, site, d & 1u, d >> 1, c, cnd0, cnd1, pmin, pmax);
         // the candidate phase with the set's column offset as a constant as well
         // (the flip phase stays specialised on the row offset alone: four copies
         // of it measured slower, from instruction-cache pressure)
         else if (d == 3u)
-            step_candidates<1, RANDOM, kSpec>(X, Y, E, D, site, s, 1u, c, cnd0, cnd1, pmin, pmax);
+            step_candidates<1, RANDOM, kSpec>(X, Y, E, D, site, 1u, c, cnd0, cnd1, pmin, pmax);
         else if (d == 2u)
-            step_candidates<1, RANDOM, kSpec>(X, Y, E, D, site, s, 0u, c, cnd0, cnd1, pmin, pmax);
+            step_candidates<1, RANDOM, kSpec>(X, Y, E, D, site, 0u, c, cnd0, cnd1, pmin, pmax);
         else if (d == 1u)
-            step_candidates<0, RANDOM, kSpec>(X, Y, E, D, site, s, 1u, c, cnd0, cnd1, pmin, pmax);
+            step_candidates<0, RANDOM, kSpec>(X, Y, E, D, site, 1u, c, cnd0, cnd1, pmin, pmax);
         else
-            step_candidates<0, RANDOM, kSpec>(X, Y, E, D, site, s, 0u, c, cnd0, cnd1, pmin, pmax);
+            step_candidates<0, RANDOM, kSpec>(X, Y, E, D, site, 0u, c, cnd0, cnd1, pmin, pmax);
         uint32_t acc = 0u;
         if (RANDOM) {
             draws += __popc(pmin | pmax);

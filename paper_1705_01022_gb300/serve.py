@@ -237,7 +237,7 @@ class ServingEngine:
             job.t += n
             self.mcs_attempts += n * job.L * job.L
             last = job.t >= job.t_max
-            if job.t in job.measure_at and not self.async_measure:
+            if not self.async_measure and job.t in job.measure_at:
                 self._deliver_one(job, batch.measure(slot), now)
             if last:
                 batch.remove(slot)
