@@ -184,8 +184,8 @@ __device__ __forceinline__ void batch_row_item(const ReplicaDev &R, const WarpDe
 
 // Larger batches take the graph's branches, whose lanes of four TC rows need
 // fewer instructions per attempt (16 MCS and the W^2 of n replicas of L=2048, 256
-// warps each, ms in row lanes and with the graph: n=16 1.38, 1.98; 24 2.00, 2.29;
-// 32 2.52, 2.69; 40 3.07, 2.93).
+// warps each, ms in row lanes and with the graph: n=16 1.36, 1.96; 24 1.98, 2.29;
+// 32 2.49, 2.64; 40 3.02, 2.87; 64 4.66, 3.25).
 constexpr uint32_t kBatchRowWarpsMax = 152u * 54u;
 
 // One warp per block, so that the blocks spread evenly over the schedulers (16

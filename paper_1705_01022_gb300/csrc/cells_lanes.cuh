@@ -2,15 +2,16 @@
 // sites, cx in {8, 16, 32}, cy in {4, 8, 16}.
 //
 // A collective step makes one attempt per cell, so a lane that holds 32 x 16
-// sites bit-parallel (cells.cuh) tests all eight rows that an attempt can fall
+// sites bit-parallel (cells.cuh) reads all eight rows that an attempt can fall
 // on for the sake of its 512 / (cx cy) attempts: two for 16 x 16 cells.  Here
 // the sub-tile lies in shared memory and a lane makes one attempt at a time,
-// three loads and up to three stores of it, whatever the cell.  Bound by
-// instruction issue and fixed latency (16 x 16 cells in 64 x 64 sub-tiles, p=0.95,
-// q=0.05: one MCS at L=8192 from 2.31 to 0.56 ms at 171 instructions per 32
-// attempts, then to 0.48 ms with the draws' places constant in loops over the
-// steps of a level block).  A warp takes the cells of a sub-tile in turns of 32 (NC of them), or
-// several sub-tiles of fewer than 32 cells at once.
+// three loads and up to three stores of it, whatever the cell.  Bound by fixed
+// latency and shared-memory round trips, issue slots 53 % (16 x 16 cells in 64 x
+// 64 sub-tiles, p=0.95, q=0.05: one MCS at L=8192 from 2.31 to 0.56 ms at 171
+// instructions per 32 attempts, then to 0.48 ms with the draws' places constant
+// in loops over the steps of a level block).  A warp takes the cells of a
+// sub-tile in turns of 32 (NC of them), or several sub-tiles of fewer than 32
+// cells at once.
 //
 // Cells and random streams are those of cells.cuh (same sites, uniforms and tie
 // order).  A group of four TC rows x 32 columns has 128/cx cells, which are
@@ -404,11 +405,11 @@ cudaError_t launch_lane_cells(const StepArgs &a, const LaneSplit &q, cudaStream_
 // and the sub-tile; the bit-parallel one costs a step of a lane for 512 / (cx cy)
 // attempts, with GX * GY of 32 lanes at work.  One MCS at L=8192, p=0.95, q=0.05
 // (us, bit-parallel and lane per cell):
-//   256x64 sub-tiles (32 groups): 8x8 281, 585; 16x8 487, 629; 32x8 773, 634;
-//                                 16x16 906, 575; 32x16 1503, 744
-//   64x64 (8 groups):             8x4 504, 525; 16x4 716, 443; 8x8 847, 429;
-//                                 16x8 1263, 421; 16x16 2332, 476; 32x16 3850, 660
-//   32x32 (2 groups):             8x4 1684, 700; 8x8 2832, 591; 16x16 7900, 863
+//   256x64 sub-tiles (32 groups): 8x8 267, 592; 16x8 443, 590; 8x16 499, 606;
+//                                 32x8 807, 613; 16x16 801, 586; 32x16 1441, 633
+//   64x64 (8 groups):             8x4 414, 524; 16x4 674, 547; 8x8 660, 436;
+//                                 16x8 1123, 429; 16x16 2036, 481; 32x16 3756, 668
+//   32x32 (2 groups):             8x4 1319, 679; 8x8 2136, 546; 16x16 6835, 703
 // so the line lies at cx cy 32 / groups = 256.  Cells four columns wide (half
 // rows of two sites) and sub-tiles whose last group row is so incomplete that
 // they need more turns than the registers hold stay bit-parallel.

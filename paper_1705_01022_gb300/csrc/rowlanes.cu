@@ -16,9 +16,10 @@ namespace oct {
 namespace {
 
 // Warps per block of a device-step launch: one while they still find free
-// places, so that the blocks spread evenly over the schedulers, else four (8
-// MCS and a W^2, us with one and with four: L=1536 257, 274; L=4096 316, 352; 4 MCS
-// at L=6144 (2304 warps) 239, 253; L=8192 (4096 warps) 391, 343).
+// places, so that the blocks spread evenly over the schedulers, else four.  8 MCS
+// and a W^2, us with one and with four, p=0.95, q=0.05: L=1536 280, 284; L=4096
+// 347, 378; L=6144 (2304 warps) 511, 540; L=7168 (3136) 667, 680; L=8192 (4096)
+// 828, 730; KPZ: 147, 166; 215, 246; 338, 354; 437, 474; 451, 468.
 constexpr uint32_t kRowWarps = 4;
 constexpr uint32_t kRowSingleMax = 152u * 20u;   // warps of a step in one-warp blocks
 // One block up to a warp per scheduler: 8 MCS and a W^2 at L=256 KPZ 135 us,

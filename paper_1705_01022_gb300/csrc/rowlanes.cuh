@@ -12,9 +12,9 @@
 // is warp-uniform.  The four lanes of a group share its Philox blocks instead
 // of repeating them: lane m generates every fourth block of the device step and
 // leaves it (of the acceptance draws, their comparison with P32) in shared
-// memory, before the step's first access to the lattice.  8 MCS and a W^2: L=256
-// KPZ 405 -> 136 us, L=3136 p=0.95 (32 x 16 sub-tiles) 640 -> 285 us, L=4096
-// p=q=0.5 667 -> 350 us, then 256 us without its ties (ties_matter).
+// memory, before the step's first access to the lattice.  8 MCS and a W^2, us on
+// packed groups and here: L=256 KPZ 266, 132; L=3136 p=0.95 (32 x 16 sub-tiles)
+// 492, 290; L=4096 p=0.95 554, 346, p=q=0.5 387, 257.
 //
 // Lanes of a sub-tile: gx + GX * tr, TC row tr = 0 .. By/4 - 1 (group row tr/4,
 // m = tr % 4), a power-of-two number of band columns GX, at most 32 lanes.
@@ -50,8 +50,11 @@ __host__ __device__ inline uint32_t row_segment(uint32_t GX, uint32_t By) {
 
 // Device steps of more warps than this keep the chip busy either way, and then
 // the lane of four TC rows needs fewer instructions per attempt (64 x 64
-// sub-tiles, us per MCS here and there: p=q=0.5, L=4096 47, 81; p=0.95, q=0.05,
-// L=8192 86, 107; L=16384 292, 262).
+// sub-tiles, us per MCS here and there):
+//   L                   4096        6144        7168        8192        8704         9216         16384
+//   KPZ                 23.8, 34.7  38.1, 37.0  55.2, 51.8  54.2, 57.7  61.4, 62.7   69.8, 67.4   178, 131
+//   p=q=0.5             28.9, 44.8  47.2, 47.0  64.8, 67.4  68.7, 73.9  75.4, 77.9   82.1, 90.7   224, 184
+//   p=0.95, q=0.05      40.1, 65.7  59.8, 68.4  80.9, 89.2  86.6, 98.4  103, 109     113, 111     293, 227
 constexpr uint32_t kRowWarpsMax = 152u * 32u;
 
 // ONE: one sub-tile per warp (the set is warp-uniform); otherwise the rows of
