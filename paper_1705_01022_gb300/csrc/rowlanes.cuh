@@ -70,7 +70,9 @@ __device__ __forceinline__ void run_rows(uint32_t *lat, uint32_t L, uint32_t pla
     uint4 *const lvl_w = site_w + 8u * kRowGroups;
     uint32_t *const ring = sm + kRowGroups * 96u + rl.gw * kRowRing;
     const uint32_t m = rl.m, gw = rl.gw;
-    // the draws of the whole device step
+    // the draws of the whole device step, over those of the step before (in the one
+    // launch of a whole run), which every lane has read
+    if (SHARED) __syncwarp();
     const uint4 setw = c.draw(c.k, kTagSet << 28);
 #pragma unroll
     for (uint32_t i = 0; i < 2u; ++i) {
